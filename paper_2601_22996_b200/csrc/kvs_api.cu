@@ -295,8 +295,18 @@ cudaError_t close_sides(kvs_ctx* ctx) {
 // [i0, i1) and are evaluations e0 .. e0 + P - 1 of a batch of P_total; `ev` already points at e0.  What chunk
 // number `chunk` uploads goes to the copy stream before the chunk's inputs (behind them it would wait in the copy
 // engine for the inputs of the chunks that follow); `feed` then sends the inputs and makes the kernels' stream wait.
-// `lane`: the pair of streams that the chunk's kernels run on, or -1 for the context's stream.
-struct FusedRange { int64_t i0, i1, e0, P_total; int chunk, lane; std::function<int()> feed; };
+// `lane`: the pair of streams that the chunk's kernels run on, or -1 for the context's stream; `light_ctas`: see lane_light_ctas.
+struct FusedRange { int64_t i0, i1, e0, P_total; int chunk, lane; int64_t light_ctas; std::function<int()> feed; };
+
+// CTA scratch of a lane, and the part of it at its start that the light variant's kernels take where the full variant's run
+// beside them.  That part is the same for all chunks of a call: a lane's stream does not wait for its side stream between two
+// chunks, so the light kernels of one run while the full kernels of the one before it may still use theirs.
+constexpr int64_t LANE_CTAS = KVS_MAX_GRID / KVS_LANES;
+int64_t lane_light_ctas(const kvs_setting* st, int64_t P) {
+  for (int64_t e = 0; e < P; ++e)
+    if (st[e].family != KVS_GSA) return LANE_CTAS / 2;
+  return 0;                                  // no evaluation of the light variant (no profile is stored here)
+}
 
 int run_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settings, int64_t P,
               const kvs_schedule_out* out, const kvs_eval_out* ev, int do_profile, const FusedRange* rg = nullptr) {
@@ -490,8 +500,8 @@ int run_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settin
   // beside start behind the light variant's.
   int64_t light_max = 0;
   for (int f = 0; f < 4; ++f) light_max = std::max(light_max, light_of[f]);
-  const int64_t lane_ctas = lane >= 0 ? KVS_MAX_GRID / KVS_LANES : KVS_MAX_GRID, lane_at = lane >= 0 ? lane * lane_ctas : 0;
-  const int64_t light_ctas = beside ? std::min(light_max, lane_ctas / 2) : lane_ctas, side_at = lane_at + light_ctas;
+  const int64_t lane_ctas = lane >= 0 ? LANE_CTAS : KVS_MAX_GRID, lane_at = lane >= 0 ? lane * lane_ctas : 0;
+  const int64_t light_ctas = !beside ? lane_ctas : (lane >= 0 ? rg->light_ctas : std::min(light_max, lane_ctas / 2)), side_at = lane_at + light_ctas;
   const int64_t side_ctas = beside ? lane_ctas - light_ctas : lane_ctas;
   auto scratch_at = [&](int64_t cta) {
     bp.lists = reinterpret_cast<int32_t*>(ws + L.lists + static_cast<size_t>(cta) * static_cast<size_t>(KVS_CTA_SCRATCH(max_n)));
@@ -831,6 +841,7 @@ int kvs_evaluate_built_host(kvs_ctx* ctx, const kvs_instances* inst, const kvs_s
   if (n_chunks < 1) n_chunks = 1;
   for (int l = 0; l < KVS_LANES && n_chunks > 1; ++l)
     if ((ce = open_side(ctx->side[2 * l + 1], ctx->stream, false)) != cudaSuccess) return fail_cuda(ctx, ce, "stream ordering");
+  const int64_t light_ctas = lane_light_ctas(settings, P);
   int64_t r0 = 0;
   for (int64_t c = 0; c < n_chunks; ++c) {
     const int64_t i0 = c * I / n_chunks, i1 = (c + 1) * I / n_chunks;
@@ -856,7 +867,7 @@ int kvs_evaluate_built_host(kvs_ctx* ctx, const kvs_instances* inst, const kvs_s
     if (r1 > r0) {
       kvs_eval_out dc = d;
       dc.peak += r0; dc.flow += r0; dc.job_steps += r0; dc.horizon += r0; dc.n_unfinished += r0; dc.feasible += r0; dc.status += r0;
-      const FusedRange rg{i0, i1, r0, P, static_cast<int>(c), lane, feed};
+      const FusedRange rg{i0, i1, r0, P, static_cast<int>(c), lane, light_ctas, feed};
       rc = run_fused(ctx, &dev, sorted.data() + r0, r1 - r0, nullptr, &dc, 1, &rg);
       if (rc) return rc;
     } else if ((rc = feed()) != KVS_OK) {

@@ -1,0 +1,319 @@
+// A CUDA runtime that runs nothing, for CPU tests of the host code of the library (csrc/kvs_api.cu): it carries out copies
+// at once, gives every copy and kernel launch the memory that it reads and writes, and follows streams and events with
+// vector clocks.  Two accesses to one place, one of them a write, race unless one of them is ordered before the other.
+// Any call can be made to fail (`fail_at`).  The programs at the end drive the C entry points; the test builds this file with
+// kvs_api.cu and runs them.
+#include <algorithm>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <random>
+#include <string>
+#include <vector>
+
+#include "kvs_internal.cuh"
+
+namespace {
+
+constexpr int MAX_STREAMS = 32;
+struct Clock {
+  long at[MAX_STREAMS] = {};
+  void join(const Clock& c) { for (int i = 0; i < MAX_STREAMS; ++i) at[i] = std::max(at[i], c.at[i]); }
+};
+struct Stream { int id; Clock clock; };
+struct Event { Clock clock; };
+
+enum Kind { READ, WRITE, ATOMIC };
+struct Access { const unsigned char* a; const unsigned char* b; Kind kind; };
+struct Op { std::string name; int stream; long seq; Clock clock; std::vector<Access> acc; };
+
+std::vector<Stream*> streams;
+std::vector<Op> ops;
+Clock host;
+int calls = 0, fail_at = -1, races = 0;
+
+Stream* stream_of(cudaStream_t s) {
+  if (streams.empty()) streams.push_back(new Stream{0, {}});       // the default stream
+  return s ? reinterpret_cast<Stream*>(s) : streams[0];
+}
+bool fails() { return calls++ == fail_at; }
+Access span(const void* p, size_t bytes, Kind kind) {
+  const unsigned char* a = static_cast<const unsigned char*>(p);
+  return Access{a, a ? a + bytes : a, kind};
+}
+void submit(const char* name, cudaStream_t s, std::vector<Access> acc) {
+  Stream* st = stream_of(s);
+  st->clock.join(host);
+  const long seq = ++st->clock.at[st->id];
+  // places that touch or overlap become one
+  std::sort(acc.begin(), acc.end(), [](const Access& x, const Access& y) { return x.kind != y.kind ? x.kind < y.kind : x.a < y.a; });
+  size_t n = 0;
+  for (const Access& x : acc) {
+    if (x.a == x.b) continue;
+    if (n && acc[n - 1].kind == x.kind && x.a <= acc[n - 1].b) acc[n - 1].b = std::max(acc[n - 1].b, x.b);
+    else acc[n++] = x;
+  }
+  acc.resize(n);
+  ops.push_back(Op{name, st->id, seq, st->clock, std::move(acc)});
+}
+
+bool before(const Op& x, const Clock& c) { return c.at[x.stream] >= x.seq; }
+void find_races() {
+  for (size_t j = 0; j < ops.size(); ++j)
+    for (size_t i = 0; i < j; ++i) {
+      if (before(ops[i], ops[j].clock)) continue;
+      for (const Access& x : ops[i].acc)
+        for (const Access& y : ops[j].acc) {
+          if (x.kind == y.kind && x.kind != WRITE) continue;
+          if (x.a < y.b && y.a < x.b) {
+            if (races++ < 5) printf("race: %s on stream %d and %s on stream %d share %zu bytes\n", ops[i].name.c_str(), ops[i].stream,
+                                    ops[j].name.c_str(), ops[j].stream, static_cast<size_t>(std::min(x.b, y.b) - std::max(x.a, y.a)));
+          }
+        }
+    }
+}
+int outstanding(const Clock& c) {
+  int n = 0;
+  for (const Op& o : ops) n += before(o, c) ? 0 : 1;
+  return n;
+}
+
+}  // namespace
+
+// ---- the runtime ------------------------------------------------------------------------------------------------
+
+extern "C" {
+cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
+cudaError_t cudaSetDevice(int) { return fails() ? cudaErrorUnknown : cudaSuccess; }
+cudaError_t cudaGetDeviceProperties_v2(cudaDeviceProp* p, int) { memset(p, 0, sizeof *p); p->multiProcessorCount = 148; return cudaSuccess; }
+const char* cudaGetErrorString(cudaError_t) { return "made to fail"; }
+cudaError_t cudaDeviceGetStreamPriorityRange(int* least, int* greatest) { *least = 0; *greatest = -5; return fails() ? cudaErrorUnknown : cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
+  if (fails()) return cudaErrorUnknown;
+  stream_of(nullptr);
+  if (streams.size() >= MAX_STREAMS) { printf("more than %d streams\n", MAX_STREAMS); exit(2); }
+  streams.push_back(new Stream{static_cast<int>(streams.size()), {}});
+  *s = reinterpret_cast<cudaStream_t>(streams.back());
+  return cudaSuccess;
+}
+cudaError_t cudaStreamCreateWithPriority(cudaStream_t* s, unsigned f, int) { return cudaStreamCreateWithFlags(s, f); }
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t s) { host.join(stream_of(s)->clock); return fails() ? cudaErrorUnknown : cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { for (Stream* s : streams) host.join(s->clock); return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
+  if (fails()) return cudaErrorUnknown;
+  stream_of(s)->clock.join(reinterpret_cast<Event*>(e)->clock);
+  return cudaSuccess;
+}
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) {
+  if (fails()) return cudaErrorUnknown;
+  *e = reinterpret_cast<cudaEvent_t>(new Event{});
+  return cudaSuccess;
+}
+cudaError_t cudaEventCreate(cudaEvent_t* e) { return cudaEventCreateWithFlags(e, 0); }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 0.f; return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
+  if (fails()) return cudaErrorUnknown;
+  Stream* st = stream_of(s);
+  st->clock.join(host);
+  reinterpret_cast<Event*>(e)->clock = st->clock;
+  return cudaSuccess;
+}
+cudaError_t cudaEventSynchronize(cudaEvent_t e) { host.join(reinterpret_cast<Event*>(e)->clock); return fails() ? cudaErrorUnknown : cudaSuccess; }
+cudaError_t cudaMallocHost(void** p, size_t n) { if (fails()) return cudaErrorUnknown; *p = calloc(1, n); return cudaSuccess; }
+cudaError_t cudaFreeHost(void* p) { free(p); return cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t n, cudaMemcpyKind, cudaStream_t s) {
+  if (fails()) return cudaErrorUnknown;
+  memcpy(dst, src, n);
+  submit("copy", s, {span(dst, n, WRITE), span(src, n, READ)});
+  return cudaSuccess;
+}
+cudaError_t cudaMemcpy(void* dst, const void* src, size_t n, cudaMemcpyKind k) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, n, k, nullptr);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(nullptr);
+}
+cudaError_t cudaMemsetAsync(void* dst, int v, size_t n, cudaStream_t s) {
+  if (fails()) return cudaErrorUnknown;
+  memset(dst, v, n);
+  submit("memset", s, {span(dst, n, WRITE)});
+  return cudaSuccess;
+}
+}  // extern "C"
+
+// ---- the kernels: what they read and write ------------------------------------------------------------------------
+
+cudaError_t kvs_setup_sort() { return cudaSuccess; }
+cudaError_t kvs_setup_generic() { return cudaSuccess; }
+cudaError_t kvs_setup_bounds() { return cudaSuccess; }
+cudaError_t kvs_setup_spec() { return cudaSuccess; }
+int kvs_build_ctas_per_sm() { return 2; }
+int kvs_fused_ctas_per_sm(int light) { return light ? 3 : 2; }
+int kvs_spec_per_cta(i64) { return 0; }
+i64 kvs_spec_warp_bytes(i64 n) { return 64 * (n + 64); }
+i64 kvs_order_chunks(i64 n) { return n / 4096 + 1; }
+i64 kvs_sweep_blocks(i64 n) { return n / 64 + 1; }
+cudaError_t kvs_fused_check_word(unsigned long long*, int*, int) { return cudaSuccess; }
+cudaError_t kvs_refill_check_word(unsigned long long*, int*, int) { return cudaSuccess; }
+cudaError_t kvs_spec_check_word(unsigned long long*, int*, int) { return cudaSuccess; }
+
+cudaError_t kvs_launch_sort(const SortParams& p, int, cudaStream_t s) {
+  if (fails()) return cudaErrorUnknown;
+  const i64 lo = p.job_off[0], n = p.job_off[p.n_instances] - lo;
+  std::vector<Access> a = {span(p.job_off, 8 * (p.n_instances + 1), READ), span(p.s + lo, 4 * n, READ), span(p.o + lo, 4 * n, READ),
+                           span(p.stats, sizeof(InstStats) * p.n_instances, WRITE)};
+  for (int32_t* w : {p.perm, p.perm_tmp, p.iperm, p.sorted_s, p.sorted_o}) a.push_back(span(w + lo, 4 * n, WRITE));
+  submit("ordering", s, a);
+  return cudaSuccess;
+}
+
+namespace {
+void evaluations(const BuildParams& p, int grid, i64 e, std::vector<Access>* a) {
+  const kvs_setting& st = p.settings[e];
+  const i64 lo = p.job_off[st.instance], n = p.job_off[st.instance + 1] - lo;
+  for (const int32_t* r : {p.sorted_s, p.sorted_o, p.iperm, p.s, p.o}) a->push_back(span(r + lo, 4 * n, READ));
+  a->push_back(span(p.stats + st.instance, sizeof(InstStats), READ));
+  for (i64* w : {p.ev.peak, p.ev.flow, p.ev.job_steps, p.ev.horizon, p.ev.n_unfinished})
+    if (w) a->push_back(span(w + e, 8, WRITE));
+  if (p.ev.status) a->push_back(span(p.ev.status + e, 4, WRITE));
+}
+void scratch(const BuildParams& p, int grid, std::vector<Access>* a) {
+  a->push_back(span(p.lists, static_cast<size_t>(grid) * KVS_CTA_SCRATCH(p.max_jobs), WRITE));
+  a->push_back(span(p.fin_rank, static_cast<size_t>(grid) * p.max_jobs * 4, WRITE));
+  a->push_back(span(p.counter, 8, WRITE));
+  a->push_back(span(p.settings, sizeof(kvs_setting) * p.P, READ));
+}
+}  // namespace
+
+cudaError_t kvs_launch_fused(const BuildParams& p, int grid, int light, int fam, cudaStream_t s) {
+  if (fails()) return cudaErrorUnknown;
+  std::vector<Access> a;
+  scratch(p, grid, &a);
+  for (ull i = 0; i < *p.eval_count; ++i) evaluations(p, grid, p.eval_list[i], &a);
+  a.push_back(span(p.slow_list, 8 * p.P, ATOMIC));
+  a.push_back(span(p.slow_count, 8, ATOMIC));
+  submit(light ? "light kernel" : "full kernel", s, a);
+  return cudaSuccess;
+}
+cudaError_t kvs_launch_build(const BuildParams& p, int grid, cudaStream_t s) {
+  if (fails()) return cudaErrorUnknown;
+  std::vector<Access> a;
+  scratch(p, grid, &a);
+  for (i64 e = 0; e < p.P; ++e) evaluations(p, grid, e, &a);
+  if (p.slow_list) { a.push_back(span(p.slow_list, 8 * p.P, READ)); a.push_back(span(p.slow_count, 8, READ)); }
+  submit("general kernel", s, a);
+  return cudaSuccess;
+}
+static cudaError_t unused() { printf("a launch that these tests do not drive\n"); exit(2); }
+cudaError_t kvs_launch_refill(const RefillParams&, cudaStream_t) { return unused(); }
+cudaError_t kvs_launch_spec(SpecParams, cudaStream_t) { return unused(); }
+cudaError_t kvs_launch_generic_tiled(GenericParams, i64, int, cudaStream_t) { return unused(); }
+cudaError_t kvs_launch_bounds(const i64*, const int32_t*, const int32_t*, i64, InstStats*, const kvs_setting*, i64, const i64*, i64, const kvs_bounds_out&, u32*, cudaStream_t) { return unused(); }
+cudaError_t kvs_launch_order_info(const i64*, const int32_t*, const int32_t*, i64, i64, OrderInfo*, int, cudaStream_t) { return unused(); }
+cudaError_t kvs_launch_order(const int32_t*, const int32_t*, i64, int, u64*, u64*, u32*, int32_t*, int32_t*, cudaStream_t) { return unused(); }
+cudaError_t kvs_launch_prefix(const int32_t*, const int32_t*, i64, i64*, i64*, u32*, i64*, cudaStream_t) { return unused(); }
+cudaError_t kvs_launch_sweep(const SweepParams&, i64*, cudaStream_t) { return unused(); }
+cudaError_t kvs_launch_completed(const i64*, const i64*, const int32_t*, i64*, i64, cudaStream_t) { return unused(); }
+
+// ---- the calls ----------------------------------------------------------------------------------------------------
+
+namespace {
+
+constexpr int JOBS = 4;               // jobs per instance
+struct Batch {
+  int I;
+  std::vector<i64> off;
+  std::vector<int32_t> s, o;
+  std::vector<kvs_setting> st;
+  explicit Batch(int n_inst) : I(n_inst) {
+    for (int i = 0; i <= I; ++i) off.push_back(static_cast<i64>(i) * JOBS);
+    s.assign(static_cast<size_t>(I) * JOBS, 3);
+    o.assign(static_cast<size_t>(I) * JOBS, 5);
+  }
+  void add(int inst, int family) {
+    kvs_setting x{};
+    x.instance = inst; x.family = family; x.alpha_num = 2; x.alpha_den = 1; x.s_bar = -1; x.M = 1000;
+    st.push_back(x);
+  }
+};
+
+struct Caller {
+  kvs_ctx* ctx = nullptr;
+  std::vector<unsigned char> memory;
+  unsigned char* ws = nullptr;
+  explicit Caller(int I, i64 P) {
+    ops.clear();
+    streams.clear();
+    host = Clock{};
+    uint64_t need = 0;
+    kvs_workspace_bytes(static_cast<i64>(I) * JOBS, I, JOBS, P, 0, 1, &need);
+    memory.resize(need + 512);
+    ws = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(memory.data()) + 255) & ~static_cast<uintptr_t>(255));
+    kvs_init_params prm{};
+    prm.workspace = ws; prm.workspace_bytes = need;
+    if (kvs_init(&prm, &ctx) != KVS_OK) { printf("kvs_init failed\n"); exit(2); }
+  }
+  ~Caller() { kvs_destroy(ctx); }
+};
+
+kvs_instances view(const Batch& b) {
+  kvs_instances in{};
+  in.n_instances = b.I; in.n_jobs_total = static_cast<i64>(b.I) * JOBS; in.max_jobs_per_instance = JOBS;
+  in.job_off = b.off.data(); in.s = b.s.data(); in.o = b.o.data();
+  return in;
+}
+
+int host_call(Caller& c, const Batch& b) {
+  const size_t P = b.st.size();
+  std::vector<i64> peak(P), flow(P);
+  std::vector<int32_t> status(P);
+  kvs_eval_out ev{};
+  ev.peak = peak.data(); ev.flow = flow.data(); ev.status = status.data();
+  const kvs_instances in = view(b);
+  return kvs_evaluate_built_host(c.ctx, &in, b.st.data(), static_cast<i64>(P), &ev);
+}
+
+void run_host(const char* name, const Batch& b) {
+  Caller c(b.I, static_cast<i64>(b.st.size()));
+  const int r0 = races;
+  for (int twice = 0; twice < 2; ++twice)
+    if (const int rc = host_call(c, b)) { printf("%s: status %d\n", name, rc); ++races; }
+  find_races();
+  if (const int n = outstanding(host)) { printf("%s: %d operations in flight after the call\n", name, n); ++races; }
+  if (races != r0) printf("%s: %d\n", name, races - r0);
+}
+
+// chunks of unequal size, chunks of unequal composition, calls that do and do not split by family
+void overlaps() {
+  for (int I : {1024, 1000, 900, 769}) {
+    Batch b(I);
+    for (int i = 0; i < I; ++i) for (int f = KVS_GBA; f <= KVS_SIMS; ++f) b.add(i, f);
+    run_host(("four families on " + std::to_string(I)).c_str(), b);
+  }
+  std::mt19937 rng(7);
+  for (int rep = 0; rep < 8; ++rep) {
+    const int I = 600 + static_cast<int>(rng() % 700);
+    Batch b(I);
+    for (int i = 0; i < I; ++i) {
+      // later instances: more evaluations of the light variant, single families, or many of the full one
+      const int more = rep % 3 == 0 ? 1 + 6 * i / I : 2;
+      b.add(i, KVS_GSA);
+      for (int k = 0; k < more; ++k) b.add(i, rep % 4 == 0 ? KVS_SPS : static_cast<int>(rng() % 4));
+      if (rep % 3 == 2 && i > I / 2) for (int k = 0; k < 5; ++k) b.add(i, KVS_GSA);
+    }
+    if (rep % 2) std::shuffle(b.st.begin(), b.st.end(), rng);
+    run_host(("mixture " + std::to_string(rep)).c_str(), b);
+  }
+}
+
+}  // namespace
+
+int main(int argc, char** argv) {
+  const std::string what = argc > 1 ? argv[1] : "";
+  if (what == "overlaps") overlaps();
+  else { printf("unknown program\n"); return 2; }
+  printf("%s: %d faults\n", what.c_str(), races);
+  return races ? 1 : 0;
+}

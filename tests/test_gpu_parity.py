@@ -286,6 +286,31 @@ def test_host_entry_point_chunks(par, est):
                 assert torch.equal(v, getattr(want, k).cpu()), k
 
 
+@pytest.mark.parametrize("I,growing", [(1000, False), (900, False), (700, True)])
+def test_host_entry_point_uneven_chunks(par, I, growing):
+    """A chunk that has more evaluations of the light variant than the one before it on its lane, by its size or by its families:
+    against the device entry point."""
+    from paper_2601_22996_b200.api import Scheduler
+    inst = workloads.random_small(602, n_inst=I, n_max=300, s_max=60, o_max=400)
+    M = _tight_M(inst, 700)
+    rows = []
+    for i in range(I):
+        fams = ("GSA",) + ("GBA", "SPS") * (1 + 3 * i // I) if growing else ("GBA", "GSA", "SPS", "SIMS")
+        rows += [dict(instance=i, family=f, M=M[i] + 50 * k) for k, f in enumerate(fams)]
+    st = binding.make_settings(rows)
+    P, n = st.shape[0], int((inst.job_off[1:] - inst.job_off[:-1]).max())
+    assert P >= 2048
+    sched = par.scheduler()
+    want = sched.evaluate(inst.to("cuda:0"), st, want_jobs=False)
+    ctx = sched.context(binding.workspace_bytes(int(inst.s.numel()), I, n, P, host_staging=True))
+    hin = workloads.Instances(inst.job_off, inst.s.pin_memory(), inst.o.pin_memory())
+    for _ in range(3):
+        hev = {k: torch.full_like(v, -5, device="cpu").pin_memory() for k, v in Scheduler.scalars(P, "cpu").items()}
+        ctx.evaluate_built_host(hin, st, hev, window=0, max_jobs=n)
+        for k, v in hev.items():
+            assert torch.equal(v, getattr(want, k).cpu()), k
+
+
 @pytest.mark.parametrize("copies,runs", [(1, False), (80, False), (1, True)])      # shared evaluations, one CTA each, general kernel
 def test_outputs_of_evaluations_that_form_none(par, copies, runs):
     """Per-job results of an infeasible evaluation and rounds behind the end of a schedule take the values that the caller sets;
