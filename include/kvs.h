@@ -224,7 +224,8 @@ int kvs_evaluate_built(kvs_ctx* ctx, const kvs_instances* inst, const kvs_settin
  * to 16 chunks (of about a thousand evaluations or more, so small batches stay in one piece): the jobs of the next chunk are copied on a second stream while the kernels of the
  * current one run, so the settings may come in any order but are evaluated grouped by instance
  * (results are returned in the caller's order).  job_off is read on the host and must be
- * nondecreasing.  The call returns after the stream has been synchronised. */
+ * nondecreasing.  The call returns after the stream has been synchronised; if it fails, after everything that it
+ * had enqueued is over.  KVS_GBAD and KVS_GSAS settings are refused. */
 int kvs_evaluate_built_host(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settings,
                             int64_t P, const kvs_eval_out* ev);
 

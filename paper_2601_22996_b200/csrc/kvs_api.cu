@@ -79,12 +79,18 @@ cudaError_t take_stage(kvs_ctx* ctx, size_t bytes, kvs_ctx::Stage** out) {
   *out = &s;
   return cudaSuccess;
 }
+// The slot is in use until the stream has got here.
+cudaError_t mark_stage(kvs_ctx::Stage* s, cudaStream_t stream) {
+  const cudaError_t e = cudaEventRecord(s->done, stream);
+  s->used = e == cudaSuccess;
+  if (e != cudaSuccess) cudaStreamSynchronize(stream);   // no event to wait for later
+  return e;
+}
 // Uploads the first `bytes` bytes of the slot and marks it as in use until that has happened.
 cudaError_t send_stage(kvs_ctx::Stage* s, void* dst, size_t bytes, cudaStream_t stream) {
-  cudaError_t e = cudaMemcpyAsync(dst, s->p, bytes, cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess) e = cudaEventRecord(s->done, stream);
-  s->used = true;
-  return e;
+  const cudaError_t e = cudaMemcpyAsync(dst, s->p, bytes, cudaMemcpyHostToDevice, stream);
+  const cudaError_t marked = mark_stage(s, stream);
+  return e != cudaSuccess ? e : marked;
 }
 
 size_t align_up(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
@@ -264,23 +270,23 @@ int check_settings(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* s
 // Opened behind what `from` holds; closing makes `to` wait.
 cudaError_t open_side(kvs_ctx::Side& sd, cudaStream_t from, bool urgent) {
   cudaError_t e = cudaSuccess;
-  if (!sd.stream) {
-    int least = 0, greatest = 0;
-    if ((e = cudaDeviceGetStreamPriorityRange(&least, &greatest)) != cudaSuccess ||
-        (e = cudaStreamCreateWithPriority(&sd.stream, cudaStreamNonBlocking, urgent ? greatest : least)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&sd.from, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&sd.done, cudaEventDisableTiming)) != cudaSuccess)
-      return e;
-  }
+  int least = 0, greatest = 0;
+  if (!sd.stream && ((e = cudaDeviceGetStreamPriorityRange(&least, &greatest)) != cudaSuccess ||
+                     (e = cudaStreamCreateWithPriority(&sd.stream, cudaStreamNonBlocking, urgent ? greatest : least)) != cudaSuccess))
+    return e;
+  for (cudaEvent_t* ev : {&sd.from, &sd.done})
+    if (!*ev && (e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) return e;
   if ((e = cudaEventRecord(sd.from, from)) != cudaSuccess) return e;
   sd.open = true;
   return cudaStreamWaitEvent(sd.stream, sd.from, 0);
 }
 cudaError_t close_side(kvs_ctx::Side& sd, cudaStream_t to) {
   if (!sd.open) return cudaSuccess;
-  sd.open = false;
-  const cudaError_t e = cudaEventRecord(sd.done, sd.stream);
-  return e != cudaSuccess ? e : cudaStreamWaitEvent(to, sd.done, 0);
+  cudaError_t e = cudaEventRecord(sd.done, sd.stream);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(to, sd.done, 0);
+  if (e != cudaSuccess) e = cudaStreamSynchronize(sd.stream);   // the events failed: wait here
+  if (e == cudaSuccess) sd.open = false;
+  return e;
 }
 cudaError_t close_sides(kvs_ctx* ctx) {
   cudaError_t e = cudaSuccess;
@@ -308,9 +314,8 @@ int64_t lane_light_ctas(const kvs_setting* st, int64_t P) {
   return 0;                                  // no evaluation of the light variant (no profile is stored here)
 }
 
-int run_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settings, int64_t P,
-              const kvs_schedule_out* out, const kvs_eval_out* ev, int do_profile, const FusedRange* rg = nullptr) {
-  if (!ctx) return KVS_E_STATE;
+int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settings, int64_t P,
+                  const kvs_schedule_out* out, const kvs_eval_out* ev, int do_profile, const FusedRange* rg) {
   int rc = check_instances(ctx, inst);
   if (rc) return rc;
   rc = check_settings(ctx, inst, settings, P);
@@ -376,7 +381,6 @@ int run_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settin
     for (const auto& x : two) { pairs[2 * n_pairs] = x.first; pairs[2 * n_pairs + 1] = x.second; ++n_pairs; }
   }
   if (n_refill || n_spec) {
-    if (rg) return fail(ctx, KVS_E_ARG, "the host entry point takes neither the dynamic refill nor speculative runs (they need per-job results and a profile on the device)");
     if (do_profile && (!o.job_start || !o.job_completion || !v.profile || o.job_start64 || o.job_completion64 || run_out))
       return fail(ctx, KVS_E_ARG, "the dynamic refill and speculative runs need job_start, job_completion and a profile (32-bit, no run list): they are their working storage");
     if (do_profile && (!v.horizon || !v.status))
@@ -627,6 +631,16 @@ int run_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settin
   return KVS_OK;
 }
 
+// A device entry point.  Where it fails half-way, what it has launched on a stream of its own is put in front of whatever the
+// caller does next on the context's stream.
+int run_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settings, int64_t P,
+              const kvs_schedule_out* out, const kvs_eval_out* ev, int do_profile) {
+  if (!ctx) return KVS_E_STATE;
+  const int rc = enqueue_fused(ctx, inst, settings, P, out, ev, do_profile, nullptr);
+  if (rc) close_sides(ctx);
+  return rc;
+}
+
 }  // namespace
 
 extern "C" {
@@ -776,15 +790,16 @@ int kvs_evaluate_built(kvs_ctx* ctx, const kvs_instances* inst, const kvs_settin
   return run_fused(ctx, inst, settings, P, out, ev, 1);
 }
 
-int kvs_evaluate_built_host(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settings, int64_t P,
-                            const kvs_eval_out* ev) {
-  if (!ctx) return KVS_E_STATE;
+static int evaluate_built_host(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settings, int64_t P, const kvs_eval_out* ev, bool* begun) {
   int rc = check_instances(ctx, inst);
   if (rc) return rc;
   if (!ev) return fail(ctx, KVS_E_ARG, "eval_out: null");
   if (ev->profile) return fail(ctx, KVS_E_ARG, "host entry point returns scalars only (profile must be NULL)");
   rc = check_settings(ctx, inst, settings, P);
   if (rc) return rc;
+  for (int64_t e = 0; e < P; ++e)
+    if (settings[e].family == KVS_GBAD || settings[e].family == KVS_GSAS)
+      return fail(ctx, KVS_E_ARG, "the host entry point takes neither the dynamic refill nor speculative runs (they need per-job results and a profile on the device)");
   const int64_t N = inst->n_jobs_total, I = inst->n_instances;
   for (int64_t i = 0; i < I; ++i)
     if (inst->job_off[i] < 0 || inst->job_off[i + 1] < inst->job_off[i] || inst->job_off[i + 1] > N)
@@ -793,11 +808,10 @@ int kvs_evaluate_built_host(kvs_ctx* ctx, const kvs_instances* inst, const kvs_s
   if (L.total > ctx->workspace_bytes) return fail(ctx, KVS_E_CAPACITY, "workspace too small for host staging (see kvs_workspace_bytes)");
   cudaError_t ce = cudaSetDevice(ctx->device);
   if (ce != cudaSuccess) return fail_cuda(ctx, ce, "cudaSetDevice");
-  if (!ctx->copy_stream) {
-    if ((ce = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking)) != cudaSuccess) return fail_cuda(ctx, ce, "cudaStreamCreate");
-    for (cudaEvent_t& e : ctx->chunk_ev)
-      if ((ce = cudaEventCreateWithFlags(&e, cudaEventDisableTiming)) != cudaSuccess) return fail_cuda(ctx, ce, "cudaEventCreate");
-  }
+  if (!ctx->copy_stream && (ce = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking)) != cudaSuccess)
+    return fail_cuda(ctx, ce, "cudaStreamCreate");
+  for (cudaEvent_t& e : ctx->chunk_ev)
+    if (!e && (ce = cudaEventCreateWithFlags(&e, cudaEventDisableTiming)) != cudaSuccess) return fail_cuda(ctx, ce, "cudaEventCreate");
   unsigned char* ws = ctx->workspace;
 
   // Evaluations are worked off chunk of instances by chunk of instances, so that the copy of the
@@ -826,6 +840,7 @@ int kvs_evaluate_built_host(kvs_ctx* ctx, const kvs_instances* inst, const kvs_s
   d.feasible = reinterpret_cast<uint8_t*>(ws + L.sc_feas);
   d.status = reinterpret_cast<int32_t*>(ws + L.sc_stat);
 
+  *begun = true;
   // the staging areas may still be read by earlier work on the context's stream
   if ((ce = cudaEventRecord(ctx->chunk_ev[KVS_HOST_CHUNKS], ctx->stream)) != cudaSuccess ||
       (ce = cudaStreamWaitEvent(ctx->copy_stream, ctx->chunk_ev[KVS_HOST_CHUNKS], 0)) != cudaSuccess)
@@ -868,7 +883,7 @@ int kvs_evaluate_built_host(kvs_ctx* ctx, const kvs_instances* inst, const kvs_s
       kvs_eval_out dc = d;
       dc.peak += r0; dc.flow += r0; dc.job_steps += r0; dc.horizon += r0; dc.n_unfinished += r0; dc.feasible += r0; dc.status += r0;
       const FusedRange rg{i0, i1, r0, P, static_cast<int>(c), lane, light_ctas, feed};
-      rc = run_fused(ctx, &dev, sorted.data() + r0, r1 - r0, nullptr, &dc, 1, &rg);
+      rc = enqueue_fused(ctx, &dev, sorted.data() + r0, r1 - r0, nullptr, &dc, 1, &rg);
       if (rc) return rc;
     } else if ((rc = feed()) != KVS_OK) {
       return rc;
@@ -918,6 +933,22 @@ int kvs_evaluate_built_host(kvs_ctx* ctx, const kvs_instances* inst, const kvs_s
     }
   }
   return KVS_OK;
+}
+
+int kvs_evaluate_built_host(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settings, int64_t P,
+                            const kvs_eval_out* ev) {
+  if (!ctx) return KVS_E_STATE;
+  bool begun = false;                        // something may have been enqueued
+  const int rc = evaluate_built_host(ctx, inst, settings, P, ev, &begun);
+  if (rc && begun) {
+    // Whatever has been enqueued before the failure is over before the caller, who may free or reuse the buffers, has the
+    // status: the lanes and their side streams, the copies, then the context's stream.
+    for (kvs_ctx::Side& sd : ctx->side)
+      if (sd.open) { cudaStreamSynchronize(sd.stream); sd.open = false; }
+    if (ctx->copy_stream) cudaStreamSynchronize(ctx->copy_stream);
+    cudaStreamSynchronize(ctx->stream);
+  }
+  return rc;
 }
 
 static int check_runs(kvs_ctx* ctx, const kvs_runs* runs, const kvs_eval_out* ev) {
@@ -1004,8 +1035,8 @@ int kvs_bounds(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* setti
   // every evaluation reads its setting twice: straight from the page-locked slot, without an upload before the kernels
   ce = kvs_launch_bounds(inst->job_off, inst->s, inst->o, max_n, reinterpret_cast<InstStats*>(ws + L.stats), geo, P, runs, n_runs, *out,
                          reinterpret_cast<u32*>(ws + L.class_counts), ctx->stream);
-  if (ce == cudaSuccess) ce = cudaEventRecord(stg->done, ctx->stream);
-  stg->used = true;
+  const cudaError_t marked = mark_stage(stg, ctx->stream);   // also after a failure: one of the two kernels may be running
+  if (ce == cudaSuccess) ce = marked;
   if (ce != cudaSuccess) return fail_cuda(ctx, ce, "bounds launch");
   return KVS_OK;
 }

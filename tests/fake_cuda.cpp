@@ -102,7 +102,7 @@ cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) { host.join(stream_of(s)->clock); return fails() ? cudaErrorUnknown : cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { for (Stream* s : streams) host.join(s->clock); return cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
-  if (fails()) return cudaErrorUnknown;
+  if (fails() || !e) return cudaErrorUnknown;
   stream_of(s)->clock.join(reinterpret_cast<Event*>(e)->clock);
   return cudaSuccess;
 }
@@ -116,7 +116,7 @@ cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 0.f; return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
-  if (fails()) return cudaErrorUnknown;
+  if (fails() || !e) return cudaErrorUnknown;
   Stream* st = stream_of(s);
   st->clock.join(host);
   reinterpret_cast<Event*>(e)->clock = st->clock;
@@ -308,11 +308,50 @@ void overlaps() {
   }
 }
 
+// A refused call enqueues nothing; a call that fails half-way (every fallible call of the runtime and every launch in turn) leaves
+// nothing behind that the next call could meet.
+void errors() {
+  Batch b(520);
+  for (int i = 0; i < b.I; ++i) for (int f = KVS_GBA; f <= KVS_SIMS; ++f) b.add(i, f);
+  auto next_call = [&](const char* name, Caller& c) {
+    if (host_call(c, b) != KVS_OK) { printf("%s: the next call fails\n", name); ++races; }
+    find_races();
+  };
+  for (int family : {KVS_GBAD, KVS_GSAS}) {
+    Batch bad = b;
+    bad.st.back().family = family;
+    Caller c(b.I, static_cast<i64>(b.st.size()));
+    if (host_call(c, bad) != KVS_E_ARG || !ops.empty()) { printf("family %d: %zu operations of a refused call\n", family, ops.size()); ++races; }
+    next_call("refused", c);
+  }
+  const kvs_instances in = view(b);
+  std::vector<i64> peak(b.st.size());
+  kvs_eval_out ev{};
+  ev.peak = peak.data();
+  for (bool device : {false, true}) {
+    int rc = KVS_E_CUDA, n = 0;
+    for (; rc != KVS_OK && n < 2000; ++n) {
+      Caller c(b.I, static_cast<i64>(b.st.size()));
+      calls = 0;
+      fail_at = n;
+      rc = device ? kvs_evaluate_built(c.ctx, &in, b.st.data(), static_cast<i64>(b.st.size()), nullptr, &ev) : host_call(c, b);
+      fail_at = -1;
+      // the host entry point is over when it returns; what a device one has launched precedes the stream's next work
+      if (const int left = outstanding(device ? stream_of(nullptr)->clock : host)) {
+        if (races++ < 5) printf("%s call, failure %d: %d operations in flight\n", device ? "device" : "host", n, left);
+      }
+      next_call("after a failure", c);
+    }
+    if (n < (device ? 10 : 80) || n == 2000) { printf("%d failures\n", n); ++races; }
+  }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "overlaps") overlaps();
+  else if (what == "errors") errors();
   else { printf("unknown program\n"); return 2; }
   printf("%s: %d faults\n", what.c_str(), races);
   return races ? 1 : 0;

@@ -311,6 +311,28 @@ def test_host_entry_point_uneven_chunks(par, I, growing):
             assert torch.equal(v, getattr(want, k).cpu()), k
 
 
+@pytest.mark.parametrize("family", ["GBAD", "GSAS"])
+def test_host_entry_point_refuses_before_it_launches(par, family):
+    """A batch with one setting that the host entry point does not take is refused whole; the call right behind it is right."""
+    from paper_2601_22996_b200.api import Scheduler
+    inst = workloads.random_small(603, n_inst=520, n_max=60, s_max=30, o_max=90)
+    M = _tight_M(inst, 300)
+    st = _all_settings(inst, lambda i: M[i])
+    bad = st.copy()
+    bad["family"][-1] = binding.FAMILY[family]
+    P, I, n = st.shape[0], inst.n_instances, int((inst.job_off[1:] - inst.job_off[:-1]).max())
+    sched = par.scheduler()
+    want = sched.evaluate(inst.to("cuda:0"), st, want_jobs=False)
+    ctx = sched.context(binding.workspace_bytes(int(inst.s.numel()), I, n, P, host_staging=True))
+    hin = workloads.Instances(inst.job_off, inst.s.pin_memory(), inst.o.pin_memory())
+    hev = {k: torch.full_like(v, -5, device="cpu").pin_memory() for k, v in Scheduler.scalars(P, "cpu").items()}
+    with pytest.raises(binding.KvsError, match="host entry point takes neither"):
+        ctx.evaluate_built_host(hin, bad, hev, window=0, max_jobs=n)
+    ctx.evaluate_built_host(hin, st, hev, window=0, max_jobs=n)
+    for k, v in hev.items():
+        assert torch.equal(v, getattr(want, k).cpu()), k
+
+
 @pytest.mark.parametrize("copies,runs", [(1, False), (80, False), (1, True)])      # shared evaluations, one CTA each, general kernel
 def test_outputs_of_evaluations_that_form_none(par, copies, runs):
     """Per-job results of an infeasible evaluation and rounds behind the end of a schedule take the values that the caller sets;

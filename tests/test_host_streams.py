@@ -27,3 +27,9 @@ def test_chunks_of_the_host_entry_point_share_no_scratch(program):
     """Chunks of unequal size or composition take turns on the lanes: no kernel uses scratch, results or inputs that another
     one, not ordered before or after it, writes."""
     _run(program, "overlaps")
+
+
+def test_failures_leave_nothing_in_flight(program):
+    """A refused call launches nothing; after one that fails at any point, no kernel and no copy of it is left for the next call to
+    race with."""
+    _run(program, "errors")
