@@ -311,6 +311,25 @@ def test_host_entry_point_uneven_chunks(par, I, growing):
             assert torch.equal(v, getattr(want, k).cpu()), k
 
 
+def test_capacities_written_by_the_library(par):
+    """One horizon tensor, filled by the library's kernels for one batch after the other, as the profile capacity of each."""
+    P = 8
+    first = par.scheduler().scalars(P, torch.device("cuda:0"))
+    for seed in (604, 605):
+        inst = workloads.random_small(seed, n_inst=P, n_max=40 * (seed - 603), s_max=20, o_max=60 * (seed - 603)).to("cuda:0")
+        st = binding.make_settings([dict(instance=i, family="GSA", M=400) for i in range(P)])
+        n = int((inst.job_off[1:] - inst.job_off[:-1]).max())
+        ctx = par.scheduler().context(binding.workspace_bytes(int(inst.s.numel()), P, n, P))
+        ctx.build_schedule(inst, st, dict(n_runs=torch.zeros(P, dtype=torch.int64, device="cuda:0")), first, max_jobs=n)
+        res = par.scheduler().evaluate(inst, st, want_profile=True, profile_capacity=first["horizon"])
+        assert res.status.tolist() == [0] * P and torch.equal(res.horizon, first["horizon"])
+        assert torch.equal(res.profile_off[1:] - res.profile_off[:-1], first["horizon"]) and int(res.profile.min()) >= 0
+        runs = dict(run_off=torch.arange(P + 1, device="cuda:0"), run_start=torch.zeros(P, dtype=torch.int64, device="cuda:0"),
+                    run_len=first["horizon"].to(torch.int32), run_s=torch.ones(P, dtype=torch.int32, device="cuda:0"))
+        res = par.scheduler().evaluate_runs(**runs, capacity=first["horizon"])
+        assert res.status.tolist() == [0] * P and torch.equal(res.peak, first["horizon"] + 1)
+
+
 @pytest.mark.parametrize("family", ["GBAD", "GSAS"])
 def test_host_entry_point_refuses_before_it_launches(par, family):
     """A batch with one setting that the host entry point does not take is refused whole; the call right behind it is right."""

@@ -51,6 +51,19 @@ def test_no_gpu_means_a_loud_failure():
     assert binding.workspace_bytes(10_000, 4, 5_000, 16) > 0        # host-only entry point still works
 
 
+def test_sizes_are_read_on_every_call():
+    """Sizes written through a raw pointer - the tensor's version counter stays - count from the next call on."""
+    from paper_2601_22996_b200.api import Scheduler
+    off = torch.tensor([0, 3, 7])
+    inst = workloads.Instances(off, torch.ones(7, dtype=torch.int32), torch.ones(7, dtype=torch.int32))
+    assert Scheduler._sizes(inst)[2] == 4
+    version = off._version
+    off.numpy()[1] = 1
+    assert off._version == version
+    N, I, largest, n_per = Scheduler._sizes(inst)
+    assert (N, I, largest, n_per.tolist()) == (7, 2, 6, [1, 6])
+
+
 def test_generators_are_deterministic_and_in_range():
     a, b = workloads.config2(n_inst=3, n=500), workloads.config2(n_inst=3, n=500)
     assert torch.equal(a.s, b.s) and torch.equal(a.o, b.o)
