@@ -330,6 +330,21 @@ def test_capacities_written_by_the_library(par):
         assert res.status.tolist() == [0] * P and torch.equal(res.peak, first["horizon"] + 1)
 
 
+def test_capacities_of_the_wrong_shape_are_refused(par):
+    inst = workloads.random_small(606, n_inst=2, n_max=20, s_max=9, o_max=20).to("cuda:0")
+    st = binding.make_settings([dict(instance=i, family="GSA", M=400) for i in range(2)])
+    one = torch.tensor([64], device="cuda:0")
+    for want_jobs in (False, True):
+        with pytest.raises(binding.KvsError):
+            par.scheduler().evaluate(inst, st, want_jobs=want_jobs, want_profile=True, profile_capacity=one)
+    i32 = dict(dtype=torch.int32, device="cuda:0")
+    runs = dict(run_off=torch.arange(3, device="cuda:0"), run_start=torch.zeros(2, dtype=torch.int64, device="cuda:0"),
+                run_len=torch.ones(2, **i32), run_s=torch.ones(2, **i32))
+    with pytest.raises(binding.KvsError):
+        par.scheduler().evaluate_runs(**runs, capacity=one)
+    assert par.scheduler().evaluate_runs(**runs, capacity=torch.tensor([4, 4])).peak.tolist() == [2, 2]      # sizes may be host values
+
+
 @pytest.mark.parametrize("family", ["GBAD", "GSAS"])
 def test_host_entry_point_refuses_before_it_launches(par, family):
     """A batch with one setting that the host entry point does not take is refused whole; the call right behind it is right."""

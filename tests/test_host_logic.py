@@ -64,6 +64,14 @@ def test_sizes_are_read_on_every_call():
     assert (N, I, largest, n_per.tolist()) == (7, 2, 6, [1, 6])
 
 
+def test_capacities_of_the_wrong_shape_are_refused():
+    from paper_2601_22996_b200.api import Scheduler
+    assert Scheduler._per_eval(np.arange(3), 3, "capacity").tolist() == [0, 1, 2]
+    for wrong in (np.arange(2), np.arange(4), np.zeros((3, 1)), np.zeros(())):
+        with pytest.raises(binding.KvsError):
+            Scheduler._per_eval(wrong, 3, "capacity")
+
+
 def test_generators_are_deterministic_and_in_range():
     a, b = workloads.config2(n_inst=3, n=500), workloads.config2(n_inst=3, n=500)
     assert torch.equal(a.s, b.s) and torch.equal(a.o, b.o)
