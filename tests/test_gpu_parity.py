@@ -345,6 +345,41 @@ def test_capacities_of_the_wrong_shape_are_refused(par):
     assert par.scheduler().evaluate_runs(**runs, capacity=torch.tensor([4, 4])).peak.tolist() == [2, 2]      # sizes may be host values
 
 
+def test_calls_under_another_stream(par):
+    """A scheduler made under one stream and called under another that is still busy making the inputs: results as on its own."""
+    from paper_2601_22996_b200.api import Scheduler
+    sched, other = Scheduler(), torch.cuda.Stream()
+    inst = workloads.random_small(607, n_inst=12, n_max=200, s_max=30, o_max=200)
+    st = _all_settings(inst, lambda i: 900)
+    P = st.shape[0]
+
+    def calls(inst, wait):
+        wait()
+        cap = torch.full((P,), 4096, dtype=torch.int64, device="cuda:0")
+        yield vars(sched.evaluate(inst, st))
+        wait()
+        yield vars(sched.evaluate(inst, st, want_profile=True, profile_capacity=cap))
+        wait()
+        yield vars(sched.evaluate(inst, st, want_profile=True, want_runs=True))
+        start = inst.o.to(torch.int64)
+        wait()
+        yield vars(sched.evaluate_runs(inst.job_off, start, inst.o, inst.s, cap[:inst.n_instances]))
+        yield sched.bounds(inst, st[st["family"] == binding.GBA])
+        yield sched.sweep_beta0(inst, 1, "GSA", 900, [0, 3, 16])
+        yield sched.sweep(inst, 1, "SPS", 900, [2, 16], [1, 8])
+
+    def flat(results):
+        return [{k: v.cpu() for k, v in r.items() if isinstance(v, torch.Tensor)} for r in results]
+
+    want = flat(calls(inst.to("cuda:0"), lambda: None))
+    with torch.cuda.stream(other):
+        got = flat(calls(inst.to("cuda:0"), lambda: torch.cuda._sleep(10_000_000)))
+    for a, b in zip(want, got, strict=True):
+        assert a.keys() == b.keys()
+        for k in a:
+            assert torch.equal(a[k], b[k]), k
+
+
 @pytest.mark.parametrize("family", ["GBAD", "GSAS"])
 def test_host_entry_point_refuses_before_it_launches(par, family):
     """A batch with one setting that the host entry point does not take is refused whole; the call right behind it is right."""
