@@ -167,7 +167,6 @@ __global__ void __launch_bounds__(BT, 3) k_class_counts(const i64* __restrict__ 
   for (i64 first = e0; first < e0 + n_e; first += BT / 32) {
     if (first != e0) { fetch(first); __syncthreads(); }
     const int m = static_cast<int>(min_i64(BT / 32, e0 + n_e - first));
-    bool rest = false;
     if (warp < m) {                                         // alpha = 2, every response in the histogram: one warp per setting
       const kvs_setting& st = sts[warp];
       const Case c = case_of(job_off, is, st);
@@ -185,7 +184,6 @@ __global__ void __launch_bounds__(BT, 3) k_class_counts(const i64* __restrict__ 
       const Case c = case_of(job_off, is, st);
       if (c.status || (is_pow2(st) && o_max < BINS)) continue;
       const i64 e = first + x;
-      rest = true;
       if (tid < 32) ladder_phases(sh, c.X, st.alpha_num, st.alpha_den, st.beta0, [](u32) { return 0u; });
       for (int i = tid; i < MAXP; i += BT) cnt[i] = 0;
       __syncthreads();
@@ -200,7 +198,7 @@ __global__ void __launch_bounds__(BT, 3) k_class_counts(const i64* __restrict__ 
       }
       __syncthreads();                                      // the next setting writes the tables again
     }
-    if (!rest) __syncthreads();                             // before the next settings are fetched
+    __syncthreads();                                        // every warp has read these settings before the next are fetched
   }
 }
 

@@ -100,3 +100,17 @@ def test_lengths_around_the_histogram(sched, o_max):
     _check(sched, inst, binding.make_settings(rows))
     _check(sched, inst, binding.make_settings([rows[k] for k in np.random.default_rng(3).permutation(len(rows))]))
     _check(sched, inst, binding.make_settings(rows[:1]))
+
+
+def test_long_runs_of_mixed_settings(sched):
+    """More settings per instance than a CTA holds at a time: those that the histogram serves, those that the whole CTA counts, and
+    infeasible ones, in any order and with an infeasible one last."""
+    inst = workloads.random_small(73, n_inst=90, n_max=120, s_max=40, o_max=300)
+    rng = np.random.default_rng(74)
+    rows = []
+    for i in range(inst.n_instances):
+        mine = [dict(instance=i, family="GBA", M=m + k, alpha=al) for k in range(10) for m in (20, 1000, 1 << 16) for al in ((2, 1), (3, 2), (7, 4))]
+        rows += [mine[k] for k in rng.permutation(len(mine))] + [dict(instance=i, family="GBA", M=15)]
+    st = binding.make_settings(rows)
+    assert st.shape[0] >= 17 * 3 * 148
+    _check(sched, inst, st, sample=sorted(rng.choice(st.shape[0], 400, replace=False)))
