@@ -38,7 +38,7 @@ enum kvs_status {
   KVS_E_CUDA = -2,      /* a CUDA runtime call failed; see kvs_last_error */
   KVS_E_CAPACITY = -3,  /* workspace too small */
   KVS_E_RANGE = -4,     /* a parameter is outside the supported range */
-  KVS_E_STATE = -5      /* context not initialised / wrong device */
+  KVS_E_STATE = -5      /* context not initialised / wrong device / no host memory left */
 };
 
 /* Schedule families.  GBA: Algorithm "Geometric Batching Algorithm"; GSA: Algorithm

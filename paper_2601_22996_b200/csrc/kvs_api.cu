@@ -53,12 +53,23 @@ namespace {
 constexpr int64_t KVS_MAX_GRID = 1024;        // upper bound on CTAs of the fused kernel (sizes the carry lists)
 constexpr int64_t KVS_TIME_LIMIT = 1ll << 31; // exclusive bound on M, tau, k
 
+// Nothing leaves a C entry point as an exception: host memory that runs out becomes a status (and, for the text of an error,
+// an empty text).
+template <class F>
+int guarded(kvs_ctx* ctx, F body) noexcept {
+  try {
+    return body();
+  } catch (...) {
+    ctx->err.clear();
+    return KVS_E_STATE;
+  }
+}
 int fail(kvs_ctx* ctx, int code, const char* msg) {
-  if (ctx) ctx->err = msg;
+  if (ctx) guarded(ctx, [&] { ctx->err = msg; return 0; });
   return code;
 }
 int fail_cuda(kvs_ctx* ctx, cudaError_t e, const char* where) {
-  if (ctx) ctx->err = std::string(where) + ": " + cudaGetErrorString(e);
+  if (ctx) guarded(ctx, [&] { ctx->err = std::string(where) + ": " + cudaGetErrorString(e); return 0; });
   return KVS_E_CUDA;
 }
 
@@ -636,7 +647,7 @@ int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* se
 int run_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settings, int64_t P,
               const kvs_schedule_out* out, const kvs_eval_out* ev, int do_profile) {
   if (!ctx) return KVS_E_STATE;
-  const int rc = enqueue_fused(ctx, inst, settings, P, out, ev, do_profile, nullptr);
+  const int rc = guarded(ctx, [&] { return enqueue_fused(ctx, inst, settings, P, out, ev, do_profile, nullptr); });
   if (rc) close_sides(ctx);
   return rc;
 }
@@ -939,7 +950,7 @@ int kvs_evaluate_built_host(kvs_ctx* ctx, const kvs_instances* inst, const kvs_s
                             const kvs_eval_out* ev) {
   if (!ctx) return KVS_E_STATE;
   bool begun = false;                        // something may have been enqueued
-  const int rc = evaluate_built_host(ctx, inst, settings, P, ev, &begun);
+  const int rc = guarded(ctx, [&] { return evaluate_built_host(ctx, inst, settings, P, ev, &begun); });
   if (rc && begun) {
     // Whatever has been enqueued before the failure is over before the caller, who may free or reuse the buffers, has the
     // status: the lanes and their side streams, the copies, then the context's stream.
@@ -1041,8 +1052,7 @@ int kvs_bounds(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* setti
   return KVS_OK;
 }
 
-int kvs_sweep(kvs_ctx* ctx, const kvs_instances* inst, const kvs_sweep_params* params, const kvs_sweep_out* out) {
-  if (!ctx) return KVS_E_STATE;
+static int sweep(kvs_ctx* ctx, const kvs_instances* inst, const kvs_sweep_params* params, const kvs_sweep_out* out) {
   int rc = check_instances(ctx, inst);
   if (rc) return rc;
   if (!params || !out) return fail(ctx, KVS_E_ARG, "sweep: params or out is null");
@@ -1132,6 +1142,11 @@ int kvs_sweep(kvs_ctx* ctx, const kvs_instances* inst, const kvs_sweep_params* p
   ce = kvs_launch_sweep(wp, reinterpret_cast<i64*>(ws + L.table), ctx->stream);
   if (ce != cudaSuccess) return fail_cuda(ctx, ce, "sweep launch");
   return KVS_OK;
+}
+
+int kvs_sweep(kvs_ctx* ctx, const kvs_instances* inst, const kvs_sweep_params* params, const kvs_sweep_out* out) {
+  if (!ctx) return KVS_E_STATE;
+  return guarded(ctx, [&] { return sweep(ctx, inst, params, out); });
 }
 
 }  // extern "C"

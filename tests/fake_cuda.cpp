@@ -7,7 +7,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <map>
+#include <new>
 #include <random>
 #include <string>
 #include <vector>
@@ -32,17 +32,25 @@ std::vector<Stream*> streams;
 std::vector<Op> ops;
 Clock host;
 int calls = 0, fail_at = -1, races = 0;
+long news = 0, no_memory_at = -1;      // allocations of the library's host code while `library` is set, and the one that fails
+bool library = false;
 
 Stream* stream_of(cudaStream_t s) {
   if (streams.empty()) streams.push_back(new Stream{0, {}});       // the default stream
   return s ? reinterpret_cast<Stream*>(s) : streams[0];
 }
 bool fails() { return calls++ == fail_at; }
+struct Outside {                       // the fake's own allocations neither count nor fail
+  bool was = library;
+  Outside() { library = false; }
+  ~Outside() { library = was; }
+};
 Access span(const void* p, size_t bytes, Kind kind) {
   const unsigned char* a = static_cast<const unsigned char*>(p);
   return Access{a, a ? a + bytes : a, kind};
 }
 void submit(const char* name, cudaStream_t s, std::vector<Access> acc) {
+  Outside outside;
   Stream* st = stream_of(s);
   st->clock.join(host);
   const long seq = ++st->clock.at[st->id];
@@ -81,6 +89,14 @@ int outstanding(const Clock& c) {
 
 }  // namespace
 
+void* operator new(size_t n) {
+  if (library && news++ == no_memory_at) throw std::bad_alloc();
+  if (void* p = malloc(n ? n : 1)) return p;
+  throw std::bad_alloc();
+}
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
+
 // ---- the runtime ------------------------------------------------------------------------------------------------
 
 extern "C" {
@@ -90,6 +106,7 @@ cudaError_t cudaGetDeviceProperties_v2(cudaDeviceProp* p, int) { memset(p, 0, si
 const char* cudaGetErrorString(cudaError_t) { return "made to fail"; }
 cudaError_t cudaDeviceGetStreamPriorityRange(int* least, int* greatest) { *least = 0; *greatest = -5; return fails() ? cudaErrorUnknown : cudaSuccess; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
+  Outside outside;
   if (fails()) return cudaErrorUnknown;
   stream_of(nullptr);
   if (streams.size() >= MAX_STREAMS) { printf("more than %d streams\n", MAX_STREAMS); exit(2); }
@@ -107,6 +124,7 @@ cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
   return cudaSuccess;
 }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) {
+  Outside outside;
   if (fails()) return cudaErrorUnknown;
   *e = reinterpret_cast<cudaEvent_t>(new Event{});
   return cudaSuccess;
@@ -126,6 +144,7 @@ cudaError_t cudaEventSynchronize(cudaEvent_t e) { host.join(reinterpret_cast<Eve
 cudaError_t cudaMallocHost(void** p, size_t n) { if (fails()) return cudaErrorUnknown; *p = calloc(1, n); return cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { free(p); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t n, cudaMemcpyKind, cudaStream_t s) {
+  Outside outside;
   if (fails()) return cudaErrorUnknown;
   memcpy(dst, src, n);
   submit("copy", s, {span(dst, n, WRITE), span(src, n, READ)});
@@ -136,6 +155,7 @@ cudaError_t cudaMemcpy(void* dst, const void* src, size_t n, cudaMemcpyKind k) {
   return e != cudaSuccess ? e : cudaStreamSynchronize(nullptr);
 }
 cudaError_t cudaMemsetAsync(void* dst, int v, size_t n, cudaStream_t s) {
+  Outside outside;
   if (fails()) return cudaErrorUnknown;
   memset(dst, v, n);
   submit("memset", s, {span(dst, n, WRITE)});
@@ -160,6 +180,7 @@ cudaError_t kvs_refill_check_word(unsigned long long*, int*, int) { return cudaS
 cudaError_t kvs_spec_check_word(unsigned long long*, int*, int) { return cudaSuccess; }
 
 cudaError_t kvs_launch_sort(const SortParams& p, int, cudaStream_t s) {
+  Outside outside;
   if (fails()) return cudaErrorUnknown;
   const i64 lo = p.job_off[0], n = p.job_off[p.n_instances] - lo;
   std::vector<Access> a = {span(p.job_off, 8 * (p.n_instances + 1), READ), span(p.s + lo, 4 * n, READ), span(p.o + lo, 4 * n, READ),
@@ -188,6 +209,7 @@ void scratch(const BuildParams& p, int grid, std::vector<Access>* a) {
 }  // namespace
 
 cudaError_t kvs_launch_fused(const BuildParams& p, int grid, int light, int fam, cudaStream_t s) {
+  Outside outside;
   if (fails()) return cudaErrorUnknown;
   std::vector<Access> a;
   scratch(p, grid, &a);
@@ -198,6 +220,7 @@ cudaError_t kvs_launch_fused(const BuildParams& p, int grid, int light, int fam,
   return cudaSuccess;
 }
 cudaError_t kvs_launch_build(const BuildParams& p, int grid, cudaStream_t s) {
+  Outside outside;
   if (fails()) return cudaErrorUnknown;
   std::vector<Access> a;
   scratch(p, grid, &a);
@@ -272,7 +295,20 @@ int host_call(Caller& c, const Batch& b) {
   kvs_eval_out ev{};
   ev.peak = peak.data(); ev.flow = flow.data(); ev.status = status.data();
   const kvs_instances in = view(b);
-  return kvs_evaluate_built_host(c.ctx, &in, b.st.data(), static_cast<i64>(P), &ev);
+  library = true;
+  const int rc = kvs_evaluate_built_host(c.ctx, &in, b.st.data(), static_cast<i64>(P), &ev);
+  library = false;
+  return rc;
+}
+int device_call(Caller& c, const Batch& b) {
+  std::vector<i64> peak(b.st.size());
+  kvs_eval_out ev{};
+  ev.peak = peak.data();
+  const kvs_instances in = view(b);
+  library = true;
+  const int rc = kvs_evaluate_built(c.ctx, &in, b.st.data(), static_cast<i64>(b.st.size()), nullptr, &ev);
+  library = false;
+  return rc;
 }
 
 void run_host(const char* name, const Batch& b) {
@@ -308,8 +344,8 @@ void overlaps() {
   }
 }
 
-// A refused call enqueues nothing; a call that fails half-way (every fallible call of the runtime and every launch in turn) leaves
-// nothing behind that the next call could meet.
+// A refused call enqueues nothing; a call that fails half-way (every fallible call of the runtime, every launch and every
+// allocation in turn) returns a status and leaves nothing behind that the next call could meet.
 void errors() {
   Batch b(520);
   for (int i = 0; i < b.I; ++i) for (int f = KVS_GBA; f <= KVS_SIMS; ++f) b.add(i, f);
@@ -324,26 +360,28 @@ void errors() {
     if (host_call(c, bad) != KVS_E_ARG || !ops.empty()) { printf("family %d: %zu operations of a refused call\n", family, ops.size()); ++races; }
     next_call("refused", c);
   }
-  const kvs_instances in = view(b);
-  std::vector<i64> peak(b.st.size());
-  kvs_eval_out ev{};
-  ev.peak = peak.data();
-  for (bool device : {false, true}) {
-    int rc = KVS_E_CUDA, n = 0;
-    for (; rc != KVS_OK && n < 2000; ++n) {
-      Caller c(b.I, static_cast<i64>(b.st.size()));
-      calls = 0;
-      fail_at = n;
-      rc = device ? kvs_evaluate_built(c.ctx, &in, b.st.data(), static_cast<i64>(b.st.size()), nullptr, &ev) : host_call(c, b);
-      fail_at = -1;
-      // the host entry point is over when it returns; what a device one has launched precedes the stream's next work
-      if (const int left = outstanding(device ? stream_of(nullptr)->clock : host)) {
-        if (races++ < 5) printf("%s call, failure %d: %d operations in flight\n", device ? "device" : "host", n, left);
+  for (bool memory : {false, true})
+    for (bool device : {false, true}) {
+      int rc = KVS_E_CUDA, n = 0;
+      for (; rc != KVS_OK && n < 2000; ++n) {
+        Caller c(b.I, static_cast<i64>(b.st.size()));
+        calls = 0;
+        news = 0;
+        no_memory_at = memory ? n : -1;
+        fail_at = memory ? -1 : n;
+        rc = device ? device_call(c, b) : host_call(c, b);
+        fail_at = -1;
+        no_memory_at = -1;
+        if (rc != KVS_OK && rc != (memory ? KVS_E_STATE : KVS_E_CUDA)) { printf("status %d\n", rc); ++races; }
+        // the host entry point is over when it returns; what a device one has launched precedes the stream's next work
+        if (const int left = outstanding(device ? stream_of(nullptr)->clock : host)) {
+          if (races++ < 5) printf("%s call, failure %d: %d operations in flight\n", device ? "device" : "host", n, left);
+        }
+        next_call("after a failure", c);
       }
-      next_call("after a failure", c);
+      const int least = memory ? (device ? 1 : 4) : (device ? 10 : 80);
+      if (n < least || n == 2000) { printf("%d failures\n", n); ++races; }
     }
-    if (n < (device ? 10 : 80) || n == 2000) { printf("%d failures\n", n); ++races; }
-  }
 }
 
 }  // namespace

@@ -30,6 +30,6 @@ def test_chunks_of_the_host_entry_point_share_no_scratch(program):
 
 
 def test_failures_leave_nothing_in_flight(program):
-    """A refused call launches nothing; after one that fails at any point, no kernel and no copy of it is left for the next call to
-    race with."""
+    """A refused call launches nothing; after one that fails at any point (a runtime call, a launch, host memory), no kernel and no
+    copy of it is left for the next call to race with, and no exception leaves the C entry point."""
     _run(program, "errors")
