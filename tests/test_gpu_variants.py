@@ -115,3 +115,15 @@ def test_variants_peak_without_profile(par, sub, pc):
             for i in (0, 1) for m in (12_000, 1 << 17, 1 << 21) for f in ("GBA", "GSA") for al in ((2, 1), (3, 2)) for s in (-1, 100)]
     for copies in (1, 4):
         par.check_batch(inst, binding.make_settings(rows * copies), want_runs=False, want_profile=False, label="peak of variants")
+
+
+def test_sweep_over_the_only_instance_of_a_larger_array(par):
+    """The instance is a part of the arrays: the same results as with arrays of its own."""
+    c = torch.arange(900)
+    s, o = workloads.uniform_int(81, c, 1, 60), workloads.uniform_int(82, c, 1, 300)
+    part = workloads.Instances(torch.tensor([200, 700]), s, o).to("cuda:0")
+    own = workloads.Instances(torch.tensor([0, 500]), s[200:700].clone(), o[200:700].clone()).to("cuda:0")
+    for fam in ("GBA", "GSA"):
+        a, b = (par.scheduler().sweep_beta0(inst, 0, fam, 4000, [0, 5, 64]) for inst in (part, own))
+        for f in a:
+            assert torch.equal(a[f], b[f]), (fam, f)
