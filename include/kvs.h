@@ -204,8 +204,7 @@ typedef struct {
 /* Builds the schedules (start and completion round of every job, optional run list):
  * ordering by (estimated) response length, geometric class / slice assignment, ranks,
  * phase bases, start = base_p + floor(r * tau_p / k_p) (Procedure StaggeredPipelineSchedule),
- * completion = start + o_i.  `settings` is a HOST array of P entries; it is copied to the
- * workspace asynchronously (the caller must not modify it before the stream reaches the copy).
+ * completion = start + o_i.  `settings` is a HOST array of P entries, copied before the call returns.
  * `ev` may be NULL; if given, only its scalar fields and status are filled (no profile, peak = -1). */
 int kvs_build_schedule(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settings, int64_t P,
                        const kvs_schedule_out* out, const kvs_eval_out* ev);
@@ -221,8 +220,8 @@ int kvs_evaluate_built(kvs_ctx* ctx, const kvs_instances* inst, const kvs_settin
  * (and o_est, arrival) to the workspace, runs the fused path, and copies the per-evaluation
  * scalars back.  Every pointer of `inst` and of `ev` is a HOST pointer here (pinned memory
  * makes the copies asynchronous); `ev->profile` must be NULL.  The instances are worked off in up
- * to 16 chunks (of about a thousand evaluations or more, so small batches stay in one piece): the jobs of the next chunk are copied on a second stream while the kernels of the
- * current one run, so the settings may come in any order but are evaluated grouped by instance
+ * to 16 chunks (of about 512 evaluations or more; a batch of fewer than 1,024 evaluations stays in one piece): the jobs of the
+ * next chunks are copied on a second stream while the kernels of the ones before run, so the settings may come in any order but are evaluated grouped by instance
  * (results are returned in the caller's order).  job_off is read on the host and must be
  * nondecreasing.  The call returns after the stream has been synchronised; if it fails, after everything that it
  * had enqueued is over.  KVS_GBAD and KVS_GSAS settings are refused. */
@@ -297,7 +296,7 @@ typedef struct {
 } kvs_bounds_out;
 
 /* Uses instance, M, alpha_num/alpha_den, beta0 and s_bar of each setting (HOST array of P entries,
- * copied to the workspace asynchronously); the family, tau and k are ignored.  The instances must
+ * copied before the call returns); the family, tau and k are ignored.  The instances must
  * be offline (window = 0); estimates, if present, are ignored: the bounds are statements about the
  * exact response lengths.  Asynchronous on the context's stream. */
 int kvs_bounds(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* settings, int64_t P,

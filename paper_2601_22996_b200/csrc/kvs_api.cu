@@ -10,13 +10,9 @@
 
 #include "kvs_internal.cuh"
 
-#ifndef KVS_CHUNK_EVALS
-#define KVS_CHUNK_EVALS 512
-#endif
-#ifndef KVS_LANES
-#define KVS_LANES 3
-#endif
-constexpr int KVS_HOST_CHUNKS = 16;   // the host entry point pipelines copies and kernels over this many chunks
+constexpr int KVS_HOST_CHUNKS = 16;   // the host entry point pipelines copies and kernels over at most this many chunks
+constexpr int KVS_CHUNK_EVALS = 512;  // of about this many evaluations
+constexpr int KVS_LANES = 3;          // that take turns on this many pairs of streams, see open_side
 
 struct kvs_ctx {
   int device = 0;
@@ -375,9 +371,11 @@ int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* se
   // The on-chip kernel of the speculative runs takes two evaluations of one instance per CTA where they fit.
   int64_t* const pairs = reinterpret_cast<int64_t*>(stg->p + pairs_at(P));
   int64_t n_pairs = 0;
-  // That kernel ends first where it has every evaluation in flight within a few turns; with many, the other one's 32 warps per
-  // SM make up for their slower rounds (config 2's lengths, 10,000 jobs: 512 evaluations 56 against 137 ms, 8,192
-  // evaluations 870 against 450 ms; the lines cross at about 1,200).
+  // That kernel ends first where it has every evaluation in flight within a few turns; with many large ones, the other kernel's
+  // 32 warps per SM make up for their slower rounds (config 2's lengths and budgets, 10,000 jobs: 512 evaluations 66 against 149 ms,
+  // 1,024: 116 against 160, 2,048: 224 against 170, 8,192: 871 against 397).  The line is drawn for those: of smaller
+  // instances more CTAs fit an SM, and this kernel is still ahead at 8,192 evaluations (2,000 jobs: 80 against 103 ms, 500
+  // jobs: 16 against 36).
   const int spec_per_cta = n_spec && n_spec <= 8 * static_cast<int64_t>(ctx->sm_count) ? kvs_spec_per_cta(max_n) : 0;
   if (spec_per_cta > 0) {
     std::vector<int64_t> by_inst(after + n_refill, after + n_refill + n_spec);
