@@ -20,6 +20,7 @@
 // adding the phases up in 128-bit divisions 765 us; a lane per phase in the same kernel 348 us (102 registers left two
 // CTAs per SM to hide the chain); as two kernels 133 us for a histogram per evaluation and 36 us for the sums; with one
 // histogram per instance (k_class_counts) 56 us and 36 us.
+#include "kvs_events.cuh"
 #include "kvs_ladder.cuh"
 
 namespace {
@@ -33,23 +34,6 @@ struct Ladder {
   u32 tau[MAXP], k[MAXP];
   int n_phases;
 };
-
-// sum_{i=0}^{n-1} floor(i * a / m), exact in 128 bits (n, a, m below 2^31): the Euclid-like
-// recursion on (a mod m, m) with the quotient parts taken out in closed form.
-__device__ u128 floor_sum128(u64 n, u64 m, u64 a) {
-  u128 ans = 0;
-  u64 b = 0;
-  for (;;) {
-    u64 q, r;
-    if (a >= m) { divmod_u(a, m, &q, &r); ans += static_cast<u128>(n - 1) * n / 2 * q; a = r; }
-    if (b >= m) { divmod_u(b, m, &q, &r); ans += static_cast<u128>(n) * q; b = r; }
-    const u64 y = a * n + b;            // below 2^31 * 2^31 + 2^31
-    if (y < m) break;
-    divmod_u(y, m, &n, &b);
-    const u64 t = m; m = a; a = t;
-  }
-  return ans;
-}
 
 __device__ __forceinline__ u128 shfl_up128(u128 v, int d) {
   const u64 lo = __shfl_up_sync(0xffffffffu, static_cast<u64>(v), d), hi = __shfl_up_sync(0xffffffffu, static_cast<u64>(v >> 64), d);
@@ -151,12 +135,7 @@ __global__ void __launch_bounds__(BT, 3) k_class_counts(const i64* __restrict__ 
   u32 sum = 0;
 #pragma unroll 1
   for (int i = 0; i < BIN_PER; ++i) { sum += bin[tid * BIN_PER + i]; bin[tid * BIN_PER + i] = sum; }
-  u32 incl = sum;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const u32 y = __shfl_up_sync(0xffffffffu, incl, d);
-    if (lane >= d) incl += y;
-  }
+  const u32 incl = warp_incl(sum);
   if (lane == 31) wsum[warp] = incl;
   __syncthreads();
   u32 before = incl - sum;
@@ -236,7 +215,7 @@ __global__ void __launch_bounds__(BW * 32) k_bounds(const i64* __restrict__ job_
       divmod_u(n_gt * t + kk - 1, kk, &qd, &r);
       const u128 S = class_prefix + excl128(on ? static_cast<u128>(qc) + t : 0, &tot_c);
       const u128 Tp = phase_prefix + excl128(on ? static_cast<u128>(qg) + t : 0, &tot_g);
-      const u128 Q = static_cast<u128>(np) * t + (np ? floor_sum128(np, kk, t) : 0);
+      const u128 Q = static_cast<u128>(np) * t + (np ? floor_sum<u128>(np, kk, t, 0) : 0);
       const u64 x = p == 0 || !on ? 0 : sh.tau[p - 1];
       const u128 area2 = static_cast<u128>(2) * static_cast<u64>(c.s_bar) * x + static_cast<u128>(x) * (x + 1);
       const u128 a = on ? static_cast<u128>(np) * S + Q : 0, b = on ? static_cast<u128>(np) * (Tp + qd) + Q : 0;

@@ -20,15 +20,16 @@
 
 #ifdef __CUDACC__
 
-// sum_{j=0}^{n-1} floor((a*j + b) / m), arithmetic modulo 2^64; a, m, n below 2^31.  The operands shrink by steps of
-// the Euclidean algorithm, so after the first step or two the divisions are 32-bit ones.
-__device__ inline u64 floor_sum(u64 n, u64 m, u64 a, u64 b) {
-  u64 ans = 0;
+// sum_{j=0}^{n-1} floor((a*j + b) / m) modulo the width of V (64 bits, or 128: exact); a, b, m, n below 2^31, n >= 1 for 128 bits.
+// The operands shrink by steps of the Euclidean algorithm, so after the first step or two the divisions are 32-bit ones.
+template <class V = u64>
+__device__ inline V floor_sum(u64 n, u64 m, u64 a, u64 b) {
+  V ans = 0;
   for (;;) {
     u64 q, r;
-    if (a >= m) { divmod_u(a, m, &q, &r); ans += (n - 1) * n / 2 * q; a = r; }
-    if (b >= m) { divmod_u(b, m, &q, &r); ans += n * q; b = r; }
-    const u64 y = a * n + b;
+    if (a >= m) { divmod_u(a, m, &q, &r); ans += static_cast<V>(n - 1) * n / 2 * q; a = r; }
+    if (b >= m) { divmod_u(b, m, &q, &r); ans += static_cast<V>(n) * q; b = r; }
+    const u64 y = a * n + b;            // below 2^31 * 2^31 + 2^31
     if (y < m) break;
     divmod_u(y, m, &n, &b);
     const u64 t = m; m = a; a = t;

@@ -820,22 +820,12 @@ __device__ __forceinline__ void block_prefix(FShared& sh, u32* out, int out_cap,
     for (int j = 0; j < 4; ++j) in[j] = x + j < n ? f(x + j) : 0u;
 #pragma unroll
     for (int j = 0; j < 4; ++j) { v[j] = tot; tot += in[j]; }
-    u32 incl = tot;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const u32 y = __shfl_up_sync(0xffffffffu, incl, d);
-      if (lane >= d) incl += y;
-    }
+    const u32 incl = warp_incl(tot);
     __syncthreads();
     if (lane == 31) sh.redA[warp] = incl;
     __syncthreads();
     const u32 w = lane < WARPS ? sh.redA[lane] : 0u;
-    u32 wi = w;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const u32 y = __shfl_up_sync(0xffffffffu, wi, d);
-      if (lane >= d) wi += y;
-    }
+    const u32 wi = warp_incl(w);
     const u32 off = run + __shfl_sync(0xffffffffu, wi - w, warp) + (incl - tot);
     run += __shfl_sync(0xffffffffu, wi, 31);
 #pragma unroll
@@ -1696,12 +1686,7 @@ __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 
             for (int u = 0; u < MAXP / 32; ++u) {
               const int q = 32 * u + lane;
               cost[u] = q < L ? ((sh.plen[q] + TILE - 1) / TILE) * 2048 + (q < n_pure ? 0 : static_cast<i64>(sh.np[q])) : 0;
-              i64 v = cost[u];
-#pragma unroll
-              for (int d = 1; d < 32; d <<= 1) {
-                const i64 y = __shfl_up_sync(0xffffffffu, v, d);
-                if (lane >= d) v += y;
-              }
+              const i64 v = warp_incl(cost[u]);
               incl[u] = total + v;
               total += __shfl_sync(0xffffffffu, v, 31);
             }

@@ -282,6 +282,17 @@ __device__ __forceinline__ T warp_max(T v) {
   return v;
 }
 
+// inclusive sum over the lanes of a warp
+template <typename V>
+__device__ __forceinline__ V warp_incl(V v) {
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const V y = __shfl_up_sync(0xffffffffu, v, d);
+    if (static_cast<int>(lane_id()) >= d) v += y;
+  }
+  return v;
+}
+
 // Block-wide reductions; `scratch` has room for 32 values; result valid in every thread.
 template <typename T>
 __device__ __forceinline__ T block_sum(T v, T* scratch) {

@@ -17,17 +17,6 @@ constexpr int OWARPS = OT / 32;
 constexpr int ORD_TILES = 4;
 constexpr int ORD_CHUNK = OT * ORD_TILES;
 
-// inclusive sum over the lanes of a warp
-template <typename V>
-__device__ __forceinline__ V warp_incl(V v) {
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const V y = __shfl_up_sync(0xffffffffu, v, d);
-    if (static_cast<int>(lane_id()) >= d) v += y;
-  }
-  return v;
-}
-
 // s_max, o_max and input checks of the jobs [job_off[0], job_off[1]) into info->stats (zeroed by the caller),
 // and the range itself.
 __global__ void __launch_bounds__(256) k_order_info(const i64* job_off, const int32_t* s, const int32_t* o, i64 n_total, i64 max_jobs, OrderInfo* info) {
