@@ -445,10 +445,12 @@ int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* se
   int64_t full_of[4] = {0, 0, 0, 0}, light_of[4] = {0, 0, 0, 0};
   if (fast) {
     const bool all_full = one_wave && do_profile;
-    // (the batching algorithm on exact keys takes its peak from run ends as well where no profile is stored at all)
+    // (the batching algorithm on exact keys takes its peak from run ends as well where no profile is stored; its variants with
+    // a profile are the general kernel's, so the light variant sees them first)
     const bool gba_light = !inst->o_est && !v.profile;
     auto is_full = [&](int64_t e) {
-      return do_profile && (all_full || settings[e].family == KVS_GSA || (settings[e].family == KVS_GBA && !gba_light));
+      const kvs_setting& s = settings[e];
+      return do_profile && (all_full || s.family == KVS_GSA || (s.family == KVS_GBA && !gba_light && !(split && (s.subroutine || s.per_class_s))));
     };
     for (int64_t e = 0; e < P; ++e)
       if (is_full(e)) ids[n_full++] = e;

@@ -127,3 +127,31 @@ def test_sweep_over_the_only_instance_of_a_larger_array(par):
         a, b = (par.scheduler().sweep_beta0(inst, 0, fam, 4000, [0, 5, 64]) for inst in (part, own))
         for f in a:
             assert torch.equal(a[f], b[f]), (fam, f)
+
+
+@pytest.mark.parametrize("copies", [1, 4])      # shared evaluations, a call that is split by family
+def test_variants_with_and_without_profile_in_one_call(par, copies):
+    """Some evaluations of a call store their profile, others have capacity 0: variants and plain schedules side by side."""
+    inst = workloads.random_small(4400, 10, 60, 30, 90)
+    M = [int(inst.s[a:b].max() + inst.o[a:b].max()) + 40 if b > a else 40 for a, b in zip(inst.job_off[:-1].tolist(), inst.job_off[1:].tolist())]
+    rows = [dict(instance=i, family=f, M=m, subroutine=sub, per_class_s=pc) for i, m in enumerate(M) for f in ("GBA", "GSA") for sub, pc in ((0, 0), (1, 0), (0, 1))]
+    st = binding.make_settings(rows * copies)
+    P = st.shape[0]
+    assert P > 148 if copies > 1 else P <= 148
+    whole = par.scheduler().evaluate(inst.to("cuda:0"), st, want_profile=True)
+    wanted = torch.arange(P) % 3 != 1
+    cap = torch.where(wanted.to("cuda:0"), whole.horizon, 0)
+    some = par.scheduler().evaluate(inst.to("cuda:0"), st, want_profile=True, profile_capacity=cap)
+    for f in ("status", "flow", "peak", "horizon", "job_steps", "n_runs", "feasible", "job_start", "job_completion"):
+        assert torch.equal(getattr(whole, f), getattr(some, f)), f
+    for e in torch.nonzero(wanted).flatten().tolist():
+        a, b = whole.profile_off[e:e + 2].tolist()
+        c, d = some.profile_off[e:e + 2].tolist()
+        assert torch.equal(whole.profile[a:b], some.profile[c:d]), e
+    for e in range(0, P // copies, 7):
+        row = st[e]
+        a, b = inst.job_off[int(row["instance"]):int(row["instance"]) + 2].tolist()
+        S = oracle.build_schedule(int(row["family"]), inst.s[a:b], inst.o[a:b], int(row["M"]), subroutine=int(row["subroutine"]), per_class_s=int(row["per_class_s"]))
+        if S.status == 0:
+            E = oracle.evaluate_dense(S.run_start, S.run_len, S.run_s, want_profile=False)
+            assert (int(some.peak[e]), int(some.flow[e])) == (E.peak, S.flow), rows[e]
