@@ -256,6 +256,17 @@ def test_peak_without_profile_sizes(par, copies, n, o_max):
     par.check_batch(inst, binding.make_settings((rows * copies)[:max(len(rows), 2 * copies)]), want_runs=False, want_profile=False, label=f"peak n={n}")
 
 
+@pytest.mark.parametrize("n", [1 << 18, (1 << 18) + 1])       # the largest instance that CTAs share, the smallest that they do not
+@pytest.mark.parametrize("families", [("GBA",), ("GSA",), ("SPS",), ("SIMS",), ("GBA", "GSA", "SIMS")])
+def test_few_evaluations_of_large_instances(par, n, families):
+    """Calls of one family, which go to that family's kernel where they are not shared, and of several."""
+    inst = workloads.config4(n=n)
+    st = binding.settings_grid(range(1), families, [1 << 22])
+    st["tau"] = np.where(st["family"] >= binding.SPS, 512, 0)
+    for profile in (True, False):
+        par.check_batch(inst, st, want_runs=False, want_profile=profile, label=f"n={n} profile={int(profile)}")
+
+
 @pytest.mark.parametrize("est", [False, True])
 def test_host_entry_point_chunks(par, est):
     """Chunks of instances that take turns on the host entry point's pairs of streams: some with every family, some with one
