@@ -45,6 +45,21 @@ def test_sweep_small_full_grid(par, fam):
 
 
 @pytest.mark.parametrize("fam", ["SPS", "SIMS"])
+def test_sweep_on_any_instance_of_a_batch(par, fam):
+    """The instance is a stretch of a larger batch (sizes are bounded by the batch's, not read): as a batch of its own."""
+    sizes = [0, 1, 700, 3, 300]
+    off = torch.tensor([0, 0, 1, 701, 704, 1004])
+    c = torch.arange(1004)
+    inst = workloads.Instances(off, workloads.uniform_int(83, c, 0, 90), workloads.pareto_int(84, c, 20.0, 1.1, 1, 900))
+    for i, n in enumerate(sizes):
+        a = int(off[i])
+        own = workloads.Instances(torch.tensor([0, n]), inst.s[a:a + n].clone(), inst.o[a:a + n].clone())
+        got, want = (par.scheduler().sweep(x.to("cuda:0"), k, fam, 5000, [1, 20, 400], [1, 7, 512]) for x, k in ((inst, i), (own, 0)))
+        for f in want:
+            assert torch.equal(got[f], want[f]), (i, f)
+
+
+@pytest.mark.parametrize("fam", ["SPS", "SIMS"])
 def test_sweep_ragged_and_tiny(par, fam):
     for n in (1, 2, 63, 64, 65, 8191, 8193):
         inst = workloads.config1(n=n)
