@@ -347,7 +347,7 @@ def run_bounds(args, rank, world, dev, local):
     assert int((out["status"] != 0).sum()) == 0
     P = settings.shape[0]
     peak_gbs, peak_kind = load_peaks()
-    alg = 4.0 * n * P + 8.0 * n * I            # the response lengths once per evaluation; s and o once for the statistics
+    alg = 8.0 * n * I + 28.0 * P               # s and o once per instance, whatever its settings; three sums and a status per evaluation
     if rank == 0:
         print(json.dumps({"metric": "bound_evaluation_jobs_per_sec", "value": P * n / sec, "unit": "jobs/s", "n_gpus": world, "steps": args.steps,
                           "warmup": args.warmup, "ms_per_step": 1e3 * sec, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -355,7 +355,7 @@ def run_bounds(args, rank, world, dev, local):
                           "config": {"workload": WORKLOADS[name][4], "instances_per_gpu": I, "jobs_per_instance": n, "evaluations_per_gpu": P},
                           "evaluations_per_sec": P / sec,
                           "roofline": {"bound": "hbm", "achieved": alg / sec / 1e9, "peak": peak_gbs, "unit": "GB/s", "frac": alg / sec / 1e9 / peak_gbs,
-                                       "traffic": None, "peak_kind": peak_kind, "kernel": "k_bounds (+ statistics pass)", "algorithmic_bytes": alg},
+                                       "traffic": None, "peak_kind": peak_kind, "kernel": "k_class_counts + k_bounds", "algorithmic_bytes": alg},
                           "gpu_launches": 2 * args.steps}))
 
 
@@ -562,7 +562,7 @@ def run_fused_workload(args, rank, world, dev, local, dist, binding, Scheduler):
         post = "k_refill" if "GBAD" in fams else "k_spec"
         line["roofline"]["kernel"] = "k_fused_eval<full> + " + post + " (timed together)"
         line["roofline"]["note"] = (post + " applies a sequential rule per evaluation, one warp each: it is bound by the latency of "
-                                    "dependent loads, and the HBM fraction is given for completeness only")
+                                    "dependent steps, and the HBM fraction is given for completeness only")
     if e2e:
         line["e2e"] = {"value": steps_all / (e2e_s / args.steps), "unit": UNIT, "h2d_bytes_per_step": e2e[1], "d2h_bytes_per_step": e2e[2],
                        "result": "scalars only (no per-job results and no profile leave the device on this path)"}
