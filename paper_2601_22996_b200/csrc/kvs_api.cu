@@ -131,8 +131,8 @@ int parts_for(int64_t P, int64_t max_n) {
   return static_cast<int>(g < 1 ? 1 : (g > KVS_MAX_PARTS ? KVS_MAX_PARTS : g));
 }
 size_t lists_bytes(int64_t P) { return CALL_COUNTERS + static_cast<size_t>(P) * (sizeof(kvs_setting) + 3 * 8); }
-size_t pairs_at(int64_t P) { return lists_bytes(P) + static_cast<size_t>(P) * sizeof(FusedShare); }
-size_t call_bytes(int64_t P) { return pairs_at(P) + static_cast<size_t>(P) * 16; }   // pairs of evaluations of the speculative runs
+size_t groups_at(int64_t P) { return lists_bytes(P) + static_cast<size_t>(P) * sizeof(FusedShare); }
+size_t call_bytes(int64_t P) { return groups_at(P) + static_cast<size_t>(P) * 8 * KVS_SPEC_GROUP; }   // groups of evaluations of the speculative runs
 
 Layout make_layout(int64_t N, int64_t I, int64_t max_n, int64_t P, bool staging) {
   Layout L{};
@@ -368,26 +368,28 @@ int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* se
   auto by_budget = [&](int64_t x, int64_t y) { return st_host[x].M < st_host[y].M; };
   std::stable_sort(after, after + n_refill, by_budget);
   std::stable_sort(after + n_refill, after + n_refill + n_spec, by_budget);
-  // The on-chip kernel of the speculative runs takes two evaluations of one instance per CTA where they fit.
-  int64_t* const pairs = reinterpret_cast<int64_t*>(stg->p + pairs_at(P));
-  int64_t n_pairs = 0;
-  // That kernel ends first where it has every evaluation in flight within a few turns; with many large ones, the other kernel's
-  // 32 warps per SM make up for their slower rounds (config 2's lengths and budgets, 10,000 jobs: 512 evaluations 66 against 149 ms,
-  // 1,024: 116 against 160, 2,048: 224 against 170, 8,192: 871 against 397).  The line is drawn for those: of smaller
-  // instances more CTAs fit an SM, and this kernel is still ahead at 8,192 evaluations (2,000 jobs: 80 against 103 ms, 500
-  // jobs: 16 against 36).
-  const int spec_per_cta = n_spec && n_spec <= 8 * static_cast<int64_t>(ctx->sm_count) ? kvs_spec_per_cta(max_n) : 0;
+  // The on-chip kernel of the speculative runs takes up to four evaluations of one instance per CTA.
+  int64_t* const groups = reinterpret_cast<int64_t*>(stg->p + groups_at(P));
+  int64_t n_groups = 0;
+  // An SM holds at least two of its evaluations, or few have to take turns: else the 32 warps per SM of the other kernel make up for
+  // their slower rounds.  Config 2's lengths and budgets, 8,192 evaluations of 500 / 2,000 / 5,000 / 10,000 jobs: 16 / 36 / 100 / 174 ms
+  // on chip, 34 / 96 / 195 / 346 in memory; 16,000 jobs (two per SM), 512 / 4,096 evaluations: 34 / 211 against 189 / 338; 24,000 jobs
+  // (one per SM), 512 / 2,048 / 3,072 / 4,096 evaluations: 79 / 273 / 400 / 532 against 254 / 338 / 457 / 511.
+  int spec_per_cta = n_spec ? kvs_spec_per_cta(max_n) : 0;
+  if (spec_per_cta == 1 && n_spec > 24 * static_cast<int64_t>(ctx->sm_count)) spec_per_cta = 0;
   if (spec_per_cta > 0) {
     std::vector<int64_t> by_inst(after + n_refill, after + n_refill + n_spec);
     std::stable_sort(by_inst.begin(), by_inst.end(), [&](int64_t x, int64_t y) { return st_host[x].instance < st_host[y].instance; });
-    std::vector<std::pair<int64_t, int64_t>> two;
-    for (size_t i = 0; i < by_inst.size(); ++i) {
-      const bool both = spec_per_cta == 2 && i + 1 < by_inst.size() && st_host[by_inst[i]].instance == st_host[by_inst[i + 1]].instance;
-      two.emplace_back(by_inst[i], both ? by_inst[i + 1] : -1);
-      if (both) ++i;
+    std::vector<std::pair<size_t, size_t>> cut;           // [first, last) of by_inst, smallest budget first
+    for (size_t i = 0, j; i < by_inst.size(); i = j) {
+      for (j = i + 1; j < by_inst.size() && j - i < static_cast<size_t>(spec_per_cta) && st_host[by_inst[i]].instance == st_host[by_inst[j]].instance; ++j) {}
+      cut.emplace_back(i, j);
     }
-    std::stable_sort(two.begin(), two.end(), [&](const auto& x, const auto& y) { return st_host[x.first].M < st_host[y.first].M; });
-    for (const auto& x : two) { pairs[2 * n_pairs] = x.first; pairs[2 * n_pairs + 1] = x.second; ++n_pairs; }
+    std::stable_sort(cut.begin(), cut.end(), [&](const auto& x, const auto& y) { return st_host[by_inst[x.first]].M < st_host[by_inst[y.first]].M; });
+    for (const auto& x : cut) {
+      int64_t* const g = groups + KVS_SPEC_GROUP * n_groups++;
+      for (size_t i = 0; i < KVS_SPEC_GROUP; ++i) g[i] = x.first + i < x.second ? by_inst[x.first + i] : -1;
+    }
   }
   if (n_refill || n_spec) {
     if (do_profile && (!o.job_start || !o.job_completion || !v.profile || o.job_start64 || o.job_completion64 || run_out))
@@ -485,7 +487,7 @@ int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* se
       init[17 + 2 * f] = static_cast<unsigned long long>(full_of[f]);
     }
   }
-  const size_t upload = n_pairs ? call_bytes(P) : (parts > 1 ? pairs_at(P) : lists_bytes(P));
+  const size_t upload = n_groups ? call_bytes(P) : (parts > 1 ? groups_at(P) : lists_bytes(P));
   ce = send_stage(stg, counters, upload, rg ? ctx->copy_stream : ctx->stream);
   if (ce != cudaSuccess) return fail_cuda(ctx, ce, "copy of the settings and evaluation lists");
   if (rg && (rc = rg->feed())) return rc;
@@ -637,7 +639,8 @@ int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* se
     const i64 want = static_cast<i64>(ctx->sm_count) * 32;
     q.n_warps = std::min<i64>(std::min<i64>(room, want), q.n_list);
     q.counter = counters + 24;
-    q.pairs = reinterpret_cast<const i64*>(call + pairs_at(P)); q.n_pairs = n_pairs;
+    // (its lists of participants take less of the working storage than the CTA scratch of as many evaluations; otherwise the other kernel takes them all)
+    q.groups = reinterpret_cast<const i64*>(call + groups_at(P)); q.n_groups = n_groups * kvs_spec_group_bytes(max_n) <= q.scratch_bytes ? n_groups : 0;
     q.left_list = reinterpret_cast<i64*>(ws + L.slow_list); q.left_count = counters + 26;   // the general kernel has run: its list is free
     ce = kvs_launch_spec(q, ctx->stream);
     if (ce != cudaSuccess) return fail_cuda(ctx, ce, "launch of the speculative runs");

@@ -433,29 +433,51 @@ __global__ void __launch_bounds__(ST) k_spec(SpecParams p) {
 
 // ---- the same simulation with its state in shared memory --------------------------------------------
 //
-// What bounds a simulation is the chain of reads from its own state, round after round: with the state in global
-// memory an evaluation of 7,500 jobs takes 130 to 200 million cycles, however few there are.  Instances of at most
-// some 17,000 jobs (lengths below 2^16) fit on chip: per evaluation 8 bytes a job - list position -> job, start of the speculative
-// run, stack entry - and a bit for `done`, next to 4 bytes a job of prompt and response lengths, which the warps of
-// a CTA share (up to two evaluations of one instance).  Besides:
-//   - runs dropped from the plan are not subtracted from the profile round by round: those in progress hold
-//     Ad + t * Cd tokens, with their ends in a ring of DROP_RING rounds (longer ones are subtracted in memory);
-//   - the rounds up to the next event are written 32 at a time: nothing can happen in a round in which nothing starts or ends, the
+// What bounds a simulation is the chain of steps of its one warp, so what counts is the number of rounds at which the warp has to
+// stop, the dependent instructions of each stop, and the evaluations that an SM has in flight.  Instances of at most some 25,000
+// jobs (lengths below 2^16) fit on chip: 4 bytes a job of prompt and response lengths, which the warps of a CTA share (up to four
+// evaluations of one instance), and per evaluation 4 bytes a job - start of the speculative run, stack entry - and two bits.  Besides:
+//   - a job that is free to start a speculative run has its bit set in a map by job index: the order of the participants is that
+//     of the indices and whoever is no participant any more is done, so the lowest free job is the first bit, found by one
+//     16-byte load a lane over 4,096 jobs; slot ends and kills set a bit and know at once whether it is the lowest;
+//   - the rounds are taken 32 at a time.  Where a window's pipeline runs are few, all of them are looked at when it begins: those
+//     of jobs that have completed are dropped there and then, together, and neither their starts nor their slot ends stop the warp;
+//   - a run dropped from the plan is not subtracted from the profile round by round: those in progress hold Ad + t * Cd tokens, with
+//     starts and ends in a ring of 256 to 1,024 rounds, ends beyond it in a list of FAR_SETS entries a lane (beyond that in memory);
+//   - the participants' list lies in memory: it is read in order, the next 32 entries ahead of time;
+//   - the rounds up to the next event are written together: nothing can happen in a round in which nothing starts or ends, the
 //     memory stays within M and the first free job does not fit;
 //   - the stack keeps the earliest completion of every 64 entries, so that a completion looks at few entries;
 //   - sums that nothing in the simulation depends on are kept per lane.
-// Rounds are kept modulo 65,535 where 16 bits hold them: a speculative run lasts less than that.
+// Starts are kept modulo 65,535: a speculative run lasts less than that.
+// 512 evaluations (64 instances of 5,000 to 10,000 jobs, eight budgets), four per SM and all in flight: 17.6 ms, the chain of the longest
+// one.  With every run's start and slot end a stop, list scans of 32 positions for the lowest free job and two evaluations per SM: 56.7 ms.
 
-constexpr int DROP_RING = 1024;
+constexpr int SPEC_WARPS = 4;            // evaluations of one CTA
+constexpr int RING_MAX = 1024, RING_MIN = 256;
+constexpr int FAR_SETS = 6;
 constexpr u32 IDLE = 0xffffu;            // sst: not running speculatively
 constexpr u32 MODT = 65535u;
 constexpr int STK_BLK = 64;
+constexpr int LOOK_AHEAD = 1024;         // runs that may start in a window whose runs are looked at together: a mask of 32 per lane
 
-// Bytes of one warp's state for instances of at most n jobs, and of the lengths that a CTA's warps share.
-__host__ __device__ inline int smem_jobs(int n) { return (n + 63) & ~63; }
-__host__ __device__ inline int smem_state_bytes(int n) {
+// The phase table of one warp; the powers of the ladder lie where the stack will be.
+struct alignas(16) SpecTable {
+  u32 tau[MAXP], k[MAXP], np[MAXP], hist[MAXP];
+  int pbase[MAXP + 1];
+  int n_phases;
+  u128 *pw_a, *pw_b;
+};
+
+// Bytes of one warp's state for instances of at most n jobs with a ring of that many rounds, and of the lengths that a CTA's warps share.
+__host__ __device__ inline int smem_jobs(int n) { return (n + 127) & ~127; }
+__host__ __device__ inline int smem_stack_bytes(int m) {
+  const int powers = 2 * (MAXP + 1) * static_cast<int>(sizeof(u128));
+  return 2 * m > powers ? 2 * m : powers;
+}
+__host__ __device__ inline int smem_state_bytes(int n, int ring) {
   const int m = smem_jobs(n);
-  return static_cast<int>(sizeof(SpecShared)) + m * 8 + DROP_RING * 8 + m / STK_BLK * 4 + m / 8 + 12 & ~15;
+  return static_cast<int>(sizeof(SpecTable)) + ring * 8 + smem_stack_bytes(m) + 2 * m + 2 * (m / 8) + ((m / STK_BLK * 4 + 15) & ~15);
 }
 __host__ __device__ inline int smem_lengths_bytes(int n) { return smem_jobs(n) * 4; }
 
@@ -472,8 +494,7 @@ struct SpecPhase {
   u64 tau_inv, k_inv;
   int np;
   int base;
-  int qt, rt;               // tau = qt * k + rt: starts of consecutive ranks differ by qt or qt + 1
-  bool single;              // tau >= k: no two ranks start in one round
+  bool ahead;               // fewer than LOOK_AHEAD runs start in a window
   __device__ __forceinline__ int start_of(int r) const { return base + static_cast<int>(div_by(static_cast<u64>(static_cast<u32>(r)) * tau, k, k_inv)); }
   // ranks that start x rounds after the phase's first round or earlier
   __device__ __forceinline__ int started(int x) const {
@@ -485,38 +506,42 @@ struct SpecPhase {
   }
 };
 
-__global__ void __launch_bounds__(64) k_spec_smem(SpecParams p, int n_cap) {
+__global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int n_cap, int ring_rounds) {
   extern __shared__ __align__(16) unsigned char raw[];
   const int lane = lane_id(), warp = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
   const int m = smem_jobs(n_cap);
-  unsigned short* const Ssh = reinterpret_cast<unsigned short*>(raw);
-  unsigned short* const Osh = Ssh + m;
-  unsigned char* at = raw + smem_lengths_bytes(n_cap) + warp * smem_state_bytes(n_cap);
-  SpecShared& sh = *reinterpret_cast<SpecShared*>(at); at += sizeof(SpecShared);
-  u32* const stk = reinterpret_cast<u32*>(at); at += m * 4;             // job << 16 | start modulo MODT
-  u32* const ring_a = reinterpret_cast<u32*>(at); at += DROP_RING * 4;
-  u32* const ring_c = reinterpret_cast<u32*>(at); at += DROP_RING * 4;
-  u32* const first_fin = reinterpret_cast<u32*>(at); at += m / STK_BLK * 4;   // no run of the block's entries completes before this round
+  u32* const lengths = reinterpret_cast<u32*>(raw);     // response length << 16 | prompt length
+  unsigned char* at = raw + smem_lengths_bytes(n_cap) + warp * smem_state_bytes(n_cap, ring_rounds);
+  SpecTable& sh = *reinterpret_cast<SpecTable*>(at); at += sizeof(SpecTable);
+  u32* const ring_a = reinterpret_cast<u32*>(at); at += ring_rounds * 4;
+  u32* const ring_c = reinterpret_cast<u32*>(at); at += ring_rounds * 4;
+  const int ring_mask = ring_rounds - 1;
+  unsigned char* const stk_at = at; at += smem_stack_bytes(m);
+  unsigned short* const stk = reinterpret_cast<unsigned short*>(stk_at);  // jobs in order of their starts; an entry whose job is not running is stale, and so is one with another above it
+  u32* const free_map = reinterpret_cast<u32*>(at); at += m / 8;          // neither done nor running
   u32* const done = reinterpret_cast<u32*>(at); at += m / 8;
-  unsigned short* const list = reinterpret_cast<unsigned short*>(at); at += m * 2;
-  unsigned short* const sst = reinterpret_cast<unsigned short*>(at);
-  const i64 mine = p.pairs[2 * static_cast<i64>(blockIdx.x) + warp];       // -1: no evaluation for the second warp
-  const i64 inst = p.settings[p.pairs[2 * static_cast<i64>(blockIdx.x)]].instance;
+  unsigned short* const sst = reinterpret_cast<unsigned short*>(at); at += m * 2;
+  u32* const first_fin = reinterpret_cast<u32*>(at);                     // no run of the block's entries completes before this round
+  const i64* const group = p.groups + SPEC_WARPS * static_cast<i64>(blockIdx.x);
+  const i64 mine = group[warp];                         // -1: no evaluation for this warp
+  const i64 inst = p.settings[group[0]].instance;
   const i64 lo = p.job_off[inst];
   const InstStats stats = p.stats[inst];
   // the memory of a round, pipeline and speculative runs before any is killed, stays below 2^32
-  // (the two warps decide together: both of them load the lengths)
-  const i64 second = blockDim.x > 32 ? p.pairs[2 * static_cast<i64>(blockIdx.x) + 1] : -1;
-  const i64 M_pair = max_i64(p.settings[p.pairs[2 * static_cast<i64>(blockIdx.x)]].M, second >= 0 ? p.settings[second].M : 0);
+  // (the warps decide together: all of them load the lengths)
+  i64 M_most = 0;
+  for (int v = 0; v < static_cast<int>(blockDim.x >> 5); ++v)
+    if (group[v] >= 0) M_most = max_i64(M_most, p.settings[group[v]].M);
   const int n = stats.flags ? 0 : static_cast<int>(p.job_off[inst + 1] - lo);
-  if (n > n_cap || stats.o_max >= static_cast<int>(MODT) || stats.s_max >= 65536 || M_pair >= (1ll << 30)) {
+  if (n > n_cap || stats.o_max >= static_cast<int>(MODT) || stats.s_max >= 65536 || M_most >= (1ll << 30)) {
     if (lane == 0 && mine >= 0) p.left_list[atomicAdd(p.left_count, 1ull)] = mine;
     return;
   }
+  unsigned short* const list = reinterpret_cast<unsigned short*>(p.scratch) + (SPEC_WARPS * static_cast<i64>(blockIdx.x) + warp) * m;   // kvs_spec_group_bytes a CTA
+  if (!KVS_OK_AT((SPEC_WARPS * static_cast<i64>(blockIdx.x) + warp + 1) * m * 2 - 1, p.scratch_bytes, CHK_SP_SCRATCH)) return;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    Ssh[i] = static_cast<unsigned short>(p.s[lo + i]);
-    Osh[i] = static_cast<unsigned short>(p.o[lo + i]);
+    lengths[i] = static_cast<u32>(p.o[lo + i]) << 16 | static_cast<u32>(p.s[lo + i]);
   }
   __syncthreads();
   if (mine < 0 || n == 0) return;
@@ -533,17 +558,23 @@ __global__ void __launch_bounds__(64) k_spec_smem(SpecParams p, int n_cap) {
   if (!KVS_OK_AT(H, p.profile_off[e + 1] - p.profile_off[e] + 1, CHK_SP_PROF)) return;
 
   // ---- phase table: ladder, classes, participants, first round of every phase ----
+  if (lane == 0) { sh.pw_a = reinterpret_cast<u128*>(stk_at); sh.pw_b = sh.pw_a + MAXP + 1; }
+  __syncwarp();
   ladder32(sh, X, set.alpha_num, set.alpha_den, set.beta0, static_cast<u32>(s_bar), static_cast<u32>(M));
   const int L = sh.n_phases;
   for (int q = lane; q < L; q += 32) sh.hist[q] = 0;
-  for (int i = lane; i < DROP_RING; i += 32) { ring_a[i] = 0; ring_c[i] = 0; }
-  for (int i = lane; i < m / 32; i += 32) done[i] = 0;
+  for (int i = lane; i < ring_rounds; i += 32) { ring_a[i] = 0; ring_c[i] = 0; }
+  for (int i = lane; i < m / 32; i += 32) {
+    const int room = n - 32 * i;
+    done[i] = 0;
+    if (i < m / STK_BLK) first_fin[i] = NO_ROUND;
+    free_map[i] = room >= 32 ? 0xffffffffu : (room > 0 ? (1u << room) - 1u : 0u);
+  }
   __syncwarp();
   const bool pow2 = set.alpha_num == 2 && set.alpha_den == 1 && set.beta0 <= 0;
   for (int i = lane; i < n; i += 32) {
-    const u32 oi = Osh[i];
+    const u32 oi = lengths[i] >> 16;
     atomicAdd(&sh.hist[pow2 ? class_pow2(static_cast<u32>(X), oi) : class_of(sh.tau, L, oi)], 1u);
-    list[i] = static_cast<unsigned short>(i);
     sst[i] = static_cast<unsigned short>(IDLE);
   }
   __syncwarp();
@@ -552,11 +583,11 @@ __global__ void __launch_bounds__(64) k_spec_smem(SpecParams p, int n_cap) {
     i64 b = 0;
     for (int q = 0; q < L; ++q) {
       sh.np[q] = later;                                 // jobs of class q or later take part in phase q
-      sh.pbase[q] = b;
+      sh.pbase[q] = static_cast<int>(b);
       if (later > 0) b += slot_of(static_cast<int>(later) - 1, sh.tau[q], sh.k[q]) + sh.tau[q];
       later -= sh.hist[q];
     }
-    sh.pbase[L] = b;
+    sh.pbase[L] = static_cast<int>(b);
   }
   __syncwarp();
   const u32 Mu = static_cast<u32>(M);
@@ -569,81 +600,260 @@ __global__ void __launch_bounds__(64) k_spec_smem(SpecParams p, int n_cap) {
     ph.tau = sh.tau[q]; ph.k = sh.k[q];
     ph.tau_inv = inverse_of(ph.tau); ph.k_inv = inverse_of(ph.k);
     ph.np = participants;
-    ph.base = static_cast<int>(sh.pbase[q]);
-    ph.qt = static_cast<int>(ph.tau / ph.k);
-    ph.rt = static_cast<int>(ph.tau % ph.k);
-    ph.single = ph.tau >= ph.k;
+    ph.base = sh.pbase[q];
+    // 32 rounds hold at most ceil(32 k / tau) + 1 starts, and as many slot ends
+    ph.ahead = static_cast<u64>(ph.k) * 32u <= static_cast<u64>(ph.tau) * (LOOK_AHEAD - 2);
   };
   enter(0, n);
-  int rs = 0, re = 0;                                   // ranks of the next run start and of the next slot end
-  int ns = 0, ne = static_cast<int>(ph.tau);            // their rounds
-  int s_rem = 0, e_rem = 0;                             // and remainders: rank * tau mod k
-  int phase_at = L > 1 && sh.np[1] > 0 ? static_cast<int>(sh.pbase[1]) : NEVER;   // first round of the next phase
+  int rs = 0, re = 0;                                   // ranks behind the runs (and the slot ends) that have been looked at
+  int ns = 0, ne = static_cast<int>(ph.tau);            // rounds of the next run start and of the next slot end
+  // The runs of 32 consecutive ranks that start next, one a lane: job, response, prompt + 1, first round, and which of them the warp
+  // still has to stop for; the same for the slot ends.  Where the window has been looked at, lane c holds the mask of its c-th 32.
+  u32 start_job = 0, start_o = 0, start_s1 = 0, end_job = 0;
+  int start_at = 0, end_at = 0, start_first = 0, end_first = 0;
+  unsigned start_mask = 0, end_mask = 0, start_masks = 0, end_masks = 0;
+  bool all_take_part = true;                            // rank = job index: no list yet
+  u32 ahead_start = 0, ahead_end = 0;                   // list entries of ranks rs + lane and re + lane, read ahead
+  // job of rank r < np
+  auto job_of = [&](int r) { return all_take_part ? static_cast<u32>(r) : static_cast<u32>(list[r]); };
+  int phase_at = L > 1 && sh.np[1] > 0 ? sh.pbase[1] : NEVER;   // first round of the next phase
   u32 A = 0;                                            // speculative runs hold A + t * cnt tokens in round t (modulo 2^32)
   int cnt = 0, top = 0;                                 // running speculative runs; entries on the stack (some stale)
-  u32 Ad = 0, Cd = 0;                                   // dropped runs in progress beyond the current window
+  u32 Ad = 0, Cd = 0;                                   // dropped runs in progress at the end of the current window
+  u32 far_v[FAR_SETS], far_c[FAR_SETS];                 // those of them that end beyond the ring (end 0: none)
+  int far_end[FAR_SETS];
+#pragma unroll
+  for (int f = 0; f < FAR_SETS; ++f) far_v[f] = far_c[f] = static_cast<u32>(far_end[f] = 0);
+  int far_next = NEVER;                                 // the earliest of them
   u32 next_comp = NO_ROUND;                             // no speculative run completes before this round
-  int fpos = 0, fhi = n;
-  int cj = -1, cs = 0;                                  // the free job at fpos and its prompt length, while known (cj = -2: none is free)
+  int fj = 0;                                           // no job below is free
+  int cj = -1, cs = 0;                                  // the lowest free job and its prompt length, while known (then fj = cj; -2: none is free)
   int left = n;
   i64 flow = 0, steps = 0;                              // flow, steps, runs, hmax, peak: per lane
   u32 runs = 0, peak = 0;
   int hmax = 0;
-  int Bw = 0;                                           // lane l holds the plan's memory of round (t & ~31) + l
+  int Bw = 0;                                           // lane l holds the plan's memory of round (t & ~31) + l,
+  int Bn = lane < H ? __ldcg(prof + lane) : 0;          // that of the window after it (past the first-level cache: atomics wrote it)
   u32 tm = 0;                                           // t modulo MODT
-  // The plan's 32 rounds from w on, less the dropped runs in progress; their ends in these rounds leave the ring.
-  auto load_window = [&](int w) {
+
+  // The next 32 of the window's runs with one that the warp stops for.
+  auto next_starts = [&]() {
+    const unsigned chunks = __ballot_sync(0xffffffffu, start_masks != 0);
+    if (!chunks) { ns = NEVER; return; }
+    const int c = __ffs(static_cast<int>(chunks)) - 1, r = start_first + 32 * c + lane;
+    start_mask = __shfl_sync(0xffffffffu, start_masks, c);
+    start_job = job_of(min(r, rs - 1));
+    const u32 so = lengths[start_job];
+    start_o = so >> 16; start_s1 = (so & 0xffffu) + 1u;
+    start_at = ph.start_of(r);
+    if (lane == c) start_masks = 0;
+    ns = __shfl_sync(0xffffffffu, start_at, __ffs(static_cast<int>(start_mask)) - 1);
+  };
+  auto next_ends = [&]() {
+    const unsigned chunks = __ballot_sync(0xffffffffu, end_masks != 0);
+    if (!chunks) { ne = NEVER; return; }
+    const int c = __ffs(static_cast<int>(chunks)) - 1, r = end_first + 32 * c + lane;
+    end_mask = __shfl_sync(0xffffffffu, end_masks, c);
+    end_job = job_of(min(r, re - 1));
+    end_at = ph.start_of(r) + static_cast<int>(ph.tau);
+    if (lane == c) end_masks = 0;
+    ne = __shfl_sync(0xffffffffu, end_at, __ffs(static_cast<int>(end_mask)) - 1);
+  };
+  // c dropped runs that last beyond the ring, with v = sum of s + 1 - start, that are in progress at the end of window w: into the
+  // list, false if it is full.
+  auto keep_far = [&](u32 v, u32 c, int end) {
+#pragma unroll
+    for (int f = 0; f < FAR_SETS; ++f) {
+      const unsigned room = __ballot_sync(0xffffffffu, far_end[f] == 0);
+      if (room) {
+        if (lane == __ffs(static_cast<int>(room)) - 1) { far_v[f] = v; far_c[f] = c; far_end[f] = end; }
+        far_next = min(far_next, end);
+        return true;
+      }
+    }
+    return false;
+  };
+  // Then they are taken out of the window after w, which is in registers, and of the rounds behind it.
+  auto drop_in_memory = [&](int w, u32 v, u32 c, int end) {
+    const int u = w + 32 + lane;
+    if (u < end) Bn -= static_cast<int>(v + c * static_cast<u32>(u));
+    for (int x = u + 32; x < end; x += 32)              // always the rounds of one lane: its later read follows
+      if (KVS_OK_AT(x, H, CHK_SP_DROP)) atomicSub(&prof[x], static_cast<int>(v + c * static_cast<u32>(x)));
+  };
+  // Runs dropped in round t of window w.
+  auto drop_now = [&](int w, int t, u32 v, u32 c, int end) {
     const int u = w + lane;
-    Bw = u < H ? __ldcg(prof + u) : 0;                  // past the first-level cache: other lanes' atomics wrote it
-    u32 ea = ring_a[u & (DROP_RING - 1)], ec = ring_c[u & (DROP_RING - 1)];
-    if (__any_sync(0xffffffffu, ec != 0)) {
-      ring_a[u & (DROP_RING - 1)] = 0;
-      ring_c[u & (DROP_RING - 1)] = 0;
+    if (u >= t && u < end) Bw -= static_cast<int>(v + c * static_cast<u32>(u));
+    if (end <= w + 32) return;
+    if (end < w + ring_rounds) {
+      Ad += v; Cd += c;
+      if (lane == 0) { ring_a[end & ring_mask] += v; ring_c[end & ring_mask] += c; }
+      __syncwarp();
+    } else if (keep_far(v, c, end)) {
+      Ad += v; Cd += c;
+    } else {
+      drop_in_memory(w, v, c, end);
+    }
+  };
+  // Looks at the runs that start and the slots that end from round t to the end of its window w: drops the runs of jobs that are
+  // done.  read: the first 32 list entries of each have been read ahead.
+  auto look_ahead = [&](int w, int t, bool read) {
+    const int r_hi = ph.started(w + 31 - ph.base);
+    start_first = rs; start_masks = 0; start_mask = 0; ns = NEVER;
+    for (int c = 0, r0 = rs; r0 < r_hi; ++c, r0 += 32) {
+      const int r = r0 + lane;
+      const bool on = r < r_hi;
+      const u32 j = !on ? 0u : (all_take_part ? static_cast<u32>(r) : (read && c == 0 ? ahead_start : static_cast<u32>(list[r])));
+      const u32 so = lengths[j], o = so >> 16, s1 = (so & 0xffffu) + 1u;
+      const bool drop = on && is_done(j);
+      const int q = ph.start_of(r);
+      const unsigned live = __ballot_sync(0xffffffffu, on && !drop);
+      if (live && ns == NEVER) {
+        start_mask = live;
+        start_job = j; start_o = o; start_s1 = s1; start_at = q;
+        ns = __shfl_sync(0xffffffffu, q, __ffs(static_cast<int>(live)) - 1);
+      } else if (lane == c) {
+        start_masks = live;
+      }
+      if (live == 0xffffffffu) continue;
+      const int end = q + static_cast<int>(min(o, ph.tau));
+      const u32 v = s1 - static_cast<u32>(q);
+      const bool far = end >= w + ring_rounds;
+      if (drop && !far) {
+        atomicSub(&ring_a[q & ring_mask], v); atomicSub(&ring_c[q & ring_mask], 1u);
+        atomicAdd(&ring_a[end & ring_mask], v); atomicAdd(&ring_c[end & ring_mask], 1u);
+      }
+      unsigned fm = __ballot_sync(0xffffffffu, drop && far);
+      while (fm) {
+        const int src = __ffs(static_cast<int>(fm)) - 1;
+        fm &= fm - 1u;
+        const u32 vs = __shfl_sync(0xffffffffu, v, src);
+        const int qs = __shfl_sync(0xffffffffu, q, src), es = __shfl_sync(0xffffffffu, end, src);
+        if (keep_far(vs, 1u, es)) {
+          if (lane == 0) { ring_a[qs & ring_mask] -= vs; ring_c[qs & ring_mask] -= 1u; }
+        } else {
+          if (w + lane >= qs) Bw -= static_cast<int>(vs + static_cast<u32>(w + lane));
+          drop_in_memory(w, vs, 1u, es);
+        }
+        __syncwarp();
+      }
+    }
+    rs = r_hi;
+    const int e_hi = ph.started(w + 31 - static_cast<int>(ph.tau) - ph.base);
+    end_first = re; end_masks = 0; end_mask = 0; ne = NEVER;
+    for (int c = 0, r0 = re; r0 < e_hi; ++c, r0 += 32) {
+      const int r = r0 + lane;
+      const bool on = r < e_hi;
+      const u32 j = !on ? 0u : (all_take_part ? static_cast<u32>(r) : (read && c == 0 ? ahead_end : static_cast<u32>(list[r])));
+      const unsigned live = __ballot_sync(0xffffffffu, on && !is_done(j));
+      if (live && ne == NEVER) {
+        end_mask = live;
+        end_job = j;
+        end_at = ph.start_of(r) + static_cast<int>(ph.tau);
+        ne = __shfl_sync(0xffffffffu, end_at, __ffs(static_cast<int>(live)) - 1);
+      } else if (lane == c) {
+        end_masks = live;
+      }
+    }
+    re = e_hi;
+    if (!all_take_part) {
+      if (rs + lane < ph.np) ahead_start = list[rs + lane];
+      if (re + lane < ph.np) ahead_end = list[re + lane];
+    }
+    __syncwarp();
+  };
+  // Takes the starts and ends of dropped runs in window w out of the ring; a, c: dropped runs in progress at its beginning.
+  auto apply_ring = [&](int w, u32 a, u32 c) {
+    const int u = w + lane, x = u & ring_mask;
+    u32 ea = ring_a[x], ec = ring_c[x];
+    if (__any_sync(0xffffffffu, (ea | ec) != 0)) {
+      ring_a[x] = 0;
+      ring_c[x] = 0;
 #pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
         const u32 ya = __shfl_up_sync(0xffffffffu, ea, d), yc = __shfl_up_sync(0xffffffffu, ec, d);
         if (lane >= d) { ea += ya; ec += yc; }
       }
+      Ad -= __shfl_sync(0xffffffffu, ea, 31);
+      Cd -= __shfl_sync(0xffffffffu, ec, 31);
     }
-    Bw -= static_cast<int>((Ad - ea) + static_cast<u32>(u) * (Cd - ec));
-    Ad -= __shfl_sync(0xffffffffu, ea, 31);
-    Cd -= __shfl_sync(0xffffffffu, ec, 31);
+    Bw -= static_cast<int>((a - ea) + static_cast<u32>(u) * (c - ec));
     __syncwarp();
   };
   auto running_for = [&](u32 start_m) { return tm >= start_m ? tm - start_m : tm + MODT - start_m; };   // rounds since a start
-  // Keeps the live entries of the stack, in order.
-  auto purge = [&]() {
+  auto prompt = [&](int j) { return static_cast<int>(lengths[j] & 0xffffu); };
+  // Job j, of prompt length s0, has become free.
+  auto freed = [&](int j, u32 s0) { if (cj == -2 || j < fj) { fj = j; cj = j; cs = static_cast<int>(s0); } };
+  // The lowest free job, -1 if there is none.
+  auto first_free = [&]() {
+    for (int b = (fj >> 5) & ~3; b < m / 32; b += 128) {
+      const int w = b + 4 * lane;
+      uint4 v = make_uint4(0, 0, 0, 0);
+      if (w < m / 32) v = *reinterpret_cast<const uint4*>(free_map + w);
+      const u32 bits = v.x ? v.x : (v.y ? v.y : (v.z ? v.z : v.w));
+      const int word = w + (v.x ? 0 : (v.y ? 1 : (v.z ? 2 : 3)));
+      const unsigned hit = __ballot_sync(0xffffffffu, bits != 0);
+      if (hit) return __shfl_sync(0xffffffffu, 32 * word + __ffs(static_cast<int>(bits)) - 1, __ffs(static_cast<int>(hit)) - 1);
+    }
+    return -1;
+  };
+  // Keeps the live entries of the stack, in order (of every running job the uppermost one, whose place waits in job_start), and forms the
+  // earliest completion of every block of entries again.
+  auto purge = [&](int t) {
+    for (int b = lane; b * STK_BLK < top; b += 32) first_fin[b] = NO_ROUND;
+    __syncwarp();
     int w = 0;
-    for (int q0 = 0; q0 < top; q0 += 32) {
-      const int q = q0 + lane;
-      const u32 v = q < top ? stk[q] : 0u;
-      const bool live = q < top && sst[v >> 16] == (v & 0xffffu);
-      const unsigned lm = __ballot_sync(0xffffffffu, live);
+    constexpr int U = 4;
+    for (int q0 = 0; q0 < top; q0 += 32 * U) {
+      u32 j[U], sm[U];
+      int place[U];
+#pragma unroll
+      for (int i = 0; i < U; ++i) {
+        const int q = q0 + 32 * i + lane;
+        j[i] = q < top ? stk[q] : 0u;
+        sm[i] = q < top ? sst[j[i]] : IDLE;
+        place[i] = js[j[i]];
+      }
       __syncwarp();
-      if (live) stk[w + __popc(lm & lt_mask)] = v;
-      w += __popc(lm);
+#pragma unroll
+      for (int i = 0; i < U; ++i) {
+        const bool live = sm[i] != IDLE && place[i] == q0 + 32 * i + lane;
+        const unsigned lm = __ballot_sync(0xffffffffu, live);
+        if (live) {
+          const int d = w + __popc(lm & lt_mask);
+          stk[d] = static_cast<unsigned short>(j[i]);
+          js[j[i]] = d;
+          atomicMin(&first_fin[d / STK_BLK], static_cast<u32>(t) + (lengths[j[i]] >> 16) - running_for(sm[i]));
+        }
+        w += __popc(lm);
+      }
       __syncwarp();
     }
     top = w;
   };
-  // Earliest completion of every block of entries, formed again (after a purge).
-  auto index_stack = [&](int t) {
-    for (int b = lane; b * STK_BLK < top; b += 32) first_fin[b] = NO_ROUND;
-    __syncwarp();
-    for (int q = lane; q < top; q += 32) {
-      const u32 v = stk[q], j = v >> 16;
-      atomicMin(&first_fin[q / STK_BLK], static_cast<u32>(t) + Osh[j] - running_for(v & 0xffffu));
-    }
-    __syncwarp();
-  };
-  int purged = 0;
   int t = 0;
   while (t <= H) {
     const u32 tu = static_cast<u32>(t);
-    if ((t & 31) == 0 && t < H) {
-      load_window(t);
-      // an entry that is not live must leave before its start comes round again modulo MODT
-      if (t - purged > 30000) { purge(); index_stack(t); purged = t; }
+    const int w = t & ~31;
+    if (t == w && t < H) {
+      Bw = Bn;
+      Bn = t + 32 + lane < H ? __ldcg(prof + t + 32 + lane) : 0;
+      const u32 a = Ad, c = Cd;
+      if (far_next < w + ring_rounds) {                 // ends that the ring has come to
+        int next = NEVER;
+#pragma unroll
+        for (int f = 0; f < FAR_SETS; ++f) {
+          if (far_end[f] != 0 && far_end[f] < w + ring_rounds) {
+            atomicAdd(&ring_a[far_end[f] & ring_mask], far_v[f]); atomicAdd(&ring_c[far_end[f] & ring_mask], far_c[f]);
+            far_end[f] = 0;
+          }
+          if (far_end[f] != 0) next = min(next, far_end[f]);
+        }
+        far_next = static_cast<int>(__reduce_min_sync(0xffffffffu, static_cast<u32>(next)));
+        __syncwarp();
+      }
+      if (ph.ahead) look_ahead(w, t, true);
+      apply_ring(w, a, c);
     }
     // (1) speculative completions
     if (tu == next_comp) {
@@ -654,214 +864,225 @@ __global__ void __launch_bounds__(64) k_spec_smem(SpecParams p, int n_cap) {
         if (f > tu) nc = min(nc, f);
         unsigned due = __ballot_sync(0xffffffffu, f <= tu);
         while (due) {
-          const int b = b0 + __ffs(static_cast<int>(due)) - 1;
+          const int b = b0 + __ffs(static_cast<int>(due)) - 1, q = b * STK_BLK + 2 * lane;
           due &= due - 1u;
-          u32 rest = NO_ROUND;
+          const u32 both = q < top ? *reinterpret_cast<const u32*>(stk + q) : 0u;
+          const u32 j0 = both & 0xffffu, j1 = q + 1 < top ? both >> 16 : 0u;
+          const u32 sm0 = q < top ? sst[j0] : IDLE, sm1 = q + 1 < top ? sst[j1] : IDLE, so0 = lengths[j0], so1 = lengths[j1];
+          const u32 ran0 = running_for(sm0), ran1 = running_for(sm1), o0 = so0 >> 16, o1 = so1 >> 16;
+          const bool fin0 = sm0 != IDLE && ran0 == o0, fin1 = sm1 != IDLE && ran1 == o1;
+          const u32 rest0 = sm0 == IDLE || fin0 ? NO_ROUND : tu + o0 - ran0, rest1 = sm1 == IDLE || fin1 ? NO_ROUND : tu + o1 - ran1;
+          const unsigned fm0 = __ballot_sync(0xffffffffu, fin0), fm1 = __ballot_sync(0xffffffffu, fin1);
+          const u32 rest = __reduce_min_sync(0xffffffffu, min(rest0, rest1));
+          if (lane == 0) first_fin[b] = rest;
+          nc = min(nc, rest);
+          if (!(fm0 | fm1)) continue;
+          if (__popc(fm0) + __popc(fm1) == 1) {         // one run
+            const u32 j = __shfl_sync(0xffffffffu, fm0 ? j0 : j1, __ffs(static_cast<int>(fm0 | fm1)) - 1), so = lengths[j], o = so >> 16;
+            if (lane == 0) {
+              done[j >> 5] |= 1u << (j & 31u);
+              sst[j] = static_cast<unsigned short>(IDLE);
+              if (KVS_OK_AT(j, n, CHK_SP_JOB)) { js[j] = t - static_cast<int>(o); jc[j] = t; }
+              steps += o; flow += t; ++runs; hmax = max(hmax, t);
+            }
+            A -= (so & 0xffffu) + 1u - (tu - o);
+            --cnt; --left;
+          } else {
+            u32 dA = 0, n_fin = 0;
 #pragma unroll
-          for (int h = 0; h < STK_BLK; h += 32) {
-            const int q = b * STK_BLK + h + lane;
-            const u32 v = q < top ? stk[q] : 0u, j = v >> 16;
-            const bool live = q < top && sst[j] == (v & 0xffffu);
-            const u32 o = Osh[j], ran = running_for(v & 0xffffu);
-            const bool fin = live && ran == o;
-            if (live && !fin) rest = min(rest, tu + o - ran);
-            const unsigned fm = __ballot_sync(0xffffffffu, fin);
-            if (fm) {
-              if (fin) {
-                atomicOr(&done[j >> 5], 1u << (j & 31u));
+            for (int h = 0; h < 2; ++h) {
+              const u32 j = h ? j1 : j0, so = h ? so1 : so0, o = so >> 16;
+              if ((h ? fin1 : fin0) && (atomicOr(&done[j >> 5], 1u << (j & 31u)) >> (j & 31u) & 1u) == 0) {   // the first of its entries
                 sst[j] = static_cast<unsigned short>(IDLE);
                 if (KVS_OK_AT(j, n, CHK_SP_JOB)) { js[j] = t - static_cast<int>(o); jc[j] = t; }
                 steps += o; flow += t; ++runs; hmax = max(hmax, t);
+                dA += (so & 0xffffu) + 1u - (tu - o);
+                ++n_fin;
               }
-              A -= __reduce_add_sync(0xffffffffu, fin ? Ssh[j] + 1u - (tu - o) : 0u);
-              cnt -= __popc(fm); left -= __popc(fm);
             }
+            const int kf = static_cast<int>(__reduce_add_sync(0xffffffffu, n_fin));
+            A -= __reduce_add_sync(0xffffffffu, dA);
+            cnt -= kf; left -= kf;
           }
-          rest = __reduce_min_sync(0xffffffffu, rest);
-          if (lane == 0) first_fin[b] = rest;
-          nc = min(nc, rest);
+          __syncwarp();
         }
       }
       next_comp = __reduce_min_sync(0xffffffffu, nc);
       __syncwarp();
     }
-    // slots that have ended: a job killed at the end of its slot is free again (see k_spec)
-    if (ne <= t && ph.single) {
-      const int eend = re + 1;
-      bool before = false;
-      if (re < fpos) {
-        const u32 j = list[re];
-        before = sst[j] == IDLE && !is_done(j);
-        if (before) { fpos = re; cj = -1; }
-      }
-      if (eend > fhi && (cj == -1 || eend > min(eend, fpos))) fhi = eend;
-      re = eend;
-      e_rem += ph.rt; ne += ph.qt;
-      if (e_rem >= static_cast<int>(ph.k)) { e_rem -= static_cast<int>(ph.k); ++ne; }
-      if (re >= ph.np) ne = NEVER;
-    } else if (ne <= t) {
-      const int eend = ph.started(t - static_cast<int>(ph.tau) - ph.base);
-      const int lim = min(eend, fpos);
-      for (int r0 = re; r0 < lim; r0 += 32) {
-        const int r = r0 + lane;
-        bool fr = false;
-        if (r < lim) { const u32 j = list[r]; fr = sst[j] == IDLE && !is_done(j); }
+    // slots that have ended: a job killed at the end of its slot is free again
+    if (ne <= t) {
+      const int eend = ph.ahead ? 0 : ph.started(t - static_cast<int>(ph.tau) - ph.base);
+      do {
+        bool act;
+        if (ph.ahead) {
+          act = (end_mask >> lane & 1u) != 0 && end_at <= t;
+          end_mask &= ~__ballot_sync(0xffffffffu, act);
+        } else {
+          const int r = re + lane;
+          act = r < eend;
+          end_job = act ? job_of(r) : 0u;
+          re = min(re + 32, eend);
+        }
+        const bool fr = act && !is_done(end_job);
+        if (fr) atomicOr(&free_map[end_job >> 5], 1u << (end_job & 31u));
         const unsigned hit = __ballot_sync(0xffffffffu, fr);
-        if (hit) { fpos = r0 + __ffs(static_cast<int>(hit)) - 1; cj = -1; break; }
-      }
-      if (eend > fhi && (cj == -1 || eend > lim)) fhi = eend;
-      re = eend;
-      ne = re < ph.np ? ph.start_of(re) + static_cast<int>(ph.tau) : NEVER;
+        if (hit) {                                      // ranks are in index order
+          const int j = static_cast<int>(__shfl_sync(0xffffffffu, end_job, __ffs(static_cast<int>(hit)) - 1));
+          freed(j, lengths[j] & 0xffffu);
+        }
+        if (ph.ahead) {
+          if (end_mask) ne = __shfl_sync(0xffffffffu, end_at, __ffs(static_cast<int>(end_mask)) - 1);
+          else next_ends();
+        } else if (re >= eend) {
+          ne = re < ph.np ? ph.start_of(re) + static_cast<int>(ph.tau) : NEVER;
+        }
+      } while (ne <= t);
+      __syncwarp();
     }
     // the next phase begins: its participants are the jobs of a later class, in index order
     if (t == phase_at) {
-      int w = 0;
+      int kept = 0;
       for (int q0 = 0; q0 < ph.np; q0 += 32) {
         const int q = q0 + lane;
-        const u32 j = q < ph.np ? list[q] : 0u;
-        const bool keep = q < ph.np && Osh[j] > ph.tau;
+        const u32 j = q < ph.np ? job_of(q) : 0u;
+        const bool keep = q < ph.np && lengths[j] >> 16 > ph.tau;
         const unsigned km = __ballot_sync(0xffffffffu, keep);
         __syncwarp();
-        if (keep) list[w + __popc(km & lt_mask)] = static_cast<unsigned short>(j);
-        w += __popc(km);
+        if (keep) list[kept + __popc(km & lt_mask)] = static_cast<unsigned short>(j);
+        kept += __popc(km);
         __syncwarp();
       }
       ++phase;
-      enter(phase, w);
+      all_take_part = kept == n;
+      enter(phase, kept);
       rs = 0; re = 0; ns = ph.base; ne = ph.base + static_cast<int>(ph.tau);
-      s_rem = 0; e_rem = 0;
-      phase_at = phase + 1 < L && sh.np[phase + 1] > 0 ? static_cast<int>(sh.pbase[phase + 1]) : NEVER;
-      fpos = 0; fhi = ph.np; cj = -1;
+      phase_at = phase + 1 < L && sh.np[phase + 1] > 0 ? sh.pbase[phase + 1] : NEVER;
+      if (ph.ahead) { look_ahead(w, t, false); apply_ring(w, 0u, 0u); }
     }
-    // (2) pipeline runs that start now.  One run: no votes and no sums over lanes
-    if (ns <= t && ph.single) {
-      const u32 j = list[rs], o = Osh[j], s1 = Ssh[j] + 1u, sm = sst[j], len = min(o, ph.tau);
-      const int end = t + static_cast<int>(len);
-      if (is_done(j)) {                                 // dropped from the plan
-        const int u = (t & ~31) + lane, w_end = (t & ~31) + 32;
-        if (u >= t && u < end) Bw -= static_cast<int>(s1 + static_cast<u32>(u - t));
-        if (end > w_end) {
-          if (end < (t & ~31) + DROP_RING) {
-            const u32 v = s1 - tu;
-            Ad += v; ++Cd;
-            if (lane == 0) { ring_a[end & (DROP_RING - 1)] += v; ++ring_c[end & (DROP_RING - 1)]; }
+    // (2) pipeline runs that start now
+    if (ns <= t) {
+      const int rend = ph.ahead ? 0 : ph.started(t - ph.base);
+      do {
+        unsigned acting;
+        if (ph.ahead) {
+          acting = __ballot_sync(0xffffffffu, (start_mask >> lane & 1u) != 0 && start_at <= t);
+          start_mask &= ~acting;
+        } else {                                        // ranks [rs, rend), 32 at a time (they concern different jobs)
+          const int r = rs + lane;
+          start_job = r < rend ? job_of(r) : 0u;
+          const u32 so = lengths[start_job];
+          start_o = so >> 16; start_s1 = (so & 0xffffu) + 1u;
+          acting = __ballot_sync(0xffffffffu, r < rend);
+          rs = min(rs + 32, rend);
+        }
+        if ((acting & (acting - 1u)) == 0) {            // one run: no votes and no sums over lanes
+          const int src = __ffs(static_cast<int>(acting)) - 1;
+          const u32 j = __shfl_sync(0xffffffffu, start_job, src), o = __shfl_sync(0xffffffffu, start_o, src), s1 = __shfl_sync(0xffffffffu, start_s1, src);
+          const u32 sm = sst[j], len = min(o, ph.tau);
+          const int end = t + static_cast<int>(len);
+          if (is_done(j)) {                             // dropped from the plan
+            drop_now(w, t, s1 - tu, 1u, end);
           } else {
-            for (int x = w_end + lane; x < end; x += 32)
-              if (KVS_OK_AT(x, H, CHK_SP_DROP)) atomicSub(&prof[x], static_cast<int>(s1 + static_cast<u32>(x - t)));
+            const bool comp = len == o;
+            if (sm != IDLE) {                           // its speculative run is killed; the stack entry goes stale
+              const u32 ran = running_for(sm);
+              A -= s1 - (tu - ran);
+              --cnt;
+              if (lane == 0) { steps += ran; runs += ran > 0 ? 1u : 0u; }
+            }
+            __syncwarp();
+            if (lane == 0) {
+              steps += len; ++runs;
+              sst[j] = static_cast<unsigned short>(IDLE);
+              free_map[j >> 5] &= ~(1u << (j & 31u));
+              if (comp) {
+                done[j >> 5] |= 1u << (j & 31u);
+                if (KVS_OK_AT(j, n, CHK_SP_JOB)) { js[j] = t; jc[j] = end; }
+                flow += end;
+                hmax = max(hmax, end);
+              }
+            }
+            left -= comp ? 1 : 0;
+            if (static_cast<int>(j) == cj) cj = -1;
           }
-        }
-      } else {
-        const bool comp = len == o;
-        if (sm != IDLE) {                               // its speculative run is killed
-          const u32 ran = running_for(sm);
-          A -= s1 - (tu - ran);
-          --cnt;
-          if (lane == 0) { steps += ran; runs += ran > 0 ? 1u : 0u; }
-        }
-        __syncwarp();
-        if (lane == 0) {
-          steps += len; ++runs;
-          sst[j] = static_cast<unsigned short>(IDLE);
-          if (comp) {
-            done[j >> 5] |= 1u << (j & 31u);
-            if (KVS_OK_AT(j, n, CHK_SP_JOB)) { js[j] = t; jc[j] = end; }
-            flow += end;
-            hmax = max(hmax, end);
+          __syncwarp();
+        } else {
+          const bool act = (acting >> lane & 1u) != 0;
+          const u32 j = act ? start_job : 0u, o = start_o, s1 = start_s1, sm = sst[j], len = min(o, ph.tau);
+          const bool dn = is_done(j), run = act && !dn, drop = act && dn, comp = run && len == o;
+          const bool kill = run && sm != IDLE;
+          const unsigned km = __ballot_sync(0xffffffffu, kill), dm = __ballot_sync(0xffffffffu, drop), cm = __ballot_sync(0xffffffffu, comp);
+          if (__any_sync(0xffffffffu, run && static_cast<int>(j) == cj)) cj = -1;
+          left -= __popc(cm);
+          if (km) {
+            const u32 ran = running_for(sm);
+            A -= __reduce_add_sync(0xffffffffu, kill ? s1 - (tu - ran) : 0u);
+            cnt -= __popc(km);
+            if (kill) { steps += ran; runs += ran > 0 ? 1u : 0u; }
           }
-        }
-        left -= comp ? 1 : 0;
-      }
-      __syncwarp();
-      if (static_cast<int>(j) == cj) cj = -1;
-      ++rs;
-      s_rem += ph.rt; ns += ph.qt;
-      if (s_rem >= static_cast<int>(ph.k)) { s_rem -= static_cast<int>(ph.k); ++ns; }
-      if (rs >= ph.np) ns = NEVER;
-    } else if (ns <= t) {                               // ranks [rs, started(t)), 32 at a time (they concern different jobs)
-      const int rend = ph.started(t - ph.base);
-      const int w_end = (t & ~31) + 32;                 // the window's rounds are in registers: they are corrected there
-      bool cand_started = false;
-      for (int r0 = rs; r0 < rend; r0 += 32) {
-        const int r = r0 + lane;
-        const bool act = r < rend;
-        const u32 j = act ? list[r] : 0u, o = Osh[j], s1 = Ssh[j] + 1u, sm = sst[j];
-        const bool dn = is_done(j);
-        __syncwarp();
-        if (cj >= 0 && __any_sync(0xffffffffu, act && static_cast<int>(j) == cj)) cand_started = true;
-        const u32 len = min(o, ph.tau);
-        const bool run = act && !dn, drop = act && dn, comp = run && len == o;
-        const bool kill = run && sm != IDLE;            // its speculative run is killed; the stack entry goes stale
-        const unsigned km = __ballot_sync(0xffffffffu, kill);
-        if (km) {
-          const u32 ran = running_for(sm);
-          A -= __reduce_add_sync(0xffffffffu, kill ? s1 - (tu - ran) : 0u);
-          cnt -= __popc(km);
-          if (kill) { steps += ran; runs += ran > 0 ? 1u : 0u; }
-        }
-        if (run) {
-          steps += len; ++runs;
-          sst[j] = static_cast<unsigned short>(IDLE);
+          if (run) {
+            steps += len; ++runs;
+            sst[j] = static_cast<unsigned short>(IDLE);
+            if (!kill) atomicAnd(&free_map[j >> 5], ~(1u << (j & 31u)));
+          }
           if (comp) {
             atomicOr(&done[j >> 5], 1u << (j & 31u));
             if (KVS_OK_AT(j, n, CHK_SP_JOB)) { js[j] = t; jc[j] = t + static_cast<int>(len); }
             flow += t + static_cast<int>(len);
             hmax = max(hmax, t + static_cast<int>(len));
           }
-        }
-        left -= __popc(__ballot_sync(0xffffffffu, comp));
-        // dropped from the plan: those that would have held their whole slot together, the others one by one
-        unsigned dm = __ballot_sync(0xffffffffu, drop);
-        if (dm) {
-          const bool whole = drop && len == ph.tau;
-          const unsigned wm = __ballot_sync(0xffffffffu, whole);
-          dm &= ~wm;
-          for (bool first = wm != 0; first || dm; first = false) {
-            u32 S1, c, d;                               // sum of s + 1, number and length of the runs of this step
-            if (first) {
-              S1 = __reduce_add_sync(0xffffffffu, whole ? s1 : 0u);
-              c = static_cast<u32>(__popc(wm));
-              d = ph.tau;
-            } else {
-              const int src = __ffs(static_cast<int>(dm)) - 1;
-              dm &= dm - 1u;
-              S1 = __shfl_sync(0xffffffffu, s1, src);
-              c = 1u;
-              d = __shfl_sync(0xffffffffu, len, src);
+          // dropped from the plan: those that would have held their whole slot together, those that reach beyond the window
+          // together, the others one by one
+          if (dm) {
+            const int end = t + static_cast<int>(len);
+            const u32 v = s1 - tu;
+            const unsigned wm = __ballot_sync(0xffffffffu, drop && len == ph.tau);
+            if (wm) drop_now(w, t, __reduce_add_sync(0xffffffffu, drop && len == ph.tau ? v : 0u), static_cast<u32>(__popc(wm)), t + static_cast<int>(ph.tau));
+            const bool rest = drop && len < ph.tau, beyond = rest && end >= w + 32 && end < w + ring_rounds;
+            const unsigned bm = __ballot_sync(0xffffffffu, beyond);
+            if (bm) {
+              const u32 V = __reduce_add_sync(0xffffffffu, beyond ? v : 0u), c = static_cast<u32>(__popc(bm));
+              if (w + lane >= t) Bw -= static_cast<int>(V + c * static_cast<u32>(w + lane));
+              Ad += V; Cd += c;
+              if (beyond) { atomicAdd(&ring_a[end & ring_mask], v); atomicAdd(&ring_c[end & ring_mask], 1u); }
             }
-            const int end = t + static_cast<int>(d);
-            const int u = (t & ~31) + lane;
-            if (u >= t && u < end) Bw -= static_cast<int>(S1 + c * static_cast<u32>(u - t));
-            if (end <= w_end) continue;
-            if (end < (t & ~31) + DROP_RING) {
-              const u32 v = S1 - c * tu;
-              Ad += v; Cd += c;
-              if (lane == 0) { ring_a[end & (DROP_RING - 1)] += v; ring_c[end & (DROP_RING - 1)] += c; }
-              __syncwarp();
-            } else {
-              for (int x = w_end + lane; x < end; x += 32)
-                if (KVS_OK_AT(x, H, CHK_SP_DROP)) atomicSub(&prof[x], static_cast<int>(S1 + c * static_cast<u32>(x - t)));
+            unsigned om = __ballot_sync(0xffffffffu, rest && !beyond);
+            while (om) {
+              const int src = __ffs(static_cast<int>(om)) - 1;
+              om &= om - 1u;
+              const u32 vs = __shfl_sync(0xffffffffu, v, src);
+              drop_now(w, t, vs, 1u, __shfl_sync(0xffffffffu, end, src));
             }
           }
+          __syncwarp();
         }
-        __syncwarp();
-      }
-      if (cand_started) cj = -1;
-      rs = rend;
-      ns = rs < ph.np ? ph.start_of(rs) : NEVER;
+        if (ph.ahead) {
+          if (start_mask) ns = __shfl_sync(0xffffffffu, start_at, __ffs(static_cast<int>(start_mask)) - 1);
+          else next_starts();
+        } else if (rs >= rend) {
+          ns = rs < ph.np ? ph.start_of(rs) : NEVER;
+        }
+      } while (ns <= t);
     }
     if (t == H) break;                                  // nothing runs in round H; only completions were due
     if (left == 0) {
       // Every job is done: what is left of the plan are the completing runs in progress (see k_spec)
       __threadfence();
       __syncwarp();
-      for (int u = t + lane; u < H; u += 32) prof[u] = 0;
+      const int first4 = t + static_cast<int>((4u - (reinterpret_cast<uintptr_t>(prof + t) >> 2 & 3u)) & 3u);
+      for (int u = t + lane; u < min(first4, H); u += 32) prof[u] = 0;
+      int last4 = first4;
+      if (first4 + 4 <= H) last4 = first4 + ((H - first4) & ~3);
+      for (int u = first4 + 4 * lane; u < last4; u += 128) *reinterpret_cast<int4*>(prof + u) = make_int4(0, 0, 0, 0);
+      for (int u = last4 + lane; u < H; u += 32) prof[u] = 0;
       hmax = warp_max(hmax);
       __syncwarp();
-      for (int r = re; r < rs; ++r) {
-        const u32 j = list[r];
+      for (int r = ph.ahead ? end_first : re; r < rs; ++r) {
+        const u32 j = job_of(r);
         const int end = jc[j];
         if (end > t && KVS_OK_AT(end, H + 1, CHK_SP_PROF)) {
-          const int first = end - static_cast<int>(Osh[j]), sj = Ssh[j];
+          const int first = end - static_cast<int>(lengths[j] >> 16), sj = prompt(j);
           for (int u = t + lane; u < end; u += 32) prof[u] += sj + (u - first) + 1;
           __syncwarp();
         }
@@ -872,99 +1093,89 @@ __global__ void __launch_bounds__(64) k_spec_smem(SpecParams p, int n_cap) {
     const u32 B = static_cast<u32>(__shfl_sync(0xffffffffu, Bw, t & 31));
     // (3) the pipeline comes first
     while (cnt > 0 && B + A + tu * static_cast<u32>(cnt) > Mu) {
-      u32 v = 0;
-      bool found = false;
-      while (top > 0) {                                 // the live entry nearest to the top
-        v = stk[--top];
-        if (sst[v >> 16] == (v & 0xffffu)) { found = true; break; }
+      u32 j = 0, sm = IDLE;
+      while (top > 0 && sm == IDLE) {                   // the live entry nearest to the top: no other of its job is above it
+        j = stk[--top];
+        sm = sst[j];
       }
-      if (!found) break;
-      const u32 j = v >> 16, ran = running_for(v & 0xffffu);
-      A -= Ssh[j] + 1u - (tu - ran);
+      if (sm == IDLE) break;
+      const u32 ran = running_for(sm), s0 = lengths[j] & 0xffffu;
+      A -= s0 + 1u - (tu - ran);
       --cnt;
-      if (lane == 0) { steps += ran; runs += ran > 0 ? 1u : 0u; sst[j] = static_cast<unsigned short>(IDLE); }
+      steps += lane == 0 ? ran : 0u;
+      runs += lane == 0 && ran > 0 ? 1u : 0u;
       __syncwarp();
-      // its position: the list is in index order
-      int a = 0, b = ph.np;
-      while (b - a > 1) {
-        const int step = (b - a + 31) / 32, x = a + (lane + 1) * step;
-        const int hits = __popc(__ballot_sync(0xffffffffu, x < b && list[x] <= j));
-        b = min(b, a + (hits + 1) * step);
-        a += hits * step;
+      if (lane == 0) {
+        sst[j] = static_cast<unsigned short>(IDLE);
+        atomicOr(&free_map[j >> 5], 1u << (j & 31u));
       }
-      if (!KVS_OK_AT(a, n, CHK_SP_LIST)) break;
-      if (a < fpos) { fpos = a; cj = -1; }              // free again: it may come before the known candidate
-      if (a >= fhi) { fhi = a + 1; if (cj == -2) cj = -1; }
+      __syncwarp();
+      freed(static_cast<int>(j), s0);
     }
-    // (4) first come first served (see k_spec)
+    // (4) first come first served: the lowest free job, and with it those of the 32 indices it lies among, as far as their
+    // first rounds fit, in order; the first that does not fit ends the round's admissions
     for (;;) {
       const int room = static_cast<int>(Mu - (B + A + tu * static_cast<u32>(cnt)));
       if (cj == -2 || (cj >= 0 && cs + 1 > room) || room <= 0) break;
-      // the jobs in a pipeline run are the ranks whose slot has begun and not ended: [re, rs)
-      if (fpos >= re && fpos < rs) fpos = rs;
-      if (fpos >= fhi) { fpos = ph.np; fhi = 0; cj = -2; break; }
-      const int q = fpos + lane;
-      bool fr = false;
-      u32 j = 0, s1 = 0;
-      if (q < fhi && !(q >= re && q < rs)) { j = list[q]; fr = sst[j] == IDLE && !is_done(j); }
-      const unsigned hit = __ballot_sync(0xffffffffu, fr);
-      if (!hit) { fpos += 32; cj = -1; continue; }
-      {
-        // the first free job does not fit: it is the candidate from now on
-        const int src = __ffs(static_cast<int>(hit)) - 1;
-        const u32 jf = list[fpos + src];
-        if (static_cast<int>(Ssh[jf]) + 1 > room) { fpos += src; cj = static_cast<int>(jf); cs = Ssh[jf]; break; }
+      if (cj == -1) {
+        const int f = first_free();
+        if (f < 0) { cj = -2; break; }
+        cj = fj = f;
+        cs = prompt(f);
+        if (cs + 1 > room) break;
       }
-      if (fr) s1 = Ssh[j] + 1u;
-      u32 need = s1;                                    // inclusive sums over the window, in list order: below 32 * 2^16
+      const u32 j = (static_cast<u32>(cj) & ~31u) + lane, bits = free_map[j >> 5], so = lengths[j];
+      const bool fr = (bits >> lane & 1u) != 0;
+      const u32 s1 = fr ? (so & 0xffffu) + 1u : 0u;
+      u32 need = __reduce_add_sync(0xffffffffu, s1);    // below 32 * 2^16
+      if (need > static_cast<u32>(room)) {              // inclusive sums, in index order
+        need = s1;
 #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const u32 y = __shfl_up_sync(0xffffffffu, need, d);
-        if (lane >= d) need += y;
-      }
-      const bool ok = fr && static_cast<int>(need) <= room;
-      const unsigned okm = __ballot_sync(0xffffffffu, ok);
-      const int got = __popc(okm);
-      if (got) {
-        if (top + 32 > m || top > 2 * cnt + 64) { purge(); index_stack(t); }
-        // blocks that hold no entry yet start without a completion
-        if (lane < 2) { const int b = (top + STK_BLK - 1) / STK_BLK + lane; if (b * STK_BLK < m) first_fin[b] = NO_ROUND; }
-        __syncwarp();
-        const u32 fin = ok ? tu + Osh[j] : NO_ROUND;
-        if (ok) {
-          const int d = top + __popc(okm & lt_mask);
-          if (KVS_OK_AT(d, m, CHK_SP_STACK)) {
-            sst[j] = static_cast<unsigned short>(tm);
-            stk[d] = j << 16 | tm;
-            atomicMin(&first_fin[d / STK_BLK], fin);
-          }
+        for (int d = 1; d < 32; d <<= 1) {
+          const u32 y = __shfl_up_sync(0xffffffffu, need, d);
+          if (lane >= d) need += y;
         }
-        A += __reduce_add_sync(0xffffffffu, ok ? s1 - tu : 0u);
-        top += got;
-        cnt += got;
-        next_comp = min(next_comp, __reduce_min_sync(0xffffffffu, fin));
-        __syncwarp();
       }
-      const unsigned failed = hit & ~okm;
+      const bool ok = fr && need <= static_cast<u32>(room);
+      const unsigned okm = __ballot_sync(0xffffffffu, ok);    // the lowest free job at least
+      const int got = __popc(okm);
+      if (top + 32 > m || top > 3 * cnt + 256) purge(t);
+      const u32 fin = ok ? tu + (so >> 16) : NO_ROUND;
+      if (ok) {
+        const int d = top + __popc(okm & lt_mask);
+        if (KVS_OK_AT(d, m, CHK_SP_STACK)) {
+          sst[j] = static_cast<unsigned short>(tm);
+          stk[d] = static_cast<unsigned short>(j);
+          js[j] = d;
+          atomicMin(&first_fin[d / STK_BLK], fin);
+        }
+      }
+      if (lane == 0) free_map[j >> 5] = bits & ~okm;
+      A += __reduce_add_sync(0xffffffffu, ok ? s1 - tu : 0u);
+      top += got;
+      cnt += got;
+      next_comp = min(next_comp, __reduce_min_sync(0xffffffffu, fin));
+      const unsigned failed = bits & ~okm;
+      __syncwarp();
       if (failed) {                                     // the first free job that does not fit is the candidate from now on
         const int src = __ffs(static_cast<int>(failed)) - 1;
-        fpos += src;
-        cj = static_cast<int>(__shfl_sync(0xffffffffu, j, src));
+        cj = fj = (cj & ~31) + src;
         cs = static_cast<int>(__shfl_sync(0xffffffffu, s1, src)) - 1;
         break;
       }
-      fpos += 32; cj = -1;
+      fj = (cj & ~31) + 32;
+      cj = -1;
     }
     if (cnt == 0) top = 0;                              // only stale entries are left
     // (5) the memory of this round, and of those up to the next event in which nothing can happen
     {
-      const int stop = static_cast<int>(min(static_cast<u32>(min(min(min(ns, ne), phase_at), min((t & ~31) + 32, H))), next_comp));
-      const int u = (t & ~31) + lane;
+      const int stop = static_cast<int>(min(static_cast<u32>(min(min(min(ns, ne), phase_at), min(w + 32, H))), next_comp));
+      const int u = w + lane;
       const u32 mem = static_cast<u32>(Bw) + A + static_cast<u32>(u) * static_cast<u32>(cnt);
       const int room = static_cast<int>(Mu - mem);
       const bool quiet = !(cnt > 0 && room < 0) && (cj == -2 || room <= 0 || (cj >= 0 && cs + 1 > room));
       const unsigned busy = __ballot_sync(0xffffffffu, u > t && u < stop && !quiet);
-      const int next = max(t + 1, busy ? (t & ~31) + __ffs(static_cast<int>(busy)) - 1 : stop);
+      const int next = max(t + 1, busy ? w + __ffs(static_cast<int>(busy)) - 1 : stop);
       if (u >= t && u < next) {
         if (KVS_OK_AT(u, H, CHK_SP_PROF)) prof[u] = static_cast<int32_t>(mem);
         peak = max(peak, mem);
@@ -995,25 +1206,31 @@ i64 kvs_spec_warp_bytes(i64 max_jobs) { return spec_stride(max_jobs); }
 
 constexpr int SPEC_SMEM = 227 * 1024;
 
-// Evaluations of one instance that a CTA of the on-chip kernel takes: 2, 1, or 0 where not even one fits.
+static int spec_ring(int n, int warps) {
+  for (int r = RING_MAX; r >= RING_MIN; r /= 2)
+    if (smem_lengths_bytes(n) + warps * smem_state_bytes(n, r) <= SPEC_SMEM) return r;
+  return 0;
+}
+
+// Evaluations of one instance that a CTA of the on-chip kernel takes: up to KVS_SPEC_GROUP, 0 where not even one fits.
 int kvs_spec_per_cta(i64 max_jobs) {
-  if (max_jobs > 20000) return 0;
-  const int n = static_cast<int>(max_jobs);
-  for (int w = 2; w >= 1; --w)
-    if (smem_lengths_bytes(n) + w * smem_state_bytes(n) <= SPEC_SMEM) return w;
+  static_assert(KVS_SPEC_GROUP == SPEC_WARPS, "groups of evaluations");
+  if (max_jobs >= 65535) return 0;                      // 16-bit job numbers, one of them spare
+  for (int w = SPEC_WARPS; w >= 1; --w)
+    if (spec_ring(static_cast<int>(max_jobs), w)) return w;
   return 0;
 }
 
 // Once per device, before the first launch.
 cudaError_t kvs_setup_spec() { return cudaFuncSetAttribute(k_spec_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, SPEC_SMEM); }
 
-// The on-chip kernel over p.pairs, if there are any, and the other one over what it has left (or over the whole list).
+// The on-chip kernel over p.groups, if there are any, and the other one over what it has left (or over the whole list).
 cudaError_t kvs_launch_spec(SpecParams p, cudaStream_t stream) {
   if (p.n_list <= 0 || p.n_warps <= 0) return cudaSuccess;
-  const int per_cta = p.n_pairs > 0 ? kvs_spec_per_cta(p.max_jobs) : 0;
+  const int per_cta = p.n_groups > 0 ? kvs_spec_per_cta(p.max_jobs) : 0;
   if (per_cta > 0) {
-    const int n = static_cast<int>(p.max_jobs);
-    k_spec_smem<<<static_cast<unsigned>(p.n_pairs), 32 * per_cta, smem_lengths_bytes(n) + per_cta * smem_state_bytes(n), stream>>>(p, n);
+    const int n = static_cast<int>(p.max_jobs), ring = spec_ring(n, per_cta);
+    k_spec_smem<<<static_cast<unsigned>(p.n_groups), 32 * per_cta, smem_lengths_bytes(n) + per_cta * smem_state_bytes(n, ring), stream>>>(p, n, ring);
   } else {
     p.left_list = nullptr;
   }

@@ -97,7 +97,7 @@ def _spec_instance(n, seed, o_max, s_max):
 
 @pytest.mark.parametrize("n", [9_000, 12_000, 20_500])
 def test_evaluations_on_chip_by_size(par, n):
-    """Two evaluations per CTA in shared memory, one, none (an odd number of budgets leaves one without a partner)."""
+    """Four evaluations per CTA of the kernel in shared memory, three, one (three budgets leave the fourth warp without one)."""
     s, o = _spec_instance(n, 63, 60, 20)
     inst = workloads.Instances(torch.tensor([0, n]), s, o)
     par.check_batch(inst, binding.settings_grid(range(1), ["GSAS"], [1 << 14, 1 << 16, 1 << 18]), want_runs=False, label=f"spec n={n}")
@@ -115,3 +115,23 @@ def test_evaluations_left_by_the_on_chip_kernel(par):
     rows = [dict(instance=i, family="GSAS", M=M) for i in range(len(sizes)) for M in (140_000, 200_000)]
     rows += [dict(instance=5, family="GSAS", M=M) for M in ((1 << 30) - 1, 1 << 30)]
     par.check_batch(inst, binding.make_settings(rows), want_runs=False, label="spec left")
+
+
+@pytest.mark.parametrize("n", [31, 33, 127, 129, 4_095, 4_097])
+def test_on_chip_maps_and_groups(par, n):
+    """Edges of the words, the 128-job rows and the 4,096-job probes of the map of free jobs; five budgets make a full CTA and a
+    CTA of one.  The small budgets' windows of 32 rounds are looked at as a whole, those of the large ones hold too many starts."""
+    s, o = _spec_instance(n, 71, 60, 20)
+    inst = workloads.Instances(torch.tensor([0, n]), s, o)
+    st = binding.settings_grid(range(1), ["GSAS"], [1 << 8, 1 << 9, 1 << 11, 1 << 14, 1 << 17])
+    par.check_batch(inst, st, want_runs=False, label=f"spec maps n={n}")
+    st["alpha_num"], st["alpha_den"] = 3, 2               # slices that occur twice: phases that nobody leaves
+    par.check_batch(inst, st[1:4], want_runs=False, label=f"spec maps 3/2 n={n}")
+
+
+@pytest.mark.parametrize("n, lo, hi, M", [(900, 2_100, 4_000, 1 << 19), (900, 2_100, 4_000, 1 << 20), (500, 300, 1_300, 1 << 17), (60, 8_000, 40_000, 1 << 18)])
+def test_long_runs_leave_the_plan(par, n, lo, hi, M):
+    """Dropped runs that end within the ring of rounds, beyond it, and more of them at a time than the list of those holds."""
+    c = torch.arange(n)
+    inst = workloads.Instances(torch.tensor([0, n]), workloads.uniform_int(81, c, 0, 20), workloads.uniform_int(82, c, lo, hi))
+    par.check_batch(inst, binding.settings_grid(range(1), ["GSAS"], [M]), want_runs=False, label=f"spec long {lo}..{hi} M={M}")
