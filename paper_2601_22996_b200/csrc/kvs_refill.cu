@@ -17,8 +17,10 @@
 // global memory).  A round that enters the ring holds what the batching schedule has there less the ramps of the jobs
 // already taken: nothing before the next job's old start, otherwise the stored profile minus the few of those
 // ramps that reach so far (old starts therefore stay in job_start until the end; the new ones wait in job_completion).
-// One warp walks the ring; the next 32 to 64 jobs are loaded ahead.  With one warp per evaluation on the plan in global memory 1,024 evaluations of 5,000 to 10,000 jobs took
-// 20.4 ms; now 3.7 ms.
+// One warp walks the ring; the next 32 to 64 jobs are loaded ahead, and up to 32 of them, of about the same length, are tried together.
+// A call of 1,024 evaluations of 5,000 to 10,000 jobs, batching schedules included: 3.0 ms (jobs of one length together, eight at a time,
+// every one of the eight tested, and 128 threads with four loads in flight for the long ones: 4.3; one warp per evaluation on the
+// plan in global memory: 21).
 #include "kvs_check.cuh"
 
 namespace {
@@ -26,7 +28,6 @@ namespace {
 constexpr int RT = 128;
 constexpr int RING = 4096;              // 16 KB
 constexpr int FILL = 128;               // rounds that enter the ring together
-constexpr int GROUP = 8;                // jobs of one response length tried together at the last admission
 
 struct Job { int j, o, s, g; };
 
@@ -50,11 +51,11 @@ __device__ __forceinline__ void quads(int* ring, int u0, int u1, F f) {
 
 __global__ void __launch_bounds__(RT) k_refill(RefillParams p) {
   __shared__ alignas(16) int ring[RING];
-  __shared__ int4 sh_job[2][32];
-  __shared__ int sh_next, sh_prev, sh_hmax;
+  __shared__ int4 sh_job[64];
+  __shared__ int sh_next, sh_prev, sh_filled, sh_max[32];
   __shared__ i64 sh_best[RT / 32], sh_peak[32];
   __shared__ int sh_arg[RT / 32];
-  __shared__ i64 sh_flow;
+  __shared__ i64 sh_sum[32];
   const int lane = lane_id(), tid = threadIdx.x;
   const i64 e = p.eval_list[blockIdx.x];
   if (p.status && p.status[e] != 0) return;            // the batching schedule was not formed or not stored in full
@@ -106,8 +107,7 @@ __global__ void __launch_bounds__(RT) k_refill(RefillParams p) {
 
   if (tid < 32) {
     int base = 0, filled = 0;                           // the ring holds rounds [base, filled)
-    int hmax = 0, x0 = 0;
-    i64 flow = 0;
+    int x0 = 0;
     bool tail = false;
     bool negative = false;                              // a word of the plan does not fit 31 bits: no short cuts
     // No admission before round t any more: the rounds before it are final.
@@ -132,106 +132,170 @@ __global__ void __launch_bounds__(RT) k_refill(RefillParams p) {
       if (!nothing) take_out(y, filled, v1, o_last, true);
       filled = v1;
     };
-    // jobs x0 .. x0 + 63 lie in sh_job (two halves of 32), the 32 after them are on their way
-    auto keep = [&](int half, const Job& b) { sh_job[half][lane] = make_int4(b.o, b.s, b.g, b.j); };
+    // Memory modulo 2^32: a word of the plan is below 2^31, the prompts of `most_jobs` jobs that fit M one by one are below 2^32, and
+    // 2^20 is room for the slopes of 32 jobs over the ring.
+    const u32 Mu = static_cast<u32>(M);
+    const int most_jobs = M >> 27 ? static_cast<int>(0xffffffffu / Mu) : 32;
+    if (M > (1ll << 31) - (1 << 20)) negative = true;
+    // jobs x0 .. x0 + 63 lie in sh_job (job x at x mod 64: response, sum of s + 1 up to it modulo 2^32, old start, index), the 32 after
+    // them are on their way
+    u32 sum = 0;
+    auto keep = [&](int from, const Job& b) {
+      const u32 P = sum + warp_incl(static_cast<u32>(b.s) + 1u);
+      sh_job[(from + lane) & 63] = make_int4(b.o, static_cast<int>(P), b.g, b.j);
+      sum = __shfl_sync(0xffffffffu, P, 31);
+    };
+    u32 before = 0;                                     // the sum up to the job before x
     keep(0, load(lane));
     Job nxt = load(32 + lane);
-    for (int half = 0; x0 < n && !tail; x0 += 32, half ^= 1) {
-      keep(half ^ 1, nxt);
+    int x = 0;
+    for (; x0 < n && !tail; x0 += 32) {
+      keep(x0 + 32, nxt);
       __syncwarp();
       nxt = load(x0 + 64 + lane);
       const int m = min(32, n - x0);
-      int x = 0;
       while (x < m) {
-        const int4 b = sh_job[half][x];
-        const int o = b.x, s = b.y, g = b.z, j = b.w;
+        const int4 b = sh_job[(x0 + x) & 63], c = sh_job[(x0 + x + lane) & 63];   // the next job; lane i: the i-th from here on
+        const int o = b.x, g = b.z;
         if (o > RING - 4) { tail = true; break; }
-        if (filled < base + o) fill_to(x0 + x, base + o, g, o);
-        if (g > base && g >= filled && !negative) {
-          // Most jobs fit where the last one was admitted, and neighbours in the order have equal response lengths: up to
-          // GROUP of them are tried together.  (Their old ramps lie outside the ring, those of all later jobs too.)  With N
-          // the plan, job k fits iff N(t + r) + (k + 1) r + sum over the jobs before it of (s + 1) <= M - s_k - 1 for
-          // every r < o: one maximum per job over the same words.  Lane k holds job k's numbers.
-          const int t = base, q0 = t & ~3;
-          int4 c = make_int4(0, 0, 0, 0);
-          if (lane < GROUP && x + lane < m) c = sh_job[half][x + lane];
-          const u32 same = __ballot_sync(0xffffffffu, lane < GROUP && x + lane < m && c.x == o);
-          const int cnt = __ffs(static_cast<int>(~same)) - 1;
-          i64 S = lane < cnt ? static_cast<i64>(c.y) + 1 : 0;          // inclusive sums of s + 1 over the first lanes
-#pragma unroll
-          for (int d = 1; d < GROUP; d <<= 1) {
-            const i64 y = __shfl_up_sync(0xffffffffu, S, d);
-            if (lane >= d) S += y;
-          }
-          const i64 limit = M - S;                                     // M - s_k - 1 - sum before
-          u32 w[8], r[8], mk[GROUP];
-#pragma unroll
-          for (int k = 0; k < GROUP; ++k) mk[k] = 0;
-          const u32 len = static_cast<u32>(o);
-          // the eight words of this lane from round q on; outside the window: r = 0
+        const int t = base;
+        // the jobs that may be tried together, see below
+        const u32 near = __ballot_sync(0xffffffffu, c.x <= min(min(o + (o >> 3) + 32, RING - 4), g - t));
+        const int cnt = min(most_jobs, near == 0xffffffffu ? 32 : __ffs(static_cast<int>(~near)) - 1);
+        const bool alone = cnt == 0;
+        const int o_last = __shfl_sync(0xffffffffu, c.x, max(cnt - 1, 0));
+        if (filled < t + o_last) fill_to(x0 + x, t + o_last, g, o_last);
+        if (g <= t) {                                   // its turn comes at its old start: it stays where it is
+          if (lane == 0) jc[b.w] = g + o;
+          before = static_cast<u32>(b.y);
+          ++x;
+          continue;
+        }
+        if (!negative) {
+          // Most jobs fit where the last one was admitted, and neighbours in the order have about the same response lengths: up to
+          // 32 of them are tried together there, if their old ramps (and so those of all later jobs) begin behind their windows.
+          // With N the plan, the first k fit if N(t + r) + S_k + k r <= M for every r below the k-th's length, S_k the sum of
+          // their s + 1 (exactly then, if their lengths are equal; otherwise the shorter ones are counted beyond their ends, and
+          // those that do not fit so are tried again behind the others).  Memory only grows with k, so many that fit are
+          // found by testing one k, cutting it down to what the worst round leaves, and so on; for k = 1 the test is exact.
+          // A job whose old ramp begins inside its window, G rounds behind t, is tried alone: there the plan loses the old
+          // ramp and gets the new one, which is G more.
+          const int q0 = t & ~3;
+          const u32 G = static_cast<u32>(g - t);
+          const u32 S = static_cast<u32>(c.y) - before;
+          // how many jobs round r leaves room for
+          auto room_at = [&](u32 r) {
+            const u32 used = static_cast<u32>(ring[(t + static_cast<int>(r)) & (RING - 1)]) + static_cast<u32>(lane + 1) * r;
+            return __popc(__ballot_sync(0xffffffffu, lane < cnt && used <= Mu && S <= Mu - used));
+          };
+          const bool once = q0 + 256 >= t + o_last;                    // one step covers the window: its words are read once
+          u32 A, C, len, w[8];
+          // the eight words of this lane from round q on
           auto read = [&](int q) {
             const int4 v0 = *reinterpret_cast<const int4*>(ring + (q & (RING - 1)));
             const int4 v1 = *reinterpret_cast<const int4*>(ring + ((q + 128) & (RING - 1)));
             w[0] = v0.x; w[1] = v0.y; w[2] = v0.z; w[3] = v0.w; w[4] = v1.x; w[5] = v1.y; w[6] = v1.z; w[7] = v1.w;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) r[i] = static_cast<u32>(q - t) + static_cast<u32>(i < 4 ? i : 124 + i);
           };
-          for (int q = q0 + 4 * lane; q - 4 * lane < t + o; q += 256) {
-            read(q);
-            u32 y[8];
+          // f(i, r, what the jobs tried add there) for those of them that lie in the window
+          auto each = [&](int q, auto f) {
+            const u32 r0 = static_cast<u32>(q - t), a0 = A + C * r0;
+            if (!alone) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) { const bool in = r[i] < len; y[i] = in ? w[i] : 0u; r[i] = in ? r[i] : 0u; }
+              for (int i = 0; i < 8; ++i) {
+                const u32 d = static_cast<u32>(i < 4 ? i : 124 + i);
+                if (r0 + d < len) f(i, r0 + d, a0 + C * d);
+              }
+            } else {
 #pragma unroll
-            for (int k = 0; k < GROUP; ++k) {
-              if (k >= cnt) break;
-#pragma unroll
-              for (int i = 0; i < 8; ++i) { y[i] += r[i]; mk[k] = max(mk[k], y[i]); }
+              for (int i = 0; i < 8; ++i) {
+                const u32 d = static_cast<u32>(i < 4 ? i : 124 + i);
+                if (r0 + d < len) f(i, r0 + d, r0 + d < G ? a0 + d : G);
+              }
+            }
+          };
+          if (once) read(q0 + 4 * lane);
+          int k = alone ? 1 : max(1, min(room_at(0u), room_at(static_cast<u32>(o) - 1u)));
+          u32 most, arg = 0;                                           // the worst round and the memory in it
+          for (;;) {
+            A = __shfl_sync(0xffffffffu, S, k - 1);
+            C = static_cast<u32>(k);
+            len = static_cast<u32>(__shfl_sync(0xffffffffu, c.x, k - 1));
+            const int end = t + static_cast<int>(len);
+            u32 top = 0, at = 0;
+            int q_top = q0 + 4 * lane;
+            for (int q = q0 + 4 * lane; q - 4 * lane < end; q += 256) {
+              if (!once) read(q);
+              u32 here = 0;
+              each(q, [&](int i, u32, u32 add) { here = max(here, w[i] + add); });
+              if (here >= top) { top = here; q_top = q; }
+            }
+            most = __reduce_max_sync(0xffffffffu, top);
+            if (most <= Mu) break;
+            if (!once) read(q_top);
+            each(q_top, [&](int i, u32 r, u32 add) { at = w[i] + add == most ? r : at; });
+            arg = __reduce_max_sync(0xffffffffu, at);
+            if (k == 1) { k = 0; break; }
+            k = room_at(arg);
+            if (k == 0) {
+              if (arg >= static_cast<u32>(o)) { k = 1; continue; }     // behind the first one's window
+              most = static_cast<u32>(ring[(t + static_cast<int>(arg)) & (RING - 1)]) + __shfl_sync(0xffffffffu, S, 0) + arg;
+              break;
             }
           }
-          u32 most = 0;
-#pragma unroll
-          for (int k = 0; k < GROUP; ++k) {
-            if (k >= cnt) break;
-            const u32 v = __reduce_max_sync(0xffffffffu, mk[k]);
-            if (lane == k) most = v;
-          }
-          const u32 bad = __ballot_sync(0xffffffffu, lane < cnt && static_cast<i64>(most) > limit);
-          const int fits = bad ? __ffs(static_cast<int>(bad)) - 1 : cnt;
-          if (fits > 0) {
-            const u32 add = static_cast<u32>(__shfl_sync(0xffffffffu, S, fits - 1)), nf = static_cast<u32>(fits);
-            const bool once = q0 + 256 >= t + o;                       // one step covered the window: the words are still here
+          if (k > 0) {
+            const u32 longest = len;
+            len = static_cast<u32>(o);                  // all k of them run for so long
             for (int q = q0 + 4 * lane; q - 4 * lane < t + o; q += 256) {
               if (!once) read(q);
-              else
-#pragma unroll
-                for (int i = 0; i < 8; ++i) r[i] = static_cast<u32>(q - t) + static_cast<u32>(i < 4 ? i : 124 + i);
-#pragma unroll
-              for (int i = 0; i < 8; ++i) w[i] += r[i] < len ? add + nf * r[i] : 0u;
+              each(q, [&](int i, u32, u32 add) { w[i] += add; });
               *reinterpret_cast<int4*>(ring + (q & (RING - 1))) = make_int4(w[0], w[1], w[2], w[3]);
               *reinterpret_cast<int4*>(ring + ((q + 128) & (RING - 1))) = make_int4(w[4], w[5], w[6], w[7]);
             }
-            if (lane < fits) jc[c.w] = t + o;
-            flow += static_cast<i64>(fits) * (t + o);
-            hmax = max(hmax, t + o);
-            x += fits;
             __syncwarp();
+            for (u32 r0 = len; r0 < longest; r0 += 32) {  // then one after the other ends
+              const u32 r = r0 + lane;
+              int ended = 0;                            // of the first k, in order
+#pragma unroll
+              for (int d = 16; d > 0; d >>= 1) {
+                const int v = __shfl_sync(0xffffffffu, c.x, ended + d - 1);
+                if (ended + d < k && static_cast<u32>(v) <= r) ended += d;
+              }
+              const u32 gone = __shfl_sync(0xffffffffu, S, max(ended - 1, 0));
+              if (r < longest) ring[(t + static_cast<int>(r)) & (RING - 1)] += static_cast<int>(A - (ended ? gone : 0u) + (C - static_cast<u32>(ended)) * r);
+            }
+            if (lane < k) jc[c.w] = t + c.x;
+            __syncwarp();
+            // old ramps that are in the ring leave it
+            if (alone) {
+              const int first = static_cast<int>(A) - g;
+              for (int u = t + o + lane; u < min(g + o, filled); u += 32) ring[u & (RING - 1)] -= first + u;
+              __syncwarp();
+            } else if (g < filled) {
+              u32 in = __ballot_sync(0xffffffffu, lane < k && c.z < filled);
+              const u32 left_of = __shfl_up_sync(0xffffffffu, S, 1), s1 = lane > 0 ? S - left_of : S;
+              while (in) {
+                const int src = __ffs(static_cast<int>(in)) - 1;
+                in &= in - 1u;
+                const int gs = __shfl_sync(0xffffffffu, c.z, src), os = __shfl_sync(0xffffffffu, c.x, src);
+                const int first = static_cast<int>(__shfl_sync(0xffffffffu, s1, src));
+                quads<true>(ring, gs, min(gs + os, filled), [&](int rel, int v) { return v - (first + rel); });
+                __syncwarp();
+              }
+            }
+            x += k;
+            before += A;
           } else {
-            // the maximising round: no start before it has passed, or before the plan may be that high
-            const u32 top = __shfl_sync(0xffffffffu, most, 0);
-            int arg = 0;
-            quads<false>(ring, t, t + o, [&](int rel, int v) { if (static_cast<u32>(v) + static_cast<u32>(rel) == top) arg = rel; return 0; });
-            arg = static_cast<int>(__reduce_max_sync(0xffffffffu, static_cast<u32>(arg)));
-            const i64 need = static_cast<i64>(top) - (M - s - 1);
-            advance(static_cast<int>(min_i64(t + min_i64(need, static_cast<i64>(arg) + 1), static_cast<i64>(g))));
+            // no start before that round has passed, or before the plan may be that high
+            advance(static_cast<int>(min_i64(t + min_i64(static_cast<i64>(most) - M, static_cast<i64>(arg) + 1), static_cast<i64>(g))));
           }
           continue;
         }
-        // One job whose old ramp is in the ring (or whose turn has come at its old start): it leaves the ring first.
+        // One job on a plan with words beyond 31 bits: its old ramp leaves the ring first.
+        const int s = static_cast<int>(static_cast<u32>(b.y) - before - 1u), j = b.w, g_next = sh_job[(x0 + x + 1) & 63].z;
         if (g < filled) {
           quads<true>(ring, g, min(g + o, filled), [&](int rel, int v) { return v - (s + rel + 1); });
           __syncwarp();
         }
-        const int g_next = x + 1 < 32 ? sh_job[half][x + 1].z : sh_job[half ^ 1][0].z;
         const i64 bound = M - s - 1;
         int d = g;
         for (;;) {
@@ -258,48 +322,38 @@ __global__ void __launch_bounds__(RT) k_refill(RefillParams p) {
         quads<true>(ring, d, d + o, [&](int rel, int v) { return v + s + rel + 1; });
         __syncwarp();
         if (lane == 0) jc[j] = d + o;
-        flow += d + o;
-        hmax = max(hmax, d + o);
+        before = static_cast<u32>(b.y);
         ++x;
       }
       if (tail) { x0 += x; break; }
+      x -= 32;                                          // jobs of the next 32 that have been taken already
     }
-    // the ring goes back to the plan
-    for (int u = base + lane; u < min(filled, H); u += 32)
-      if (KVS_OK_AT(u, pcap, CHK_RF_PROF_OUT)) prof[u] = ring[u & (RING - 1)];
-    __syncwarp();
     x0 = min(x0, n);
-    if (tail) {
-      // and so that the rest of the plan holds the remaining jobs' old ramps only
-      const int g = js[perm[x0]];
-      for (int u = filled + lane; u < min(g, H); u += 32)
-        if (KVS_OK_AT(u, pcap, CHK_RF_PROF_OUT)) prof[u] = 0;
-      __syncwarp();
-      if (x0 > 0) take_out(x0, max(filled, g), H, Oo[x0 - 1], false);
-    } else {
-      for (int u = filled + lane; u < H; u += 32)
-        if (KVS_OK_AT(u, pcap, CHK_RF_PROF_OUT)) prof[u] = 0;
-    }
-    if (lane == 0) { sh_next = x0; sh_prev = base; sh_hmax = hmax; sh_flow = flow; }
+    if (lane == 0) { sh_next = x0; sh_prev = base; sh_filled = filled; }
   }
   __syncthreads();
+  // the ring goes back to the plan, the rest of which holds the remaining jobs' old ramps only
+  const int next = sh_next, filled = sh_filled;
+  const bool tail = next < n;
+  const int g_next = tail ? js[perm[next]] : H;
+  for (int u = sh_prev + tid; u < min(filled, H); u += RT)
+    if (KVS_OK_AT(u, pcap, CHK_RF_PROF_OUT)) prof[u] = ring[u & (RING - 1)];
+  for (int u = filled + tid; u < min(g_next, H); u += RT)
+    if (KVS_OK_AT(u, pcap, CHK_RF_PROF_OUT)) prof[u] = 0;
+  __syncthreads();
   // ---- jobs that are longer than the ring: the whole CTA, the plan in global memory ----
-  int prev = sh_prev, hmax = sh_hmax;
-  i64 flow = sh_flow;
-  constexpr int U = 4;                                  // loads in flight per thread
-  for (int x = sh_next; x < n; ++x) {
+  int prev = sh_prev;
+  if (tail) {
+    if (tid < 32 && next > 0) take_out(next, max(filled, g_next), H, Oo[next - 1], false);
+    __syncthreads();
+  }
+  constexpr int U = 8;                                  // loads in flight per thread
+  for (int x = next; x < n; ++x) {
     const Job b = load(x);
     const int o = b.o, g = b.g;
-    for (int u0 = tid; u0 < o; u0 += U * RT) {
-      int v[U];
-#pragma unroll
-      for (int i = 0; i < U; ++i) { const int u = u0 + i * RT; v[i] = u < o && KVS_OK_AT(g + u, pcap, CHK_RF_PROF_OUT) ? prof[g + u] : 0; }
-#pragma unroll
-      for (int i = 0; i < U; ++i) { const int u = u0 + i * RT; if (u < o && KVS_OK_AT(g + u, pcap, CHK_RF_PROF_OUT)) prof[g + u] = v[i] - (b.s + u + 1); }
-    }
-    __syncthreads();
     const i64 bound = M - b.s - 1;
     int d = g, t = prev;
+    // the job's own old ramp stays in the plan until its new start is known: it is left out of what is read
     while (t < g) {
       i64 best = -1;
       int arg = t;
@@ -310,7 +364,7 @@ __global__ void __launch_bounds__(RT) k_refill(RefillParams p) {
 #pragma unroll
         for (int i = 0; i < U; ++i) {
           const int u = u0 + i * RT;
-          const i64 r = static_cast<i64>(v[i]) + u;
+          const i64 r = static_cast<i64>(v[i] - (u >= g ? b.s + (u - g) + 1 : 0)) + u;
           if (u < t + o && r >= best) { best = r; arg = u; }
         }
       }
@@ -328,24 +382,50 @@ __global__ void __launch_bounds__(RT) k_refill(RefillParams p) {
       if (best - t <= bound) { d = t; break; }
       t = static_cast<int>(min_i64(best - bound, static_cast<i64>(arg) + 1));
     }
-    for (int u0 = tid; u0 < o; u0 += U * RT) {
-      int v[U];
+    if (d < g) {                                        // out at the old start, in at the new one
+      auto move = [&](int from, int to) {
+        for (int u0 = from + tid; u0 < to; u0 += U * RT) {
+          int v[U];
 #pragma unroll
-      for (int i = 0; i < U; ++i) { const int u = u0 + i * RT; v[i] = u < o && KVS_OK_AT(d + u, pcap, CHK_RF_PROF_IN) ? prof[d + u] : 0; }
+          for (int i = 0; i < U; ++i) { const int u = u0 + i * RT; v[i] = u < to && KVS_OK_AT(u, pcap, CHK_RF_PROF_IN) ? prof[u] : 0; }
 #pragma unroll
-      for (int i = 0; i < U; ++i) { const int u = u0 + i * RT; if (u < o && KVS_OK_AT(d + u, pcap, CHK_RF_PROF_IN)) prof[d + u] = v[i] + b.s + u + 1; }
+          for (int i = 0; i < U; ++i) {
+            const int u = u0 + i * RT;
+            if (u < to && KVS_OK_AT(u, pcap, CHK_RF_PROF_OUT)) prof[u] = v[i] + (u < d + o ? b.s + (u - d) + 1 : 0) - (u >= g ? b.s + (u - g) + 1 : 0);
+          }
+        }
+      };
+      move(d, min(d + o, g));
+      move(g, g + o);
+      __syncthreads();
     }
-    __syncthreads();
     if (tid == 0) jc[b.j] = d + o;
-    flow += d + o;
-    hmax = max(hmax, d + o);
     prev = d;
   }
   __syncthreads();
-  // the starts: completion less response, both by position now
-  for (int x = tid; x < n; x += RT) { const int j = perm[x]; if (KVS_OK_AT(j, n, CHK_RF_JOB)) js[j] = jc[j] - Oo[x]; }
-  i64 peak = 0;
-  for (int u = tid; u < hmax; u += RT) peak = max_i64(peak, prof[u]);
+  // the starts: completion less response, both by position now; flow and horizon
+  i64 flow = 0;
+  int hmax = 0;
+  for (int x0 = tid; x0 < n; x0 += U * RT) {
+    int j[U], v[U];
+#pragma unroll
+    for (int i = 0; i < U; ++i) { const int x = x0 + i * RT; j[i] = x < n ? perm[x] : 0; v[i] = x < n ? Oo[x] : 0; }
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      const int end = x0 + i * RT < n && KVS_OK_AT(j[i], n, CHK_RF_JOB) ? jc[j[i]] : 0;
+      flow += end;
+      hmax = max(hmax, end);
+      v[i] = end - v[i];
+    }
+#pragma unroll
+    for (int i = 0; i < U; ++i) if (x0 + i * RT < n && KVS_OK_AT(j[i], n, CHK_RF_JOB)) js[j[i]] = v[i];
+  }
+  flow = block_sum(flow, sh_sum);
+  hmax = block_max(hmax, sh_max, 0);
+  int most = 0;
+#pragma unroll 8
+  for (int u = tid; u < hmax; u += RT) most = max(most, prof[u]);
+  i64 peak = most;
   peak = block_max(peak, sh_peak, static_cast<i64>(0));
   if (tid == 0) {
     if (p.peak) p.peak[e] = peak;

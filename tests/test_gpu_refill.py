@@ -77,3 +77,24 @@ def test_edges_of_the_ring(par, o_max):
     inst = workloads.Instances(torch.tensor([0, o.numel()]), s, o)
     rows = [dict(instance=0, family="GBAD", M=M) for M in (o_max + 50, o_max + 51, 2 * o_max + 100, 5 * o_max, 1 << 18)]
     par.check_batch(inst, binding.make_settings(rows), want_runs=False, label=f"refill ring {o_max}")
+
+
+@pytest.mark.parametrize("n, lo, hi, s_max", [(200, 250, 262, 40), (150, 1, 4, 3), (300, 60, 90, 600), (70, 4_050, 4_140, 50), (129, 500, 640, 0), (33, 1_000, 9_000, 20)])
+def test_jobs_tried_together(par, n, lo, hi, s_max):
+    """Windows of one step of 256 rounds and of several, at the ring's length and beyond it, lengths that are equal, close and far apart,
+    old ramps inside a job's own window, in the ring and behind it; budgets that few, some and all jobs fit."""
+    c = torch.arange(n)
+    inst = workloads.Instances(torch.tensor([0, n]), workloads.uniform_int(91, c, 0, s_max), workloads.uniform_int(92, c, lo, hi))
+    area = (hi + s_max) * n
+    Ms = [hi + s_max + 1, 3 * (hi + s_max), area // 8 + hi + s_max, area // 2 + hi, 2 * area + hi]
+    # the sums of 32 prompts beyond 2^32, and budgets that the 32-bit short cuts do not cover
+    Ms += [(1 << 28) + 1, (1 << 31) - (1 << 20), (1 << 31) - (1 << 20) + 1, (1 << 31) - 1]
+    par.check_batch(inst, binding.settings_grid(range(1), ["GBAD"], Ms), want_runs=False, label=f"refill together {lo}..{hi}")
+
+
+def test_long_prompts_tried_together(par):
+    """Prompts of which 32 do not add up in 32 bits."""
+    n = 90
+    c = torch.arange(n)
+    inst = workloads.Instances(torch.tensor([0, n]), workloads.uniform_int(93, c, 1 << 27, 1 << 28), workloads.uniform_int(94, c, 20, 30))
+    par.check_batch(inst, binding.settings_grid(range(1), ["GBAD"], [(1 << 28) + 100, (1 << 30) + 5, (1 << 31) - (1 << 20), (1 << 31) - 2]), want_runs=False, label="refill long prompts")
