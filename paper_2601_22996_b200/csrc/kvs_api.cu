@@ -511,6 +511,7 @@ int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* se
   bp.settings = settings_dev;
   bp.fill = ctx->fill ? 1 : 0; bp.fill_job = ctx->fill_job; bp.fill_prof = ctx->fill_prof;
   bp.parts = 1;
+  for (int64_t e = 0; e < P && !bp.variants; ++e) bp.variants = settings[e].subroutine || settings[e].per_class_s;
   bp.P = P; bp.out = o; bp.ev = v; bp.do_profile = do_profile;
   auto grid_for = [&](int ctas_per_sm, int64_t most) {
     int64_t g = static_cast<int64_t>(ctx->sm_count) * ctas_per_sm;

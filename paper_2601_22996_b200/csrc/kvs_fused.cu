@@ -1084,7 +1084,13 @@ struct FAcc {
 // other, calls with estimates lost a tenth to spills); a family id (KVS_GBA .. KVS_SIMS) gives the kernel compiled
 // for that family on exact response lengths only (the caller lists nothing else for it), so that
 // each keeps just its own paths and gets its own register allocation.
-template <bool LIGHT, int FAM>
+// VARIANTS: with the code for simultaneous batches and per-phase prompt lengths.  The full batching kernel never has it (the light one
+// takes those, or leaves them to the general kernel): 176 bytes of spills a thread with it, 12 without, 4,096 evaluations of 50,000
+// jobs with their profiles 4.03 and 3.36 ms.  The kernel for shared evaluations exists with it, without it, and without it for calls
+// with estimates (spill loads a thread 2,932, 2,248 and 1,840 bytes; one kernel for all three: 3,568): 64 instances of 50,000 jobs
+// in windows 1,432 -> 1,270 us, four evaluations of 1,000 jobs 177 -> 170, 64 initial slices 429 -> 406.  The slicing
+// kernel spills no less without it.
+template <bool LIGHT, int FAM, bool VARIANTS>
 __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 1 : KVS_EVAL_MIN_CTAS) k_fused_eval(BuildParams p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FShared& sh = *reinterpret_cast<FShared*>(smem_raw);
@@ -1117,7 +1123,7 @@ __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 
     // A call with few evaluations shares each of them between `parts` CTAs: all of them form the plan (its scratch is
     // the CTA's own), each takes a share of the job results and, since the phases' rounds are disjoint, walks a range of
     // phases of about equal cost; the CTA that finishes last writes the scalars.
-    constexpr bool SHARED = FAM == KVS_FUSED_SHARED;
+    constexpr bool SHARED = FAM == KVS_FUSED_SHARED || FAM == KVS_FUSED_SHARED_EST;
     const int all_parts = SHARED ? p.parts : 1;
     const int my_part = SHARED ? static_cast<int>(sh.next_eval % all_parts) : 0;
     const i64 slot_no = SHARED ? sh.next_eval / all_parts : sh.next_eval;
@@ -1133,13 +1139,10 @@ __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 
     const int family = FAM < 0 ? st.family : FAM;
     const bool geometric = family == KVS_GBA || family == KVS_GSA;
     const bool sim = family == KVS_SIMS;
-    // The full batching kernel gets no variants (the light one takes those, or leaves them to the general kernel): with the code for
-    // them it spilled 176 bytes a thread, now 12 (4,096 batching evaluations of 50,000 jobs with their profiles 4.03 -> 3.36 ms).
-    constexpr bool VARIANTS = LIGHT || FAM != KVS_GBA;
     const bool batches = VARIANTS && geometric && st.subroutine == 1;      // simultaneous batches inside the phases
     const bool per_class = VARIANTS && geometric && st.per_class_s == 1;   // parallelism from the longest prompt of a phase
     const bool slots = sim || batches;                         // runs start together, k of them at a time
-    const bool est = FAM < 0 && p.key != nullptr;
+    const bool est = FAM == KVS_FUSED_SHARED_EST || (FAM == KVS_FUSED_ANY && p.key != nullptr);
     const bool keyed = !(family == KVS_GSA && !est);          // plain GSA keeps the index order
     const bool carry = geometric && (family == KVS_GSA || est);
     const bool est_class = est && family == KVS_GBA;          // classes by the clipped estimate
@@ -1157,7 +1160,7 @@ __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 
     const i64 prof_base = p.ev.profile_off ? p.ev.profile_off[e] : 0;
     const i64 prof_cap = (p.ev.profile && p.ev.profile_off) ? p.ev.profile_off[e + 1] - prof_base : 0;
     int32_t* const prof = p.ev.profile ? p.ev.profile + prof_base : nullptr;
-    if ((batches || per_class) && (est || (p.do_profile && prof_cap > 0))) {
+    if (geometric && (st.subroutine == 1 || st.per_class_s == 1) && (!VARIANTS || est || (p.do_profile && prof_cap > 0))) {
       // these variants on estimates, and their profiles, are the general kernel's
       if (tid == 0 && my_part == 0) p.slow_list[atomicAdd(p.slow_count, 1ull)] = e;
       continue;
@@ -1996,11 +1999,11 @@ __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 
 
 static size_t fused_smem_bytes(bool light) { return light ? offsetof(FShared, dA) : sizeof(FShared); }
 
-template <bool LIGHT, int FAM>
+template <bool LIGHT, int FAM, bool VARIANTS>
 static int ctas_per_sm() {
   int n = 0;
-  cudaFuncSetAttribute(k_fused_eval<LIGHT, FAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(fused_smem_bytes(LIGHT)));
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused_eval<LIGHT, FAM>, KVS_EVAL_THREADS, fused_smem_bytes(LIGHT)) != cudaSuccess) n = 1;
+  cudaFuncSetAttribute(k_fused_eval<LIGHT, FAM, VARIANTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(fused_smem_bytes(LIGHT)));
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused_eval<LIGHT, FAM, VARIANTS>, KVS_EVAL_THREADS, fused_smem_bytes(LIGHT)) != cudaSuccess) n = 1;
   return n < 1 ? 1 : n;
 }
 
@@ -2008,17 +2011,18 @@ static int ctas_per_sm() {
 int kvs_fused_ctas_per_sm(int light) {
   int n;
   if (light) {
-    n = ctas_per_sm<true, KVS_FUSED_ANY>();
-    n = min(n, min(min(ctas_per_sm<true, KVS_GBA>(), ctas_per_sm<true, KVS_GSA>()), min(ctas_per_sm<true, KVS_SPS>(), ctas_per_sm<true, KVS_SIMS>())));
+    n = ctas_per_sm<true, KVS_FUSED_ANY, true>();
+    n = min(n, min(min(ctas_per_sm<true, KVS_GBA, true>(), ctas_per_sm<true, KVS_GSA, true>()), min(ctas_per_sm<true, KVS_SPS, true>(), ctas_per_sm<true, KVS_SIMS, true>())));
   } else {
-    n = min(min(ctas_per_sm<false, KVS_FUSED_ANY>(), ctas_per_sm<false, KVS_FUSED_SHARED>()), min(ctas_per_sm<false, KVS_GBA>(), ctas_per_sm<false, KVS_GSA>()));
+    n = min(ctas_per_sm<false, KVS_FUSED_ANY, true>(), min(ctas_per_sm<false, KVS_GBA, false>(), ctas_per_sm<false, KVS_GSA, true>()));
+    n = min(n, min(min(ctas_per_sm<false, KVS_FUSED_SHARED, false>(), ctas_per_sm<false, KVS_FUSED_SHARED, true>()), ctas_per_sm<false, KVS_FUSED_SHARED_EST, false>()));
   }
   return n;
 }
 
-template <bool LIGHT, int FAM>
+template <bool LIGHT, int FAM, bool VARIANTS>
 static cudaError_t launch(const BuildParams& p, int grid, cudaStream_t stream) {
-  k_fused_eval<LIGHT, FAM><<<grid, KVS_EVAL_THREADS, fused_smem_bytes(LIGHT), stream>>>(p);
+  k_fused_eval<LIGHT, FAM, VARIANTS><<<grid, KVS_EVAL_THREADS, fused_smem_bytes(LIGHT), stream>>>(p);
   return cudaGetLastError();
 }
 
@@ -2029,17 +2033,18 @@ cudaError_t kvs_launch_fused(const BuildParams& p, int grid, int light, int fam,
   if (p.P <= 0) return cudaSuccess;
   if (light) {
     switch (fam) {
-      case KVS_GBA: return launch<true, KVS_GBA>(p, grid, stream);
-      case KVS_GSA: return launch<true, KVS_GSA>(p, grid, stream);
-      case KVS_SPS: return launch<true, KVS_SPS>(p, grid, stream);
-      case KVS_SIMS: return launch<true, KVS_SIMS>(p, grid, stream);
-      default: return launch<true, KVS_FUSED_ANY>(p, grid, stream);
+      case KVS_GBA: return launch<true, KVS_GBA, true>(p, grid, stream);
+      case KVS_GSA: return launch<true, KVS_GSA, true>(p, grid, stream);
+      case KVS_SPS: return launch<true, KVS_SPS, true>(p, grid, stream);
+      case KVS_SIMS: return launch<true, KVS_SIMS, true>(p, grid, stream);
+      default: return launch<true, KVS_FUSED_ANY, true>(p, grid, stream);
     }
   }
-  if (fam == KVS_GBA) return launch<false, KVS_GBA>(p, grid, stream);
-  if (fam == KVS_GSA) return launch<false, KVS_GSA>(p, grid, stream);
-  if (fam == KVS_FUSED_SHARED) return launch<false, KVS_FUSED_SHARED>(p, grid, stream);
-  return launch<false, KVS_FUSED_ANY>(p, grid, stream);
+  if (fam == KVS_GBA) return launch<false, KVS_GBA, false>(p, grid, stream);
+  if (fam == KVS_GSA) return launch<false, KVS_GSA, true>(p, grid, stream);
+  if (fam == KVS_FUSED_SHARED && p.key) return launch<false, KVS_FUSED_SHARED_EST, false>(p, grid, stream);
+  if (fam == KVS_FUSED_SHARED) return p.variants ? launch<false, KVS_FUSED_SHARED, true>(p, grid, stream) : launch<false, KVS_FUSED_SHARED, false>(p, grid, stream);
+  return launch<false, KVS_FUSED_ANY, true>(p, grid, stream);
 }
 
 // First violation recorded by the checked build (0 = none); `compiled` = 1 if this library was built with

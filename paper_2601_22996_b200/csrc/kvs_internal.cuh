@@ -88,6 +88,7 @@ struct BuildParams {
   int32_t fill_job, fill_prof;
   // the kernel for any family may give every evaluation of its list to `parts` CTAs (shares: one entry per list entry)
   int parts;
+  int variants;             // some evaluation runs simultaneous batches or sizes its phases by their own prompts
   FusedShare* shares;
 };
 
@@ -197,7 +198,7 @@ cudaError_t kvs_launch_sort(const SortParams& p, int capacity, cudaStream_t stre
 cudaError_t kvs_launch_build(const BuildParams& p, int grid, cudaStream_t stream);
 int kvs_build_ctas_per_sm();
 // Instantiations of the fast kernel for any family, with one CTA per evaluation and with several; the others are named by the family id
-enum { KVS_FUSED_ANY = -1, KVS_FUSED_SHARED = -2 };
+enum { KVS_FUSED_ANY = -1, KVS_FUSED_SHARED = -2, KVS_FUSED_SHARED_EST = -3 };   // the last: of a call with estimates, chosen by the launch
 cudaError_t kvs_launch_fused(const BuildParams& p, int grid, int light, int fam, cudaStream_t stream);
 int kvs_fused_ctas_per_sm(int light);
 cudaError_t kvs_fused_check_word(unsigned long long* word, int* compiled, int reset);

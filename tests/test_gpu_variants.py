@@ -155,3 +155,23 @@ def test_variants_with_and_without_profile_in_one_call(par, copies):
         if S.status == 0:
             E = oracle.evaluate_dense(S.run_start, S.run_len, S.run_s, want_profile=False)
             assert (int(some.peak[e]), int(some.flow[e])) == (E.peak, S.flow), rows[e]
+
+
+@pytest.mark.parametrize("want_profile", [True, False])
+@pytest.mark.parametrize("kind", ["plain", "one variant", "estimates", "estimates and windows"])
+def test_shared_evaluations_by_kernel(par, kind, want_profile):
+    """Calls of few evaluations, each of which several CTAs share: without variants, with one among plain evaluations, on estimates."""
+    est = kind.startswith("estimates")
+    inst = workloads.random_small(4300, 5, 700, 60, 200, with_est=est)
+    window = 0
+    if kind == "estimates and windows":
+        off = inst.job_off
+        inst.arrival = torch.cat([torch.arange(int(off[i + 1] - off[i])) * 2 for i in range(inst.n_instances)])
+        window = 151
+    rows = []
+    for i in range(inst.n_instances):
+        for fam in ("GBA", "GSA", "SPS", "SIMS"):
+            rows.append(dict(instance=i, family=fam, M=2_000 + 900 * i))
+    if kind == "one variant":
+        rows[5].update(subroutine=1, per_class_s=1)
+    par.check_batch(inst, binding.make_settings(rows), window=window, want_runs=False, want_profile=want_profile, label=f"shared {kind}")
