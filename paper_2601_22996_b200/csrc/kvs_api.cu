@@ -497,7 +497,7 @@ int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* se
   if (!beside && lane >= 0 && (ce = close_side(side, stream)) != cudaSuccess) return fail_cuda(ctx, ce, "stream ordering");
 
   if (ctx->timing && !rg) cudaEventRecord(ctx->ev[0], ctx->stream);
-  ce = kvs_launch_sort(sp, ctx->sm_count * 2, stream);
+  ce = kvs_launch_sort(sp, ctx->sm_count * KVS_SORT_CTAS, stream);
   if (ce != cudaSuccess) return fail_cuda(ctx, ce, "sort launch");
   if (ctx->timing && !rg) cudaEventRecord(ctx->ev[1], ctx->stream);
 

@@ -12,7 +12,9 @@ typedef unsigned long long ull;   // the type CUDA's 64-bit atomics are declared
 typedef unsigned int u32;
 
 constexpr int KVS_MAX_PHASES = 96;      // slices of one geometric ladder
-constexpr int KVS_SORT_THREADS = 1024;  // one CTA sorts one (instance, window) segment at a time
+constexpr int KVS_SORT_THREADS = 512;    // one CTA sorts one (instance, window) segment at a time
+constexpr int KVS_SORT_ITEMS = 4;        // jobs per thread and tile
+constexpr int KVS_SORT_CTAS = 2;            // CTAs per SM
 #ifndef KVS_EVAL_THREADS_CFG
 #define KVS_EVAL_THREADS_CFG 512
 #define KVS_EVAL_ITEMS_CFG 8

@@ -6,20 +6,46 @@
 // (ties keep the original index order) is what makes the order unique, so that the per-job
 // results agree bit for bit with a stable comparison sort.
 //
-// Each pass ranks one tile of 1024 jobs at a time: lanes with equal digits find each other with
-// a warp match, per-warp digit counts go to shared memory, one column scan per digit turns them
-// into offsets behind the running bucket position.  Only 4 bytes per job move per pass: the
-// index, together with the key in the upper half of the word when both fit 16 bits; otherwise the
-// next pass re-reads the key through the index.
+// Each pass ranks one tile of KVS_SORT_TILE jobs at a time.  A warp takes 32 * ITEMS consecutive ones, row by row: lanes with equal
+// digits find each other with a warp match and stand behind what the warp has counted so far of their digit in its row of counters
+// in shared memory; one column scan per tile, eight counters a thread, turns the counters into offsets behind the running
+// bucket position.  Two block barriers per tile.  Only 4 bytes per job move per pass: the index, together with the key in the
+// upper half of the word when both fit 16 bits; otherwise the next pass re-reads the key through the index.
+//
+// What bounds it: latencies - of the loads (DRAM and L2), of the match chains and at the barriers - and the scattered 4-byte stores, not
+// bandwidth (32 bytes a job must move, some 60 do).  More instances in flight do not help, their arrays leave the L2: 2,048 instances of
+// 50,000 jobs take 3.04 ms with two CTAs of 512 threads and four jobs a thread and tile per SM, 3.75 with four of them, 3.9 with three and
+// eight jobs a thread, 3.4 with one of 1,024 threads (two of 1,024 threads and one job a thread and tile: 3.42).
 #include "kvs_internal.cuh"
 
 namespace {
 
 constexpr int T = KVS_SORT_THREADS;
 constexpr int WARPS = T / 32;
+constexpr int ITEMS = KVS_SORT_ITEMS;
+constexpr int TILE_N = T * ITEMS;
+constexpr int PER_DIGIT = T / 256;                       // threads that scan the column of one digit
+constexpr int ROWS = WARPS / PER_DIGIT;                  // counters each of them takes
+// Words per row of counters: the PER_DIGIT threads of a digit and those of its neighbours fall into different banks.
+constexpr int ROW_W = 256 + (PER_DIGIT == 4 ? 1 : 2);
+static_assert(PER_DIGIT >= 1 && PER_DIGIT <= 4 && ROWS == 8, "column scan");
 
 __device__ __forceinline__ int32_t key_at(const SortParams& p, i64 lo, int idx) {
   return p.key ? p.key[lo + idx] : p.o[lo + idx];
+}
+
+// Counts the digits of a key; most keys have 0 as their second digit and above (of a warp's keys one addition books them).
+__device__ __forceinline__ void count_digits(u32 (*hist)[256], u32 key, bool valid, int first, int passes) {
+  for (int d = first; d < passes; ++d) {
+    const u32 digit = (key >> (8 * d)) & 255u;
+    if (d == 0) {
+      if (valid) atomicAdd(&hist[0][digit], 1u);
+    } else {
+      const u32 zeros = __ballot_sync(0xffffffffu, valid && digit == 0);
+      if (lane_id() == 0 && zeros) atomicAdd(&hist[d][0], static_cast<u32>(__popc(zeros)));
+      if (valid && digit != 0) atomicAdd(&hist[d][digit], 1u);
+    }
+  }
 }
 
 // Sort positions [seg_lo, seg_hi) of the instance starting at global job index lo.  The last pass
@@ -28,9 +54,10 @@ __device__ __forceinline__ int32_t key_at(const SortParams& p, i64 lo, int idx) 
 // whether it did.
 // packed: indices and keys are below 2^16, so a pass that is not the last stores (key << 16 | index)
 // and the next pass needs no look-up of the key through the index.
-__device__ bool sort_segment(const SortParams& p, i64 lo, int seg_lo, int seg_hi, int passes, bool packed,
-                             u32 (*warp_cnt)[256], u32 (*warp_off)[256], u32 (*hist)[256]) {
-  const int tid = threadIdx.x, warp = tid >> 5;
+// counted: hist holds the counts of the first that many digits.
+__device__ __forceinline__ bool sort_segment(const SortParams& p, i64 lo, int seg_lo, int seg_hi, int passes, bool packed, int counted,
+                             u32* counters, u32 (*hist)[256]) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
   const int n = seg_hi - seg_lo;
   int32_t* const out = p.perm + lo + seg_lo;
   if (passes == 0 || n <= 1) {
@@ -38,26 +65,24 @@ __device__ bool sort_segment(const SortParams& p, i64 lo, int seg_lo, int seg_hi
     __syncthreads();
     return false;
   }
-  // digit histograms of all passes in one sweep
-  for (int i = tid; i < 4 * 256; i += T) (&hist[0][0])[i] = 0;
-  for (int i = tid; i < WARPS * 256; i += T) (&warp_cnt[0][0])[i] = 0;   // stays zero between tiles, see below
-  __syncthreads();
-  for (int j = tid; j < n; j += T) {
-    u32 key = static_cast<u32>(key_at(p, lo, seg_lo + j));
-    for (int d = 0; d < passes; ++d) atomicAdd(&hist[d][(key >> (8 * d)) & 255u], 1u);
+  // digit histograms of the passes that are not counted yet, in one sweep
+  u32* const row = counters + warp * ROW_W;
+  for (int d = lane; d < 256; d += 32) row[d] = 0;         // stays zero between tiles, see below
+  if (counted < passes) {
+    for (int i = tid + counted * 256; i < passes * 256; i += T) (&hist[0][0])[i] = 0;
+    __syncthreads();
+    for (int j0 = 0; j0 < n; j0 += T) {
+      const int j = j0 + tid;
+      count_digits(hist, j < n ? static_cast<u32>(key_at(p, lo, seg_lo + j)) : 0u, j < n, counted, passes);
+    }
   }
   __syncthreads();
   // exclusive scan of each histogram: warp d scans histogram d, 8 digits per lane
   if (warp < passes) {
     u32 v[8], sum = 0;
-    for (int i = 0; i < 8; ++i) { v[i] = hist[warp][lane_id() * 8 + i]; sum += v[i]; }
-    u32 incl = sum;
-    for (int d = 1; d < 32; d <<= 1) {
-      u32 y = __shfl_up_sync(0xffffffffu, incl, d);
-      if (static_cast<int>(lane_id()) >= d) incl += y;
-    }
-    u32 run = incl - sum;
-    for (int i = 0; i < 8; ++i) { hist[warp][lane_id() * 8 + i] = run; run += v[i]; }
+    for (int i = 0; i < 8; ++i) { v[i] = hist[warp][lane * 8 + i]; sum += v[i]; }
+    u32 run = warp_incl(sum) - sum;
+    for (int i = 0; i < 8; ++i) { hist[warp][lane * 8 + i] = run; run += v[i]; }
   }
   __syncthreads();
 
@@ -67,43 +92,73 @@ __device__ bool sort_segment(const SortParams& p, i64 lo, int seg_lo, int seg_hi
     int32_t* dst = (to_perm ? p.perm : p.perm_tmp) + lo + seg_lo;
     const int32_t* src = (to_perm ? p.perm_tmp : p.perm) + lo + seg_lo;
     int32_t* const key_dst = pass == passes - 1 ? (p.key ? p.sorted_key : p.sorted_o) + lo + seg_lo : nullptr;
-    u32 bucket = tid < 256 ? hist[pass][tid] : 0u;   // thread d keeps the running position of digit d
-    for (int j0 = 0; j0 < n; j0 += T) {
-      // Two barriers per tile: the counts are written before the first and read before the second;
-      // the offsets are written between them and read after the second (and not overwritten
-      // before the first barrier of the next tile, which every thread reaches only after its store).
-      // The lane that wrote a count clears it after the second barrier.
-      const int j = j0 + tid;
-      const bool valid = j < n;
-      int idx = 0;
-      u32 key = 0, digit = 256;  // sentinel for lanes past the end
-      if (valid) {
-        if (pass == 0) { idx = seg_lo + j; key = static_cast<u32>(key_at(p, lo, idx)); }
-        else if (packed) { const u32 rec = static_cast<u32>(src[j]); idx = static_cast<int>(rec & 0xffffu); key = rec >> 16; }
-        else { idx = src[j]; key = static_cast<u32>(key_at(p, lo, idx)); }
-        digit = (key >> (8 * pass)) & 255u;
-      }
-      const u32 peers = __match_any_sync(0xffffffffu, digit);
-      const u32 rank = __popc(peers & lanemask_lt());
-      const bool leader = valid && rank == 0;
-      if (leader) warp_cnt[warp][digit] = __popc(peers);
-      __syncthreads();
-      if (tid < 256) {
-        u32 acc = bucket;
+    const int shift = 8 * pass;
+    for (int j0 = 0; j0 < n; j0 += TILE_N) {
+      const int jw = j0 + warp * (32 * ITEMS) + lane;
+      int idx[ITEMS];
+      u32 key[ITEMS], rank[ITEMS];
 #pragma unroll
-        for (int w = 0; w < WARPS; ++w) {
-          warp_off[w][tid] = acc;
-          acc += warp_cnt[w][tid];
+      for (int i = 0; i < ITEMS; ++i) {
+        const int j = jw + 32 * i;
+        idx[i] = seg_lo + j;
+        key[i] = 0;
+        if (j < n) {
+          if (pass == 0) key[i] = static_cast<u32>(key_at(p, lo, idx[i]));
+          else idx[i] = src[j];
         }
-        bucket = acc;
+      }
+      if (pass > 0) {
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+          if (packed) { key[i] = static_cast<u32>(idx[i]) >> 16; idx[i] &= 0xffff; }
+          else if (jw + 32 * i < n) key[i] = static_cast<u32>(key_at(p, lo, idx[i]));
+        }
+      }
+      // rank among the warp's jobs of the same digit, in order
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) {
+        const bool valid = jw + 32 * i < n;
+        const u32 digit = valid ? (key[i] >> shift) & 255u : 256u;     // jobs past the end keep to themselves
+        const u32 peers = __match_any_sync(0xffffffffu, digit);
+        const u32 below = __popc(peers & lanemask_lt());
+        const u32 before = valid ? row[digit] : 0u;
+        rank[i] = before + below;
+        __syncwarp();
+        if (valid && below == 0) row[digit] = before + __popc(peers);
+        __syncwarp();
       }
       __syncthreads();
-      if (valid) {
-        const u32 pos = warp_off[warp][digit] + rank;
-        dst[pos] = (packed && !key_dst) ? static_cast<int32_t>(key << 16 | static_cast<u32>(idx)) : idx;
-        if (key_dst) key_dst[pos] = static_cast<int32_t>(key);
+      {
+        const int digit = tid / PER_DIGIT, part = tid % PER_DIGIT;
+        u32* const column = counters + part * ROWS * ROW_W + digit;
+        u32 c[ROWS], sum = 0;
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) { c[i] = column[i * ROW_W]; sum += c[i]; }
+        u32 incl = sum;
+#pragma unroll
+        for (int d = 1; d < PER_DIGIT; d <<= 1) {
+          const u32 y = __shfl_up_sync(0xffffffffu, incl, d);
+          if (part >= d) incl += y;
+        }
+        u32 at = hist[pass][digit] + incl - sum;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) { column[i * ROW_W] = at; at += c[i]; }
+        if (part == PER_DIGIT - 1) hist[pass][digit] = at;               // running position of the digit
       }
-      if (leader) warp_cnt[warp][digit] = 0;
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) {
+        if (jw + 32 * i < n) {
+          const u32 pos = row[(key[i] >> shift) & 255u] + rank[i];
+          dst[pos] = (packed && !key_dst) ? static_cast<int32_t>(key[i] << 16 | static_cast<u32>(idx[i])) : idx[i];
+          if (key_dst) key_dst[pos] = static_cast<int32_t>(key[i]);
+        }
+      }
+      // the row is the warp's own again until the next tile's barrier
+      __syncwarp();
+#pragma unroll
+      for (int d = 0; d < 8; ++d) row[32 * d + lane] = 0;
       __syncwarp();
     }
     __syncthreads();   // the next pass reads what this one stored
@@ -111,15 +166,13 @@ __device__ bool sort_segment(const SortParams& p, i64 lo, int seg_lo, int seg_hi
   return true;
 }
 
-__global__ void __launch_bounds__(KVS_SORT_THREADS) k_stats_sort(SortParams p) {
-  extern __shared__ __align__(16) u32 dyn[];
-  u32 (*const warp_cnt)[256] = reinterpret_cast<u32 (*)[256]>(dyn);
-  u32 (*const warp_off)[256] = reinterpret_cast<u32 (*)[256]>(dyn + WARPS * 256);
+__global__ void __launch_bounds__(KVS_SORT_THREADS, KVS_SORT_CTAS) k_stats_sort(SortParams p) {
+  extern __shared__ __align__(16) u32 counters[];
   __shared__ u32 hist[4][256];
   __shared__ int red[32];
   __shared__ i64 wsum[32];
   __shared__ int seg_end;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
 
   // Windows are ordered independently: a batch of few instances with windows gives each of them to several CTAs (parts), which
   // take its windows in turn; each forms the statistics it needs by itself.
@@ -131,14 +184,35 @@ __global__ void __launch_bounds__(KVS_SORT_THREADS) k_stats_sort(SortParams p) {
     int flags = 0;
     if (hi < lo || hi - lo > p.max_jobs) flags = KVS_EVAL_BAD_INPUT;
     const int n = flags ? 0 : static_cast<int>(hi - lo);
+    // an instance that is ordered as a whole has the first two digits of its keys counted on the way
+    const bool windows = p.window > 0 && p.arrival;
+    const bool count = p.need_order && !windows;
+    if (count) {
+      __syncthreads();
+      for (int i = tid; i < 512; i += T) (&hist[0][0])[i] = 0;
+      __syncthreads();
+    }
     int s_max = 0, o_max = 0, key_max = 0, bad = 0;
-    for (int j = tid; j < n; j += T) {
-      const int sv = p.s[lo + j], ov = p.o[lo + j], kv = key_at(p, lo, j);
-      s_max = max(s_max, sv); o_max = max(o_max, ov); key_max = max(key_max, kv);
-      bad |= (sv < 0) | (ov < 1) | (kv < 1);
-      if (p.arrival) {
-        const i64 a = p.arrival[lo + j];
-        bad |= (a < 0) | (j > 0 && p.arrival[lo + j - 1] > a);
+    constexpr int U = 4;
+    for (int j0 = 0; j0 < n; j0 += U * T) {
+      int sv[U], ov[U], kv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + u * T + tid;
+        sv[u] = j < n ? p.s[lo + j] : 0;
+        ov[u] = j < n ? p.o[lo + j] : 1;
+        kv[u] = p.key && j < n ? p.key[lo + j] : ov[u];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + u * T + tid;
+        if (j < n) { s_max = max(s_max, sv[u]); o_max = max(o_max, ov[u]); key_max = max(key_max, kv[u]); }
+        bad |= (sv[u] < 0) | (ov[u] < 1) | (kv[u] < 1);
+        if (count) count_digits(hist, static_cast<u32>(kv[u]), j < n, 0, 2);
+        if (p.arrival && j < n) {
+          const i64 a = p.arrival[lo + j];
+          bad |= (a < 0) | (j > 0 && p.arrival[lo + j - 1] > a);
+        }
       }
     }
     s_max = block_max(s_max, red, 0);
@@ -153,7 +227,7 @@ __global__ void __launch_bounds__(KVS_SORT_THREADS) k_stats_sort(SortParams p) {
     int seg_lo = 0;
     for (int w = 0; seg_lo < n; ++w) {
       if (tid < 32) {
-        const int end = p.window > 0 && p.arrival ? window_end(p.arrival + lo, seg_lo, n, p.window) : n;
+        const int end = windows ? window_end(p.arrival + lo, seg_lo, n, p.window) : n;
         if (tid == 0) seg_end = end;
       }
       __syncthreads();
@@ -163,18 +237,29 @@ __global__ void __launch_bounds__(KVS_SORT_THREADS) k_stats_sort(SortParams p) {
         seg_lo = seg_hi;
         continue;
       }
-      const bool have_key = sort_segment(p, lo, seg_lo, seg_hi, passes, n <= 65536 && key_max < 65536, warp_cnt, warp_off, hist);
+      const bool have_key = sort_segment(p, lo, seg_lo, seg_hi, passes, n <= 65536 && key_max < 65536, count ? min(passes, 2) : 0, counters, hist);
       __syncthreads();
-      for (int j = seg_lo + tid; j < seg_hi; j += T) {
-        const int idx = p.perm[lo + j];
-        __stcs(&p.sorted_s[lo + j], p.s[lo + idx]);     // streaming stores: read back much later, by another kernel
-        if (p.key) {
-          __stcs(&p.sorted_o[lo + j], p.o[lo + idx]);
-          if (!have_key) __stcs(&p.sorted_key[lo + j], p.key[lo + idx]);
-        } else if (!have_key) {
-          __stcs(&p.sorted_o[lo + j], p.o[lo + idx]);
+      for (int j0 = seg_lo + tid; j0 < seg_hi; j0 += U * T) {
+        int idx[U], sv[U], ov[U], kv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) idx[u] = j0 + u * T < seg_hi ? p.perm[lo + j0 + u * T] : seg_lo;
+        // streaming stores: read back much later, by another kernel
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          sv[u] = p.s[lo + idx[u]];
+          ov[u] = p.key || !have_key ? p.o[lo + idx[u]] : 0;
+          kv[u] = p.key && !have_key ? p.key[lo + idx[u]] : 0;
         }
-        if (p.iperm) p.iperm[lo + idx] = j;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int j = j0 + u * T;
+          if (j < seg_hi) {
+            __stcs(&p.sorted_s[lo + j], sv[u]);
+            if (p.key || !have_key) __stcs(&p.sorted_o[lo + j], ov[u]);
+            if (p.key && !have_key) __stcs(&p.sorted_key[lo + j], kv[u]);
+            if (p.iperm) p.iperm[lo + idx[u]] = j;
+          }
+        }
       }
       __syncthreads();
       seg_lo = seg_hi;
@@ -185,28 +270,38 @@ __global__ void __launch_bounds__(KVS_SORT_THREADS) k_stats_sort(SortParams p) {
       i64* const ps = p.prefix_s + lo + inst;
       i64 run = 0;
       if (tid == 0) ps[0] = 0;
-      for (int j0 = 0; j0 < n; j0 += T) {
-        const int j = j0 + tid;
-        const i64 v = j < n ? p.sorted_s[lo + j] : 0;
-        i64 incl = v;
+      for (int j0 = 0; j0 < n; j0 += TILE_N) {
+        // a warp takes 32 * ITEMS consecutive ones, row by row
+        const int jw = j0 + warp * (32 * ITEMS) + lane;
+        u32 v[ITEMS];
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const i64 y = __shfl_up_sync(0xffffffffu, incl, d);
-          if (static_cast<int>(lane_id()) >= d) incl += y;
-        }
-        __syncthreads();
-        if (lane_id() == 31) wsum[tid >> 5] = incl;
-        __syncthreads();
-        const i64 w = static_cast<int>(lane_id()) < WARPS ? wsum[lane_id()] : 0;
-        i64 wi = w;
+        for (int i = 0; i < ITEMS; ++i) v[i] = jw + 32 * i < n ? static_cast<u32>(p.sorted_s[lo + jw + 32 * i]) : 0u;
+        i64 total = 0;
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const i64 y = __shfl_up_sync(0xffffffffu, wi, d);
-          if (static_cast<int>(lane_id()) >= d) wi += y;
-        }
-        const i64 before = run + __shfl_sync(0xffffffffu, wi - w, tid >> 5);   // all lanes take part in the shuffle
-        if (j < n) __stcs(&ps[j + 1], before + incl);
+        for (int i = 0; i < ITEMS; ++i) total += v[i];
+        total = warp_sum(total);
+        __syncthreads();
+        if (lane == 0) wsum[warp] = total;
+        __syncthreads();
+        const i64 w = lane < WARPS ? wsum[lane] : 0;
+        const i64 wi = warp_incl(w);
+        i64 before = run + __shfl_sync(0xffffffffu, wi - w, warp);     // all lanes take part in the shuffle
         run += __shfl_sync(0xffffffffu, wi, 31);
+        if (s_max < (1 << 26)) {                        // a row adds up in 32 bits
+#pragma unroll
+          for (int i = 0; i < ITEMS; ++i) {
+            const u32 incl = warp_incl(v[i]);
+            if (jw + 32 * i < n) __stcs(&ps[jw + 32 * i + 1], before + incl);
+            before += __shfl_sync(0xffffffffu, incl, 31);
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < ITEMS; ++i) {
+            const i64 incl = warp_incl(static_cast<i64>(v[i]));
+            if (jw + 32 * i < n) __stcs(&ps[jw + 32 * i + 1], before + incl);
+            before += __shfl_sync(0xffffffffu, incl, 31);
+          }
+        }
       }
     }
   }
@@ -252,7 +347,7 @@ __global__ void __launch_bounds__(256) k_stats(SortParams p) {
 
 }  // namespace
 
-static constexpr size_t SORT_SMEM = 2 * WARPS * 256 * sizeof(u32);   // digit counts and offsets per warp
+static constexpr size_t SORT_SMEM = WARPS * ROW_W * sizeof(u32);   // digit counts per warp
 
 // Once per device, before the first launch.
 cudaError_t kvs_setup_sort() {

@@ -446,3 +446,15 @@ def test_windows_of_shared_evaluations(par, est, W):
     rows = [dict(instance=0, family=f, M=m) for f in ("GBA", "GSA", "SPS", "SIMS") for m in (1500, 40_000)]
     for prof in (True, False):
         par.check_batch(inst, binding.make_settings(rows), window=W, want_runs=False, want_profile=prof, label=f"shared windows {W}")
+
+
+@pytest.mark.parametrize("n, o_max", [(31, 5), (33, 300), (2_047, 200), (2_049, 70_000), (4_096, 255), (4_097, 256), (65_536, 900), (65_537, 900)])
+def test_order_at_the_edges_of_tiles(par, n, o_max):
+    """One to three digits, rows and tiles that are full, one more and one less, 16-bit indices and beyond; two instances that
+    do not start at a multiple of anything."""
+    c = torch.arange(n)
+    one = lambda k: (workloads.uniform_int(8100 + k, c, 0, 90), workloads.pareto_int(8200 + k, c, 2.0, 0.8, 1, o_max))
+    (s0, o0), (s1, o1) = one(0), one(1)
+    inst = workloads.Instances(torch.tensor([0, 7, 7 + n, 7 + 2 * n]), torch.cat([s0[:1].repeat(7), s0, s1]), torch.cat([o0[:1].repeat(7), o0, o1]))
+    M = 4 * (90 + o_max)
+    par.check_batch(inst, binding.settings_grid(range(3), ["GBA", "SPS", "SIMS"], [M, 1 << 21]), want_runs=False, want_profile=False, label=f"order n={n} o<={o_max}")
