@@ -167,6 +167,21 @@ typedef struct {
                                    among that phase's participants instead of s_bar; the ladder still ends at M - s_bar */
 } kvs_setting;
 
+/* Sizes that lie in device memory and that a caller needs on the host before it can allocate the outputs of a call: the jobs
+ * per instance and, where profiles are wanted, the rounds reserved for each evaluation.  In two halves, so that the
+ * caller can work while the values are on their way.  kvs_sizes_begin copies `job_off` (DEVICE [n_instances + 1]) and / or
+ * `capacity` (DEVICE [P]; either may be NULL) to page-locked memory behind what `stream` (a cudaStream_t) holds.  kvs_sizes_end
+ * waits for that, fills `out` and uploads, on the same stream, the offsets 0, c_0, c_0 + c_1, .. of the evaluations' job
+ * results (`job_out_off`, DEVICE [P + 1]; the jobs of each setting's instance) and profiles (`profile_off`, DEVICE [P + 1]);
+ * either may be NULL.  A setting that names no instance of the batch is refused (KVS_E_ARG) before any indexing. */
+typedef struct kvs_sizes {
+  int64_t max_jobs;        /* largest instance */
+  int64_t job_results;     /* job_out_off[P] */
+  int64_t profile_rounds;  /* profile_off[P] */
+} kvs_sizes;
+int kvs_sizes_begin(kvs_ctx* ctx, void* stream, const int64_t* job_off, int64_t n_instances, const int64_t* capacity, int64_t P);
+int kvs_sizes_end(kvs_ctx* ctx, const kvs_setting* settings, int64_t P, int64_t* job_out_off, int64_t* profile_off, kvs_sizes* out);
+
 /* Per-job and per-run outputs of the builder.  Any pointer may be NULL to skip that output. */
 typedef struct {
   const int64_t* job_out_off;   /* DEVICE [P + 1]: evaluation e writes its n jobs at job_out_off[e] + i,

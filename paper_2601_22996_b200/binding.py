@@ -72,13 +72,17 @@ class _SweepOut(Structure):
                 ("job_steps", c_void_p), ("feasible", c_void_p)]
 
 
+class _Sizes(Structure):
+    _fields_ = [("max_jobs", c_int64), ("job_results", c_int64), ("profile_rounds", c_int64)]
+
+
 class _BoundsOut(Structure):
     _fields_ = [("upper_gba", c_void_p), ("upper_gsa", c_void_p), ("lower_2m", c_void_p), ("status", c_void_p)]
 
 
 EXPORTS = ["kvs_init", "kvs_destroy", "kvs_last_error", "kvs_set_timing", "kvs_last_timing", "kvs_last_timing_split", "kvs_debug_check_word", "kvs_workspace_bytes",
            "kvs_build_schedule", "kvs_evaluate_built", "kvs_evaluate_built_host", "kvs_evaluate_schedule", "kvs_evaluate_schedule_sized", "kvs_set_unwritten", "kvs_sweep",
-           "kvs_evaluate_schedule_noalloc", "kvs_bounds"]
+           "kvs_evaluate_schedule_noalloc", "kvs_bounds", "kvs_sizes_begin", "kvs_sizes_end"]
 
 _lib = None
 
@@ -109,6 +113,8 @@ def load(path: str | None = None):
         L.kvs_set_unwritten.argtypes = [c_void_p, c_int32, c_int32, c_int32]
         L.kvs_sweep.argtypes = [c_void_p, POINTER(_Instances), POINTER(_SweepParams), POINTER(_SweepOut)]
         L.kvs_bounds.argtypes = [c_void_p, POINTER(_Instances), c_void_p, c_int64, POINTER(_BoundsOut)]
+        L.kvs_sizes_begin.argtypes = [c_void_p, c_void_p, c_void_p, c_int64, c_void_p, c_int64]
+        L.kvs_sizes_end.argtypes = [c_void_p, c_void_p, c_int64, c_void_p, c_void_p, POINTER(_Sizes)]
         L.kvs_evaluate_schedule_noalloc.argtypes = [c_int32, c_void_p, POINTER(_Runs), POINTER(_EvalOut), c_int64,
                                                     ctypes.c_char_p, c_uint64]
         _lib = L
@@ -264,6 +270,12 @@ class Context:
         self._check(fn(self._ctx, ctypes.byref(ci), settings.ctypes.data, settings.shape[0],
                        ctypes.byref(so) if so else None, ctypes.byref(eo) if eo else None))
 
+    def evaluate_structs(self, inst: Instances, settings: np.ndarray, so: _ScheduleOut, eo: _EvalOut, window: int, max_jobs: int, tensors):
+        """kvs_evaluate_built with structs that the caller has filled from ``tensors``."""
+        ci = self._instances(inst, window, max_jobs)
+        self._keep = (settings, inst, tensors)   # alive until the stream has consumed them
+        self._check(self._lib.kvs_evaluate_built(self._ctx, ctypes.byref(ci), settings.ctypes.data, settings.shape[0], ctypes.byref(so), ctypes.byref(eo)))
+
     def build_schedule(self, inst: Instances, settings: np.ndarray, out: dict, ev: dict | None = None,
                        window: int = 0, max_jobs: int | None = None):
         """kvs_build_schedule: ``out`` / ``ev`` map field names of the C structs to CUDA tensors."""
@@ -296,6 +308,20 @@ class Context:
         """kvs_set_unwritten: outputs that an evaluation does not form take these values from now on (no argument: they keep
         what the buffers held)."""
         self._check(self._lib.kvs_set_unwritten(self._ctx, 0 if job_value is None else 1, job_value or 0, profile_value))
+
+    def sizes_begin(self, stream: torch.cuda.Stream, job_off: torch.Tensor | None, capacity: torch.Tensor | None):
+        """kvs_sizes_begin: contiguous int64 CUDA tensors, read behind what ``stream`` holds."""
+        self._sizes_of = (job_off, capacity)     # alive until they have been read
+        self._check(self._lib.kvs_sizes_begin(self._ctx, stream.cuda_stream, _p(job_off), 0 if job_off is None else job_off.numel() - 1,
+                                              _p(capacity), 0 if capacity is None else capacity.numel()))
+
+    def sizes_end(self, settings: np.ndarray | None, P: int, job_out_off: torch.Tensor | None, profile_off: torch.Tensor | None) -> _Sizes:
+        """kvs_sizes_end: waits, fills the offset tensors [P + 1] and returns max_jobs, job_results and profile_rounds."""
+        out = _Sizes()
+        self._check(self._lib.kvs_sizes_end(self._ctx, None if settings is None else settings.ctypes.data, P, _p(job_out_off), _p(profile_off),
+                                            ctypes.byref(out)))
+        self._sizes_of = None
+        return out
 
     def evaluate_schedule(self, runs: dict, ev: dict, capacity_total: int | None = None):
         """kvs_evaluate_schedule: ``runs`` maps run_off, run_start, run_len, run_s [, run_flow, M].  With ``capacity_total``

@@ -83,7 +83,7 @@ constexpr int BINS = 16512;                                 // 64.5 KB of shared
 constexpr int BT = 512;
 constexpr int BIN_PER = BINS / BT + 1;                      // bins per thread of the scan: odd, no bank conflicts
 __global__ void __launch_bounds__(BT, 3) k_class_counts(const i64* __restrict__ job_off, const int32_t* __restrict__ s, const int32_t* __restrict__ o, i64 max_jobs,
-                                                        InstStats* __restrict__ stats, const kvs_setting* __restrict__ settings,
+                                                        InstStats* __restrict__ stats, const __grid_constant__ BoundSettings settings,
                                                         const i64* __restrict__ runs, u32* __restrict__ counts) {
   extern __shared__ u32 bin[];                              // BIN_PER * BT words
   __shared__ Ladder sh;
@@ -96,8 +96,9 @@ __global__ void __launch_bounds__(BT, 3) k_class_counts(const i64* __restrict__ 
   // the settings lie in page-locked host memory (a read takes microseconds): one per warp, all of them together
   constexpr int SW = sizeof(kvs_setting) / 4;
   auto fetch = [&](i64 first) {
-    const int n_words = static_cast<int>(min_i64(BT / 32, e0 + n_e - first)) * SW;
-    for (int i = tid; i < n_words; i += BT) reinterpret_cast<u32*>(sts)[i] = reinterpret_cast<const u32*>(settings + first)[i];
+    const int n_sets = static_cast<int>(min_i64(BT / 32, e0 + n_e - first)), n_words = n_sets * SW;
+    if (settings.brief) { if (tid < n_sets) sts[tid] = settings[first + tid]; }
+    else for (int i = tid; i < n_words; i += BT) reinterpret_cast<u32*>(sts)[i] = reinterpret_cast<const u32*>(settings.full + first)[i];
   };
   fetch(e0);
   __syncthreads();
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(BT, 3) k_class_counts(const i64* __restrict__ 
 
 // The sums over the phases, one warp per evaluation, one lane per phase.
 __global__ void __launch_bounds__(BW * 32) k_bounds(const i64* __restrict__ job_off, const InstStats* __restrict__ stats,
-                                                    const kvs_setting* __restrict__ settings, i64 P, const u32* __restrict__ counts,
+                                                    const __grid_constant__ BoundSettings settings, i64 P, const u32* __restrict__ counts,
                                                     kvs_bounds_out out) {
   __shared__ Ladder shs[BW];
   const int lane = lane_id();
@@ -245,9 +246,11 @@ cudaError_t kvs_setup_bounds() {
 }
 
 // runs: n_runs pairs (first evaluation, number of evaluations) of evaluations of one instance; counts: P * KVS_MAX_PHASES words
-cudaError_t kvs_launch_bounds(const i64* job_off, const int32_t* s, const int32_t* o, i64 max_jobs, InstStats* stats, const kvs_setting* settings, i64 P,
+cudaError_t kvs_launch_bounds(const i64* job_off, const int32_t* s, const int32_t* o, i64 max_jobs, InstStats* stats, const kvs_setting* list, i64 P,
                               const i64* runs, i64 n_runs, const kvs_bounds_out& out, u32* counts, cudaStream_t stream) {
   if (P <= 0) return cudaSuccess;
+  const bool in_brief = list[0].family == KVS_SETTINGS_BRIEF;
+  const BoundSettings settings{list, in_brief ? reinterpret_cast<const int2*>(list + 1) : nullptr, list[0]};
   k_class_counts<<<static_cast<unsigned>(n_runs), BT, BIN_PER * BT * 4, stream>>>(job_off, s, o, max_jobs, stats, settings, runs, counts);
   k_bounds<<<static_cast<unsigned>((P + BW - 1) / BW), BW * 32, 0, stream>>>(job_off, stats, settings, P, counts, out);
   return cudaGetLastError();

@@ -218,6 +218,25 @@ cudaError_t kvs_setup_spec();
 // The caller zeroes the counters.
 cudaError_t kvs_launch_spec(SpecParams p, cudaStream_t stream);
 cudaError_t kvs_setup_bounds();
+// Settings of the bounds: in full, or (brief given) instance and budget of each, the rest from `base`.  The launch takes page-locked
+// host memory: the settings in full, or in brief - one setting of this family, otherwise what all of them share, and behind it
+// instance and budget of each.
+constexpr int32_t KVS_SETTINGS_BRIEF = -1;
+struct BoundSettings {
+  const kvs_setting* full;
+  const int2* brief;
+  kvs_setting base;
+#ifdef __CUDACC__
+  __device__ __forceinline__ kvs_setting operator[](i64 e) const {
+    if (!brief) return full[e];
+    const int2 v = brief[e];
+    kvs_setting st = base;
+    st.instance = v.x;
+    st.M = v.y;
+    return st;
+  }
+#endif
+};
 cudaError_t kvs_launch_bounds(const i64* job_off, const int32_t* s, const int32_t* o, i64 max_jobs, InstStats* stats, const kvs_setting* settings, i64 P,
                               const i64* runs, i64 n_runs, const kvs_bounds_out& out, u32* counts, cudaStream_t stream);
 // One instance ordered by the whole GPU (kvs_order.cu).

@@ -114,3 +114,24 @@ def test_long_runs_of_mixed_settings(sched):
     st = binding.make_settings(rows)
     assert st.shape[0] >= 17 * 3 * 148
     _check(sched, inst, st, sample=sorted(rng.choice(st.shape[0], 400, replace=False)))
+
+
+@pytest.mark.parametrize("odd_at", [None, 0, 1, 37, 71])
+@pytest.mark.parametrize("odd", [dict(s_bar=9), dict(beta0=3), dict(alpha_num=3, alpha_den=2), dict(tau=5, k=3)])
+def test_settings_that_differ_in_more_than_instance_and_budget(sched, odd_at, odd):
+    """Settings alike but for instance and budget reach the kernels in brief; one that differs makes them all go in full, wherever it is."""
+    inst = workloads.config2(n_inst=24, n=130)
+    st = binding.settings_grid(range(24), ["GBA"], [1 << 15, 1 << 18, 1 << 20])
+    if odd_at is not None:
+        for f, v in odd.items():
+            st[f][odd_at] = v
+    _check(sched, inst, st)
+    bad = st.copy()
+    bad["instance"][40] = 24
+    with pytest.raises(binding.KvsError):
+        sched.bounds(inst.to("cuda:0"), bad)
+    bad["instance"][40] = 0
+    bad["M"][40] = 0
+    with pytest.raises(binding.KvsError):
+        sched.bounds(inst.to("cuda:0"), bad)
+    _check(sched, inst, st[:1])

@@ -458,3 +458,40 @@ def test_order_at_the_edges_of_tiles(par, n, o_max):
     inst = workloads.Instances(torch.tensor([0, 7, 7 + n, 7 + 2 * n]), torch.cat([s0[:1].repeat(7), s0, s1]), torch.cat([o0[:1].repeat(7), o0, o1]))
     M = 4 * (90 + o_max)
     par.check_batch(inst, binding.settings_grid(range(3), ["GBA", "SPS", "SIMS"], [M, 1 << 21]), want_runs=False, want_profile=False, label=f"order n={n} o<={o_max}")
+
+
+def test_sizes_read_by_the_library(par):
+    """Sizes that the library reads itself (int64, on the device) against those that pass through the host: the same outputs, offsets and
+    refusals, per-job results of 32 and 64 bits, with and without them, also under another stream and on a fresh workspace."""
+    from paper_2601_22996_b200.api import Scheduler
+    inst = workloads.random_small(8300, 40, 90, 30, 60).to("cuda:0")
+    st = binding.settings_grid(range(40), ["GBA", "GSA", "SPS"], [400, 3_000])
+    P = st.shape[0]
+    cap = torch.full((P,), 1 << 14, dtype=torch.int64, device="cuda:0")
+    cap[::5] = 0
+    sch = Scheduler()
+    for jobs in (True, False):
+        for wide in (False, True) if jobs else (False,):
+            for c in (cap, None):
+                kw = dict(want_jobs=jobs, time64=wide, want_profile=c is not None)
+                a = sch.evaluate(inst, st, profile_capacity=c, **kw)
+                b = par.scheduler().evaluate(inst, st, profile_capacity=None if c is None else c.to(torch.int32), **kw) if c is not None else None
+                side = torch.cuda.Stream()
+                with torch.cuda.stream(side):
+                    d = sch.evaluate(inst, st, profile_capacity=c, **kw)
+                side.synchronize()
+                for x in (b, d):
+                    if x is None:
+                        continue
+                    for f, v in vars(a).items():
+                        w = getattr(x, f)
+                        assert (v is None) == (w is None), f
+                        assert v is None or torch.equal(v, w), (f, kw)
+    bad = st.copy()
+    bad["instance"][7] = 40
+    for c in (cap, None):
+        with pytest.raises(binding.KvsError):
+            sch.evaluate(inst, bad, want_profile=c is not None, profile_capacity=c)
+    with pytest.raises(binding.KvsError):
+        sch.evaluate(inst, st, want_profile=True, profile_capacity=cap[:-1])
+    assert torch.equal(sch.evaluate(inst, st).flow, par.scheduler().evaluate(inst, st, want_jobs=False).flow)
