@@ -7,10 +7,12 @@
 //
 // k_tile_eval: one CTA per (evaluation, tile of rounds).  The CTA reads all runs of its evaluation (they stay in L2
 // over the tiles), scatters the events of its rounds into difference arrays in shared memory and sums up, in registers, what
-// the runs that cross its first round hold there, so the tiles do not depend on each other.  It is bound by the visits of
-// the runs (about 25 instructions each) and shared-memory atomics; the 24 bytes per run and 4 per round that it has to move
-// are a third of its time.  With the arrays in global memory (k_generic_eval, four global atomics per run and 12 bytes
-// of scratch per round to clear and re-read) 256 schedules of 15,000 runs took 142 us and 45 us for clearing the scratch.
+// the runs that cross its first round hold there, so the tiles do not depend on each other.  The sums over all runs are formed by the
+// first tile alone, which leaves its flags to the last one.  It is bound by the visits of the runs (every tile looks at all of
+// them) and shared-memory atomics; the 24 bytes per run and 4 per round that it has to move are a third of its time.  256
+// schedules of 10,000 to 20,000 runs: a call of 123 us, 129 with every tile forming the sums; tiles of 27,648 rounds, one CTA of
+// 1,024 threads per SM, which look at the runs half as often: 153.  With the arrays in global memory (k_generic_eval, four global
+// atomics per run and 12 bytes of scratch per round to clear and re-read) the kernels alone took 142 us and 45 us.
 // Arithmetic is modulo 2^32, exact as long as the sum of s + len over the runs, which bounds the memory of any round, is
 // below 2^32; other evaluations (and ones with a negative s) are listed for k_generic_eval, which works in 64 bits.
 #include <atomic>
@@ -79,7 +81,9 @@ __global__ void __launch_bounds__(TT, 2) k_tile_eval(GenericParams p) {
   i64 steps = 0, hmax = 0, flow = 0;
   u64 total = 0;
   u32 A0 = 0, B0 = 0;                                    // held in round t0 by runs that started before it
-  int bad = 0, clipped = 0, wide = 0;
+  int flags = 0;                                         // 1: bad input, 2: beyond the capacity, 4: not for 32 bits
+  int last = 0;                                          // rounds of the tile up to the last run end
+  const bool first = my == 0;                            // this tile forms what concerns all runs alike
   __syncthreads();
   constexpr int U = 4;
   for (i64 rb = r0; rb < r1; rb += U * TT) {
@@ -93,43 +97,54 @@ __global__ void __launch_bounds__(TT, 2) k_tile_eval(GenericParams p) {
       ln[u] = on ? __ldg(R.run_len + r) : 0;
       sv[u] = on ? __ldg(R.run_s + r) : 0;
     }
-    if (R.run_flow && my == 0) {
+    if (R.run_flow && first) {
 #pragma unroll
       for (int u = 0; u < U; ++u) { const i64 r = rb + u * TT + tid; if (r < r1) flow += __ldg(R.run_flow + r); }
     }
+    if (first) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (ln[u] <= 0) continue;
+        if (st[u] < 0) { flags |= 1; continue; }
+        const i64 end = st[u] + ln[u];
+        steps += ln[u];
+        hmax = max_i64(hmax, end);
+        flags |= (end > cap ? 2 : 0) | (sv[u] < 0 ? 4 : 0);
+        total += static_cast<u64>(static_cast<i64>(sv[u]) + ln[u]);
+      }
+    }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (ln[u] <= 0) continue;
-      if (st[u] < 0) { bad = 1; continue; }
-      const i64 start = st[u], end = start + ln[u];
-      steps += ln[u];
-      hmax = max_i64(hmax, end);
-      clipped |= end > cap ? 1 : 0;
-      wide |= sv[u] < 0 ? 1 : 0;
-      total += static_cast<u64>(static_cast<i64>(sv[u]) + ln[u]);
-      if (start >= t1 || end <= t0) continue;
-      const u32 c = static_cast<u32>(sv[u]) + 1u - static_cast<u32>(start);
-      if (start < t0) { A0 += c; B0 += 1u; }
-      else { atomicAdd(&dA[start - t0], c); atomicAdd(&dB[start - t0], 1u); }
-      if (end < t1) { atomicAdd(&dA[end - t0], 0u - c); atomicAdd(&dB[end - t0], 0xffffffffu); }
+      if (ln[u] <= 0 || st[u] < 0) continue;
+      const i64 rs = st[u] - t0, re = rs + ln[u];          // from the tile's first round on
+      if (re <= 0) continue;
+      last = max(last, static_cast<int>(min_i64(re, tile)));
+      if (rs >= tile) continue;
+      const u32 c = static_cast<u32>(sv[u]) + 1u - static_cast<u32>(st[u]);
+      if (rs < 0) { A0 += c; B0 += 1u; }
+      else { atomicAdd(&dA[rs], c); atomicAdd(&dB[rs], 1u); }
+      if (re < tile) { atomicAdd(&dA[re], 0u - c); atomicAdd(&dB[re], 0xffffffffu); }
     }
   }
-  hmax = block_max(hmax, red64, static_cast<i64>(0));
-  total = block_sum(total, redu);
-  const int flags = block_max((bad << 0), red32, 0) | block_max(clipped, red32, 0) << 1 | block_max(wide, red32, 0) << 2;
-  bad = flags & 1; clipped = flags >> 1 & 1; wide = flags >> 2;
-  if (wide || total >= (static_cast<u64>(1) << 32)) {
-    if (my == 0 && tid == 0) p.wide_list[atomicAdd(p.wide_count, 1u)] = e;
-    return;
+  if (first) {
+    hmax = block_max(hmax, red64, static_cast<i64>(0));
+    total = block_sum(total, redu);
+    flags = block_max(flags & 1, red32, 0) | block_max(flags & 2, red32, 0) | block_max(flags & 4, red32, 0);
+    if ((flags & 4) || total >= (static_cast<u64>(1) << 32)) {
+      // the 64-bit kernel, which runs next, writes every output of this evaluation, also those that its other tiles have written
+      if (tid == 0) p.wide_list[atomicAdd(p.wide_count, 1u)] = e;
+      return;
+    }
   }
+  last = block_max(last, red32, 0);
   A0 = block_sum(A0, scanA);
   B0 = block_sum(B0, scanB);
-  if (my == 0) {
+  if (first) {
     steps = block_sum(steps, red64);
     flow = block_sum(flow, red64);
   }
   // prefix sums over the tile: a thread's stretch, then the threads
-  const i64 t_end = min_i64(min_i64(hmax, cap), t1);      // rounds [t0, t_end) of this tile exist
+  const i64 t_end = min_i64(t0 + last, cap);              // rounds [t0, t_end) of this tile exist
   const int e0 = tid * per;
   u32 sa = 0, sb = 0;
   for (int i = 0; i < per; ++i) { sa += dA[e0 + i]; sb += dB[e0 + i]; }
@@ -164,13 +179,16 @@ __global__ void __launch_bounds__(TT, 2) k_tile_eval(GenericParams p) {
   if (tid != 0) return;
   // the tile that finishes last holds the largest memory of all of them
   atomicMax(&p.tile_peak[e], peak);
-  if (my == 0) {
+  if (first) {
     if (p.ev.flow) p.ev.flow[e] = flow;
     if (p.ev.job_steps) p.ev.job_steps[e] = steps;
     if (p.ev.horizon) p.ev.horizon[e] = hmax;
   }
   __threadfence();
-  if (atomicAdd(&p.tile_done[e], 1u) + 1u != static_cast<u32>(n_tiles)) return;
+  // finished tiles in the lower 28 bits, the first tile's flags above them
+  const u32 mine = first ? 1u + (static_cast<u32>(flags) << 28) : 1u, sum = atomicAdd(&p.tile_done[e], mine) + mine;
+  if ((sum & 0x0fffffffu) != static_cast<u32>(n_tiles)) return;
+  const bool bad = (sum >> 28 & 1u) != 0, clipped = (sum >> 29 & 1u) != 0;
   __threadfence();
   const i64 top = static_cast<i64>(atomicMax(&p.tile_peak[e], 0u));
   int status = 0;
