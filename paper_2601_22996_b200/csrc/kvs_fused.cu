@@ -52,6 +52,8 @@ constexpr int RPT = 4;                       // consecutive ranks per thread in 
 constexpr int MAXP = KVS_MAX_PHASES;
 constexpr int RINGW = 2 * TILE + (2 * TILE) / 8;
 constexpr int GCOL = 2049;
+constexpr int PAIR_CYCLES = 60;              // see the use
+constexpr u64 SHARED_PAIRS = 1u << 20;       // more pairs of run ends and runs in a phase are shared between an evaluation's CTAs
 static_assert((TILE & (TILE - 1)) == 0 && ITEMS % 4 == 0 && ITEMS <= 32 && 32 % ITEMS == 0, "tile layout");
 constexpr u32 TIME_LIMIT = 0x7fffffffu - 4u * TILE;   // phase ends stay below this
 
@@ -836,25 +838,30 @@ __device__ __forceinline__ void block_prefix(FShared& sh, u32* out, int out_cap,
 
 // Peak of one staggered phase without its rounds: memory grows between the ends of runs, so its maximum is the memory in
 // the last round of some run, summed here over the ranks that have started and whose slots have not ended then - at
-// most k of them.  job(r) = (s, o) of rank r.  Returns this thread's maximum.
+// most k of them.  job(r) = (s, o) of rank r.  First every rank's s less its start and its end go to `list` (which may be where
+// job reads from), so that a pair of a run end and a rank costs a load, a comparison and two additions.  Of the run ends this CTA
+// takes those of `part` of `parts`.  Returns this thread's maximum.
 template <class F>
-__device__ __forceinline__ u32 ends_peak(u32 N, u32 tau, u32 k, u64 kinv, F job) {
+__device__ __forceinline__ u32 ends_peak(uint2* list, int list_cap, u32 N, u32 tau, u32 k, u64 kinv, int part, int parts, F job) {
+  (void)list_cap;
+  for (u32 r = threadIdx.x; r < N; r += T) {
+    const uint2 e = job(static_cast<int>(r));
+    const u32 q = slot_mul(r, tau, k, kinv);
+    if (KVS_IN(r, list_cap, CHK_LIST_OUT)) list[r] = make_uint2(e.x - q, q + min(e.y, tau));
+  }
+  __syncthreads();
   u32 peak = 0;
-  const u32 qt = tau / k, rt = tau - qt * k;
-  for (u32 i = threadIdx.x; i < N; i += T) {
-    const u32 t1 = slot_mul(i, tau, k, kinv) + min(job(static_cast<int>(i)).y, tau);      // last round of the run, plus one
+  for (u32 i = threadIdx.x + static_cast<u32>(part) * T; i < N; i += static_cast<u32>(parts) * T) {
+    const u32 t1 = list[i].y;                                      // last round of the run, plus one
     const u32 rb = static_cast<u32>(min_i64(N, ceil_div_u(static_cast<u64>(t1) * k, tau)));
     const u32 ra = t1 <= tau ? 0u : static_cast<u32>(ceil_div_u(static_cast<u64>(t1 - tau) * k, tau));
-    u64 q_, r_;
-    divmod_u(static_cast<u64>(ra) * tau, k, &q_, &r_);
-    u32 q = static_cast<u32>(q_), rem = static_cast<u32>(r_), sum = 0;
+    u32 sum = 0, cnt = 0;
+#pragma unroll 4
     for (u32 r = ra; r < rb; ++r) {
-      const uint2 e = job(static_cast<int>(r));
-      if (q + min(e.y, tau) >= t1) sum += e.x + t1 - q;
-      rem += rt; q += qt;
-      if (rem >= k) { rem -= k; ++q; }
+      const uint2 e = list[r];
+      if (e.y >= t1) { sum += e.x; ++cnt; }
     }
-    peak = max(peak, sum);
+    peak = max(peak, sum + cnt * t1);
   }
   return peak;
 }
@@ -1720,6 +1727,7 @@ __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 
           any_pure = __syncthreads_or(mine) != 0;
         }
         bool begun = false;
+        int turn = 0;
         auto s_plus_1 = [&](int x) { return static_cast<u32>(__ldg(S_ord + seg_lo + x)) + 1u; };
         if (carry && !est) {
           if (any_pure && !peak_only) block_prefix(sh, PS, 2 * list_cap, nseg, s_plus_1);
@@ -1730,12 +1738,17 @@ __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 
           const int ph = peak_only ? L - 1 - it : it;
           const int N = static_cast<int>(sh.np[ph]);
           if (N == 0) continue;
+          int part_of = 0, parts_of = 1;           // share of a phase that all CTAs of the evaluation look at
           // tile origins keep the profile stores 16-byte aligned
           const int a0 = -static_cast<int>((prof_base + sh.pbase[ph]) & 3);
           const int n_tiles = static_cast<int>((sh.plen[ph] - a0 + TILE - 1) / TILE);
           int tile_lo = 0, tile_hi = n_tiles;
           if (SHARED && parts > 1 && peak_only) {
-            if (it % parts != part) continue;
+            // The phases are taken in turn, but one of many pairs of run ends and runs is looked at by all CTAs, each of which takes a
+            // share of its run ends: 64 initial slices on 20,000 jobs, whose longest evaluations have few phases, 420 -> 250 us.
+            const u64 pairs = static_cast<u64>(N) * min(static_cast<u32>(N), sh.k[ph]), rounds = static_cast<u64>(n_tiles) * 6000;
+            if (!batches && !sim && ph >= n_pure && pairs > SHARED_PAIRS && rounds >= static_cast<u64>(N) && pairs / T * PAIR_CYCLES / parts < rounds) { part_of = part; parts_of = parts; }
+            else if (turn++ % parts != part) continue;
             // what the other CTAs of this evaluation have found
             __syncthreads();
             if (tid == 0) sh.redA[0] = atomicMax(&p.shares[slot_no].peak, top);
@@ -1812,9 +1825,11 @@ __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 
               }
               return block_max(W, sh.redA, 0u);
             };
-            // Cycles of a CTA, roughly: 60 per step of a thread over the pairs of a run end and a run that may be active
-            // then, against 6,000 per tile and 8 per run; the bound takes the prefix sums over the ranks.
-            const u64 pairs = static_cast<u64>(N) * kk, by_ends = pairs / T * 60 + 1500, by_rounds = static_cast<u64>(n_tiles) * 6000 + static_cast<u64>(N) * (sliced ? 1 : 8);
+            // Cycles of a CTA, roughly: PAIR_CYCLES per step of a thread over the pairs of a run end and a run that may be active
+            // then, against 6,000 per tile and 8 per run; the bound takes the prefix sums over the ranks.  (A pair costs less by
+            // itself; 40 and 100 instead of 60: 1,024 instances from host memory 3,414 and 3,224 us against 3,235, 128 instances of
+            // 3,000 jobs 472 and 457 against 458, 60 of 10,000 at one budget 177 and 173 against 173.)
+            const u64 pairs = static_cast<u64>(N) * kk, by_ends = pairs / T * PAIR_CYCLES / parts_of + 1500, by_rounds = static_cast<u64>(n_tiles) * 6000 + static_cast<u64>(N) * (sliced ? 1 : 8);
             if (pure) {
               // the window of all these phases at their largest parallelism bounds each of them
               if (!have_ps) {
@@ -1831,8 +1846,8 @@ __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 
             }
             if (!straight && by_ends < by_rounds) {
               u32 pk;
-              if (listed) pk = ends_peak(N, P.tau, P.k, sh.kinv[ph], [&](int r) { return KVS_IN(r, list_cap, CHK_LIST) ? cur[r] : make_uint2(0, 1); });
-              else pk = ends_peak(N, P.tau, P.k, sh.kinv[ph], [&](int r) { return make_uint2(static_cast<u32>(__ldg(P.S + P.x_lo + r)), static_cast<u32>(__ldg(P.O + P.x_lo + r))); });
+              if (listed) pk = ends_peak(cur, list_cap, N, P.tau, P.k, sh.kinv[ph], part_of, parts_of, [&](int r) { return KVS_IN(r, list_cap, CHK_LIST) ? cur[r] : make_uint2(0, 1); });
+              else pk = ends_peak(cur, list_cap, N, P.tau, P.k, sh.kinv[ph], part_of, parts_of, [&](int r) { return make_uint2(static_cast<u32>(__ldg(P.S + P.x_lo + r)), static_cast<u32>(__ldg(P.O + P.x_lo + r))); });
               acc.peak = max(acc.peak, pk);
               top = max(top, block_max(pk, sh.redA, 0u));
               continue;

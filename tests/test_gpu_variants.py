@@ -175,3 +175,12 @@ def test_shared_evaluations_by_kernel(par, kind, want_profile):
     if kind == "one variant":
         rows[5].update(subroutine=1, per_class_s=1)
     par.check_batch(inst, binding.make_settings(rows), window=window, want_runs=False, want_profile=want_profile, label=f"shared {kind}")
+
+
+@pytest.mark.parametrize("n, alpha", [(6_000, (2, 1)), (2_500, (3, 2)), (513, (2, 1))])
+def test_few_long_phases_are_shared_between_ctas(par, n, alpha):
+    """Evaluations without a profile whose long slices pair many run ends with many runs: every CTA of an evaluation takes some of the ends."""
+    inst = workloads.config2(n_inst=1, n=n)
+    rows = [dict(instance=0, family=fam, M=M, beta0=b, alpha=alpha) for fam in ("GBA", "GSA") for M in (1 << 20, 1 << 22) for b in (0, 40, 700, 3_000)]
+    par.check_batch(inst, binding.make_settings(rows), want_runs=False, want_profile=False, label=f"long phases n={n}")
+    par.check_batch(inst, binding.make_settings(rows[8:9]), want_runs=False, want_profile=False, label=f"long phases alone n={n}")
