@@ -1094,7 +1094,7 @@ struct FAcc {
 // VARIANTS: with the code for simultaneous batches and per-phase prompt lengths.  The full batching kernel never has it (the light one
 // takes those, or leaves them to the general kernel): 176 bytes of spills a thread with it, 12 without, 4,096 evaluations of 50,000
 // jobs with their profiles 4.03 and 3.36 ms.  The kernel for shared evaluations exists with it, without it, and without it for calls
-// with estimates (spill loads a thread 2,932, 2,248 and 1,840 bytes; one kernel for all three: 3,568): 64 instances of 50,000 jobs
+// with estimates (spill loads a thread 3,080, 2,328 and 1,840 bytes; one kernel for all three: 3,568): 64 instances of 50,000 jobs
 // in windows 1,432 -> 1,270 us, four evaluations of 1,000 jobs 177 -> 170, 64 initial slices 429 -> 406.  The slicing
 // kernel spills no less without it.
 template <bool LIGHT, int FAM, bool VARIANTS>
