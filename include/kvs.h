@@ -18,6 +18,8 @@
  *     tensors) that must stay alive until the stream has finished the call.
  *   - All work is enqueued on the context's CUDA stream; calls do not synchronise the host
  *     unless stated.
+ *   - Calls on one context (or one reader, see kvs_sizes_begin) do not overlap: threads that share
+ *     one take turns.
  *   - Argument errors are found on the host before any launch.  Data errors (a job that
  *     cannot fit, an output range or capacity that is too small) are reported per
  *     evaluation in `status[]`; the kernels skip or clip the offending evaluation and
@@ -173,14 +175,23 @@ typedef struct {
  * `capacity` (DEVICE [P]; either may be NULL) to page-locked memory behind what `stream` (a cudaStream_t) holds.  kvs_sizes_end
  * waits for that, fills `out` and uploads, on the same stream, the offsets 0, c_0, c_0 + c_1, .. of the evaluations' job
  * results (`job_out_off`, DEVICE [P + 1]; the jobs of each setting's instance) and profiles (`profile_off`, DEVICE [P + 1]);
- * either may be NULL.  A setting that names no instance of the batch is refused (KVS_E_ARG) before any indexing. */
+ * either may be NULL.  A setting that names no instance of the batch is refused (KVS_E_ARG) before any indexing.
+ *
+ * A request belongs to a reader, which no context shares: page-locked memory of its own for one request at a time.  A request that
+ * has been begun is ended, whatever kvs_sizes_end returns, before the next one is begun on the same reader; a begin in between
+ * is refused (KVS_E_STATE) and leaves the open request as it is, an end without a begin too.  Threads that read sizes at the same time use a reader each.
+ * kvs_reader_close waits for what is in flight, of a request that was never ended too.  kvs_reader_error: as kvs_last_error. */
+typedef struct kvs_reader kvs_reader; /* opaque; owned by the library (host object only) */
+int kvs_reader_open(int32_t device, kvs_reader** out);
+int kvs_reader_close(kvs_reader* reader);
+const char* kvs_reader_error(const kvs_reader* reader);
 typedef struct kvs_sizes {
   int64_t max_jobs;        /* largest instance */
   int64_t job_results;     /* job_out_off[P] */
   int64_t profile_rounds;  /* profile_off[P] */
 } kvs_sizes;
-int kvs_sizes_begin(kvs_ctx* ctx, void* stream, const int64_t* job_off, int64_t n_instances, const int64_t* capacity, int64_t P);
-int kvs_sizes_end(kvs_ctx* ctx, const kvs_setting* settings, int64_t P, int64_t* job_out_off, int64_t* profile_off, kvs_sizes* out);
+int kvs_sizes_begin(kvs_reader* reader, void* stream, const int64_t* job_off, int64_t n_instances, const int64_t* capacity, int64_t P);
+int kvs_sizes_end(kvs_reader* reader, const kvs_setting* settings, int64_t P, int64_t* job_out_off, int64_t* profile_off, kvs_sizes* out);
 
 /* Per-job and per-run outputs of the builder.  Any pointer may be NULL to skip that output. */
 typedef struct {

@@ -82,7 +82,7 @@ class _BoundsOut(Structure):
 
 EXPORTS = ["kvs_init", "kvs_destroy", "kvs_last_error", "kvs_set_timing", "kvs_last_timing", "kvs_last_timing_split", "kvs_debug_check_word", "kvs_workspace_bytes",
            "kvs_build_schedule", "kvs_evaluate_built", "kvs_evaluate_built_host", "kvs_evaluate_schedule", "kvs_evaluate_schedule_sized", "kvs_set_unwritten", "kvs_sweep",
-           "kvs_evaluate_schedule_noalloc", "kvs_bounds", "kvs_sizes_begin", "kvs_sizes_end"]
+           "kvs_evaluate_schedule_noalloc", "kvs_bounds", "kvs_reader_open", "kvs_reader_close", "kvs_reader_error", "kvs_sizes_begin", "kvs_sizes_end"]
 
 _lib = None
 
@@ -113,6 +113,10 @@ def load(path: str | None = None):
         L.kvs_set_unwritten.argtypes = [c_void_p, c_int32, c_int32, c_int32]
         L.kvs_sweep.argtypes = [c_void_p, POINTER(_Instances), POINTER(_SweepParams), POINTER(_SweepOut)]
         L.kvs_bounds.argtypes = [c_void_p, POINTER(_Instances), c_void_p, c_int64, POINTER(_BoundsOut)]
+        L.kvs_reader_open.argtypes = [c_int32, POINTER(c_void_p)]
+        L.kvs_reader_close.argtypes = [c_void_p]
+        L.kvs_reader_error.argtypes = [c_void_p]
+        L.kvs_reader_error.restype = c_char_p
         L.kvs_sizes_begin.argtypes = [c_void_p, c_void_p, c_void_p, c_int64, c_void_p, c_int64]
         L.kvs_sizes_end.argtypes = [c_void_p, c_void_p, c_int64, c_void_p, c_void_p, POINTER(_Sizes)]
         L.kvs_evaluate_schedule_noalloc.argtypes = [c_int32, c_void_p, POINTER(_Runs), POINTER(_EvalOut), c_int64,
@@ -206,6 +210,40 @@ def workspace_bytes(n_jobs_total, n_instances, max_jobs, n_evaluations, generic_
     if rc:
         raise KvsError(rc, "kvs_workspace_bytes")
     return int(out.value)
+
+
+class SizesReader:
+    """kvs_reader: brings sizes from device memory to the host, one request at a time."""
+
+    def __init__(self, device: int):
+        self._lib = load()
+        self._reader = c_void_p()
+        rc = self._lib.kvs_reader_open(device, ctypes.byref(self._reader))
+        if rc:
+            raise KvsError(rc, "kvs_reader_open")
+
+    def __del__(self):
+        if getattr(self, "_reader", None):
+            self._lib.kvs_reader_close(self._reader)     # waits for a request that was not ended
+            self._reader = None
+
+    def _check(self, rc):
+        if rc:
+            raise KvsError(rc, self._lib.kvs_reader_error(self._reader).decode())
+
+    def begin(self, stream: torch.cuda.Stream, job_off: torch.Tensor | None, capacity: torch.Tensor | None):
+        """kvs_sizes_begin: contiguous int64 CUDA tensors, read behind what ``stream`` holds."""
+        self._check(self._lib.kvs_sizes_begin(self._reader, stream.cuda_stream, _p(job_off), 0 if job_off is None else job_off.numel() - 1,
+                                              _p(capacity), 0 if capacity is None else capacity.numel()))
+        self._keep = (job_off, capacity)         # alive until they have been read
+
+    def end(self, settings: np.ndarray | None, P: int, job_out_off: torch.Tensor | None, profile_off: torch.Tensor | None) -> _Sizes:
+        """kvs_sizes_end: waits, fills the offset tensors [P + 1] and returns max_jobs, job_results and profile_rounds."""
+        out = _Sizes()
+        self._check(self._lib.kvs_sizes_end(self._reader, None if settings is None else settings.ctypes.data, P, _p(job_out_off), _p(profile_off),
+                                            ctypes.byref(out)))
+        self._keep = None
+        return out
 
 
 class Context:
@@ -308,20 +346,6 @@ class Context:
         """kvs_set_unwritten: outputs that an evaluation does not form take these values from now on (no argument: they keep
         what the buffers held)."""
         self._check(self._lib.kvs_set_unwritten(self._ctx, 0 if job_value is None else 1, job_value or 0, profile_value))
-
-    def sizes_begin(self, stream: torch.cuda.Stream, job_off: torch.Tensor | None, capacity: torch.Tensor | None):
-        """kvs_sizes_begin: contiguous int64 CUDA tensors, read behind what ``stream`` holds."""
-        self._sizes_of = (job_off, capacity)     # alive until they have been read
-        self._check(self._lib.kvs_sizes_begin(self._ctx, stream.cuda_stream, _p(job_off), 0 if job_off is None else job_off.numel() - 1,
-                                              _p(capacity), 0 if capacity is None else capacity.numel()))
-
-    def sizes_end(self, settings: np.ndarray | None, P: int, job_out_off: torch.Tensor | None, profile_off: torch.Tensor | None) -> _Sizes:
-        """kvs_sizes_end: waits, fills the offset tensors [P + 1] and returns max_jobs, job_results and profile_rounds."""
-        out = _Sizes()
-        self._check(self._lib.kvs_sizes_end(self._ctx, None if settings is None else settings.ctypes.data, P, _p(job_out_off), _p(profile_off),
-                                            ctypes.byref(out)))
-        self._sizes_of = None
-        return out
 
     def evaluate_schedule(self, runs: dict, ev: dict, capacity_total: int | None = None):
         """kvs_evaluate_schedule: ``runs`` maps run_off, run_start, run_len, run_s [, run_flow, M].  With ``capacity_total``

@@ -41,8 +41,19 @@ struct kvs_ctx {
   bool fill = false;          // kvs_set_unwritten
   int32_t fill_job = 0, fill_prof = 0;
   void* pinned = nullptr;   // 256 bytes of page-locked memory for values that the host has to see
-  // What kvs_sizes_begin has sent to the host: job offsets, then capacities (counts; -1: not asked for)
-  struct Sizes { int64_t* p = nullptr; size_t bytes = 0; cudaStream_t stream = nullptr; int64_t n_off = -1, n_cap = -1; bool open = false; } sizes;
+  std::string err;
+};
+
+// One caller's sizes on their way (kvs_sizes_begin, kvs_sizes_end).  Apart from the contexts: the wait for them is long, and another
+// thread may use, or replace by a larger one, the context that the call will run on meanwhile.
+struct kvs_reader {
+  int device = 0;
+  cudaStream_t stream = nullptr;                           // of the last request
+  struct Pinned { int64_t* p = nullptr; size_t bytes = 0; } in, rows;   // what is read: job offsets, then capacities; what goes up
+  int64_t n_off = -1, n_cap = -1;                          // of the open request (-1: not asked for)
+  bool open = false;
+  cudaEvent_t sent = nullptr;                              // the rows of the last request have gone up
+  bool sending = false;
   std::string err;
 };
 
@@ -53,21 +64,23 @@ constexpr int64_t KVS_TIME_LIMIT = 1ll << 31; // exclusive bound on M, tau, k
 
 // Nothing leaves a C entry point as an exception: host memory that runs out becomes a status (and, for the text of an error,
 // an empty text).
-template <class F>
-int guarded(kvs_ctx* ctx, F body) noexcept {
+template <class H, class F>
+int guarded(H* handle, F body) noexcept {
   try {
     return body();
   } catch (...) {
-    ctx->err.clear();
+    handle->err.clear();
     return KVS_E_STATE;
   }
 }
-int fail(kvs_ctx* ctx, int code, const char* msg) {
-  if (ctx) guarded(ctx, [&] { ctx->err = msg; return 0; });
+template <class H>
+int fail(H* handle, int code, const char* msg) {
+  if (handle) guarded(handle, [&] { handle->err = msg; return 0; });
   return code;
 }
-int fail_cuda(kvs_ctx* ctx, cudaError_t e, const char* where) {
-  if (ctx) guarded(ctx, [&] { ctx->err = std::string(where) + ": " + cudaGetErrorString(e); return 0; });
+template <class H>
+int fail_cuda(H* handle, cudaError_t e, const char* where) {
+  if (handle) guarded(handle, [&] { handle->err = std::string(where) + ": " + cudaGetErrorString(e); return 0; });
   return KVS_E_CUDA;
 }
 
@@ -747,8 +760,6 @@ int kvs_destroy(kvs_ctx* ctx) {
       if (s.stream) cudaStreamDestroy(s.stream);
     }
     if (ctx->pinned) cudaFreeHost(ctx->pinned);
-    if (ctx->sizes.open) cudaStreamSynchronize(ctx->sizes.stream);
-    if (ctx->sizes.p) cudaFreeHost(ctx->sizes.p);
     for (kvs_ctx::Stage& s : ctx->stage) {
       if (s.used) cudaEventSynchronize(s.done);
       if (s.done) cudaEventDestroy(s.done);
@@ -767,54 +778,88 @@ int kvs_set_unwritten(kvs_ctx* ctx, int32_t enabled, int32_t job_value, int32_t 
   return KVS_OK;
 }
 
-int kvs_sizes_begin(kvs_ctx* ctx, void* stream, const int64_t* job_off, int64_t n_instances, const int64_t* capacity, int64_t P) {
-  if (!ctx) return KVS_E_STATE;
-  if (n_instances < 0 || P < 0) return fail(ctx, KVS_E_ARG, "sizes: negative count");
-  kvs_ctx::Sizes& z = ctx->sizes;
-  cudaError_t ce = cudaSetDevice(ctx->device);
-  if (ce == cudaSuccess && z.open) ce = cudaStreamSynchronize(z.stream);     // begun and never ended
-  if (ce != cudaSuccess) return fail_cuda(ctx, ce, "sizes");
-  z.open = false;
-  z.stream = static_cast<cudaStream_t>(stream);
-  z.n_off = job_off ? n_instances + 1 : -1;
-  z.n_cap = capacity ? P : -1;
-  const size_t off_bytes = job_off ? static_cast<size_t>(n_instances + 1) * 8 : 0, cap_bytes = capacity ? static_cast<size_t>(P) * 8 : 0;
-  if (z.bytes < off_bytes + cap_bytes) {
-    if (z.p) cudaFreeHost(z.p);
-    z.p = nullptr; z.bytes = 0;
-    const size_t want = off_bytes + cap_bytes + (off_bytes + cap_bytes) / 2 + 4096;
-    if ((ce = cudaMallocHost(reinterpret_cast<void**>(&z.p), want)) != cudaSuccess) return fail_cuda(ctx, ce, "cudaMallocHost");
-    z.bytes = want;
+int kvs_reader_open(int32_t device, kvs_reader** out) {
+  if (!out) return KVS_E_ARG;
+  *out = nullptr;
+  int count = 0;
+  if (cudaGetDeviceCount(&count) != cudaSuccess || count <= 0) return KVS_E_CUDA;
+  if (device < 0 || device >= count) return KVS_E_ARG;
+  kvs_reader* r = new (std::nothrow) kvs_reader();
+  if (!r) return KVS_E_STATE;
+  r->device = device;
+  if (cudaSetDevice(device) != cudaSuccess || cudaEventCreateWithFlags(&r->sent, cudaEventDisableTiming) != cudaSuccess) {
+    delete r;
+    return KVS_E_CUDA;
   }
-  if (off_bytes) ce = cudaMemcpyAsync(z.p, job_off, off_bytes, cudaMemcpyDeviceToHost, z.stream);
-  z.open = ce == cudaSuccess;
-  if (ce == cudaSuccess && cap_bytes) ce = cudaMemcpyAsync(reinterpret_cast<unsigned char*>(z.p) + off_bytes, capacity, cap_bytes, cudaMemcpyDeviceToHost, z.stream);
+  *out = r;
+  return KVS_OK;
+}
+
+int kvs_reader_close(kvs_reader* r) {
+  if (r) {
+    if (r->open) cudaStreamSynchronize(r->stream);         // begun and never ended
+    if (r->sending) cudaEventSynchronize(r->sent);
+    cudaEventDestroy(r->sent);
+    for (kvs_reader::Pinned* m : {&r->in, &r->rows}) if (m->p) cudaFreeHost(m->p);
+  }
+  delete r;
+  return KVS_OK;
+}
+
+const char* kvs_reader_error(const kvs_reader* r) { return r ? r->err.c_str() : "no reader"; }
+
+// Room for at least `bytes` bytes in memory that nothing in flight uses.
+static cudaError_t make_room(kvs_reader::Pinned& m, size_t bytes) {
+  if (m.bytes >= bytes) return cudaSuccess;
+  if (m.p) cudaFreeHost(m.p);
+  m.p = nullptr; m.bytes = 0;
+  const size_t want = bytes + bytes / 2 + 4096;
+  const cudaError_t ce = cudaMallocHost(reinterpret_cast<void**>(&m.p), want);
+  if (ce == cudaSuccess) m.bytes = want;
+  return ce;
+}
+
+int kvs_sizes_begin(kvs_reader* r, void* stream, const int64_t* job_off, int64_t n_instances, const int64_t* capacity, int64_t P) {
+  if (!r) return KVS_E_STATE;
+  if (r->open) return fail(r, KVS_E_STATE, "sizes: this reader's last request has not been ended");
+  if (n_instances < 0 || P < 0) return fail(r, KVS_E_ARG, "sizes: negative count");
+  r->stream = static_cast<cudaStream_t>(stream);
+  r->n_off = job_off ? n_instances + 1 : -1;
+  r->n_cap = capacity ? P : -1;
+  const size_t off_bytes = job_off ? static_cast<size_t>(n_instances + 1) * 8 : 0, cap_bytes = capacity ? static_cast<size_t>(P) * 8 : 0;
+  cudaError_t ce = cudaSetDevice(r->device);
+  if (ce == cudaSuccess) ce = make_room(r->in, off_bytes + cap_bytes);
+  if (ce == cudaSuccess && off_bytes) ce = cudaMemcpyAsync(r->in.p, job_off, off_bytes, cudaMemcpyDeviceToHost, r->stream);
+  r->open = ce == cudaSuccess;
+  if (ce == cudaSuccess && cap_bytes) ce = cudaMemcpyAsync(reinterpret_cast<unsigned char*>(r->in.p) + off_bytes, capacity, cap_bytes, cudaMemcpyDeviceToHost, r->stream);
   if (ce != cudaSuccess) {
-    if (z.open) cudaStreamSynchronize(z.stream);
-    z.open = false;
-    return fail_cuda(ctx, ce, "read of the sizes");
+    if (r->open) cudaStreamSynchronize(r->stream);
+    r->open = false;
+    return fail_cuda(r, ce, "read of the sizes");
   }
   return KVS_OK;
 }
 
-static int sizes_end(kvs_ctx* ctx, const kvs_setting* settings, int64_t P, int64_t* job_out_off, int64_t* profile_off, kvs_sizes* out) {
-  kvs_ctx::Sizes& z = ctx->sizes;
-  if (!z.open) return fail(ctx, KVS_E_STATE, "sizes: not begun");
-  z.open = false;
-  cudaError_t ce = cudaStreamSynchronize(z.stream);
-  if (ce != cudaSuccess) return fail_cuda(ctx, ce, "read of the sizes");
-  if (P < 0 || (job_out_off && (z.n_off < 1 || (P > 0 && !settings))) || (profile_off && z.n_cap != P)) return fail(ctx, KVS_E_ARG, "sizes: not those that were asked for");
-  const int64_t *off = z.p, *cap = z.p + (z.n_off > 0 ? z.n_off : 0);
+static int sizes_end(kvs_reader* r, const kvs_setting* settings, int64_t P, int64_t* job_out_off, int64_t* profile_off, kvs_sizes* out) {
+  if (!r->open) return fail(r, KVS_E_STATE, "sizes: not begun");
+  r->open = false;
+  cudaError_t ce = cudaSetDevice(r->device);
+  const cudaError_t waited = cudaStreamSynchronize(r->stream);
+  if (ce == cudaSuccess) ce = waited;
+  if (ce != cudaSuccess) return fail_cuda(r, ce, "read of the sizes");
+  if (P < 0 || (job_out_off && (r->n_off < 1 || (P > 0 && !settings))) || (profile_off && r->n_cap != P)) return fail(r, KVS_E_ARG, "sizes: not those that were asked for");
+  const int64_t *off = r->in.p, *cap = r->in.p + (r->n_off > 0 ? r->n_off : 0);
   kvs_sizes s{};
-  for (int64_t i = 0; i + 1 < z.n_off; ++i) s.max_jobs = std::max(s.max_jobs, off[i + 1] - off[i]);
+  for (int64_t i = 0; i + 1 < r->n_off; ++i) s.max_jobs = std::max(s.max_jobs, off[i + 1] - off[i]);
   if (job_out_off)
     for (int64_t e = 0; e < P; ++e)
-      if (settings[e].instance < 0 || settings[e].instance + 1 >= z.n_off) return fail(ctx, KVS_E_ARG, "settings: instance out of range");
+      if (settings[e].instance < 0 || settings[e].instance + 1 >= r->n_off) return fail(r, KVS_E_ARG, "settings: instance out of range");
   if (job_out_off || profile_off) {
     const size_t row = static_cast<size_t>(P) + 1;
-    kvs_ctx::Stage* stg = nullptr;
-    if ((ce = take_stage(ctx, 16 * row, &stg)) != cudaSuccess) return fail_cuda(ctx, ce, "staging");
-    int64_t* const rows = reinterpret_cast<int64_t*>(stg->p);
+    if (r->sending && (ce = cudaEventSynchronize(r->sent)) != cudaSuccess) return fail_cuda(r, ce, "copy of the offsets");
+    r->sending = false;
+    if ((ce = make_room(r->rows, 16 * row)) != cudaSuccess) return fail_cuda(r, ce, "cudaMallocHost");
+    int64_t* const rows = r->rows.p;
     auto fill = [&](int64_t* at, auto count) {
       int64_t sum = 0;
       for (int64_t e = 0; e < P; ++e) { at[e] = sum; sum += count(e); }
@@ -823,21 +868,23 @@ static int sizes_end(kvs_ctx* ctx, const kvs_setting* settings, int64_t P, int64
     if (job_out_off) s.job_results = fill(rows, [&](int64_t e) { return off[settings[e].instance + 1] - off[settings[e].instance]; });
     if (profile_off) s.profile_rounds = fill(rows + row, [&](int64_t e) { return cap[e]; });
     if (job_out_off && profile_off == job_out_off + row) {               // one piece
-      ce = cudaMemcpyAsync(job_out_off, rows, 16 * row, cudaMemcpyHostToDevice, z.stream);
+      ce = cudaMemcpyAsync(job_out_off, rows, 16 * row, cudaMemcpyHostToDevice, r->stream);
     } else {
-      if (job_out_off) ce = cudaMemcpyAsync(job_out_off, rows, 8 * row, cudaMemcpyHostToDevice, z.stream);
-      if (ce == cudaSuccess && profile_off) ce = cudaMemcpyAsync(profile_off, rows + row, 8 * row, cudaMemcpyHostToDevice, z.stream);
+      if (job_out_off) ce = cudaMemcpyAsync(job_out_off, rows, 8 * row, cudaMemcpyHostToDevice, r->stream);
+      if (ce == cudaSuccess && profile_off) ce = cudaMemcpyAsync(profile_off, rows + row, 8 * row, cudaMemcpyHostToDevice, r->stream);
     }
-    const cudaError_t marked = mark_stage(stg, z.stream);
+    const cudaError_t marked = cudaEventRecord(r->sent, r->stream);
+    r->sending = marked == cudaSuccess;
+    if (!r->sending) cudaStreamSynchronize(r->stream);                   // no event to wait for later
     if (ce == cudaSuccess) ce = marked;
-    if (ce != cudaSuccess) return fail_cuda(ctx, ce, "copy of the offsets");
+    if (ce != cudaSuccess) return fail_cuda(r, ce, "copy of the offsets");
   }
   if (out) *out = s;
   return KVS_OK;
 }
-int kvs_sizes_end(kvs_ctx* ctx, const kvs_setting* settings, int64_t P, int64_t* job_out_off, int64_t* profile_off, kvs_sizes* out) {
-  if (!ctx) return KVS_E_STATE;
-  return guarded(ctx, [&] { return sizes_end(ctx, settings, P, job_out_off, profile_off, out); });
+int kvs_sizes_end(kvs_reader* r, const kvs_setting* settings, int64_t P, int64_t* job_out_off, int64_t* profile_off, kvs_sizes* out) {
+  if (!r) return KVS_E_STATE;
+  return guarded(r, [&] { return sizes_end(r, settings, P, job_out_off, profile_off, out); });
 }
 
 const char* kvs_last_error(const kvs_ctx* ctx) { return ctx ? ctx->err.c_str() : "no context"; }

@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <new>
 #include <random>
 #include <string>
@@ -30,6 +31,7 @@ struct Op { std::string name; int stream; long seq; Clock clock; std::vector<Acc
 
 std::vector<Stream*> streams;
 std::vector<Op> ops;
+std::map<const unsigned char*, size_t> locked;                     // page-locked memory
 Clock host;
 int calls = 0, fail_at = -1, races = 0;
 long news = 0, no_memory_at = -1;      // allocations of the library's host code while `library` is set, and the one that fails
@@ -141,8 +143,25 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
   return cudaSuccess;
 }
 cudaError_t cudaEventSynchronize(cudaEvent_t e) { host.join(reinterpret_cast<Event*>(e)->clock); return fails() ? cudaErrorUnknown : cudaSuccess; }
-cudaError_t cudaMallocHost(void** p, size_t n) { if (fails()) return cudaErrorUnknown; *p = calloc(1, n); return cudaSuccess; }
-cudaError_t cudaFreeHost(void* p) { free(p); return cudaSuccess; }
+cudaError_t cudaMallocHost(void** p, size_t n) {
+  Outside outside;
+  if (fails()) return cudaErrorUnknown;
+  *p = calloc(1, n);
+  locked[static_cast<unsigned char*>(*p)] = n;
+  return cudaSuccess;
+}
+// Memory that is given back is in no operation that the host has not waited for.
+cudaError_t cudaFreeHost(void* p) {
+  Outside outside;
+  const unsigned char* a = static_cast<const unsigned char*>(p);
+  const unsigned char* b = a + locked[a];
+  for (const Op& o : ops)
+    for (const Access& x : o.acc)
+      if (x.a < b && a < x.b && !before(o, host) && races++ < 5) printf("%s on stream %d is in flight where page-locked memory is given back\n", o.name.c_str(), o.stream);
+  locked.erase(a);
+  free(p);
+  return cudaSuccess;
+}
 cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t n, cudaMemcpyKind, cudaStream_t s) {
   Outside outside;
   if (fails()) return cudaErrorUnknown;
@@ -311,6 +330,39 @@ int device_call(Caller& c, const Batch& b) {
   return rc;
 }
 
+// What a program does that does not know its sizes: they are read and the offsets formed, then the call is made.
+int sized_call(Caller& c, kvs_reader* r, const Batch& b) {
+  const i64 P = static_cast<i64>(b.st.size());
+  std::vector<i64> cap, offsets(2 * static_cast<size_t>(P) + 2);
+  for (i64 e = 0; e < P; ++e) cap.push_back(e % 7);
+  i64 *const job_off = offsets.data(), *const prof_off = job_off + P + 1;
+  kvs_sizes sizes{};
+  library = true;
+  int rc = kvs_sizes_begin(r, nullptr, b.off.data(), b.I, cap.data(), P);
+  if (rc == KVS_OK) rc = kvs_sizes_end(r, b.st.data(), P, job_off, prof_off, &sizes);
+  library = false;
+  if (rc != KVS_OK) return rc;
+  i64 jobs = 0, rounds = 0;
+  for (i64 e = 0; e < P; ++e) {
+    const i64 inst = b.st[static_cast<size_t>(e)].instance;
+    if (job_off[e] != jobs || prof_off[e] != rounds) { printf("offsets of evaluation %ld: %ld, %ld\n", static_cast<long>(e), static_cast<long>(job_off[e]), static_cast<long>(prof_off[e])); ++races; break; }
+    jobs += b.off[static_cast<size_t>(inst) + 1] - b.off[static_cast<size_t>(inst)];
+    rounds += cap[static_cast<size_t>(e)];
+  }
+  if (sizes.max_jobs != JOBS || sizes.job_results != jobs || sizes.profile_rounds != rounds) { printf("wrong sizes\n"); ++races; }
+  std::vector<int32_t> start(static_cast<size_t>(jobs)), done(start.size());
+  std::vector<i64> peak(static_cast<size_t>(P));
+  kvs_schedule_out out{};
+  out.job_out_off = job_off; out.job_start = start.data(); out.job_completion = done.data();
+  kvs_eval_out ev{};
+  ev.peak = peak.data();
+  const kvs_instances in = view(b);
+  library = true;
+  rc = kvs_evaluate_built(c.ctx, &in, b.st.data(), P, &out, &ev);
+  library = false;
+  return rc;
+}
+
 void run_host(const char* name, const Batch& b) {
   Caller c(b.I, static_cast<i64>(b.st.size()));
   const int r0 = races;
@@ -344,6 +396,49 @@ void overlaps() {
   }
 }
 
+// Requests for sizes: several at a time on readers of their own, one at a time on one reader, sizes that grow, readers on two streams.
+void sizes() {
+  Caller c(1, 1);
+  auto expect = [&](const char* what, bool ok) { if (!ok) { printf("%s\n", what); ++races; } };
+  kvs_reader *x = nullptr, *y = nullptr;
+  expect("open", kvs_reader_open(0, &x) == KVS_OK && kvs_reader_open(0, &y) == KVS_OK && kvs_reader_open(1, nullptr) == KVS_E_ARG);
+  const std::vector<i64> a = {0, 3, 7}, b = {0, 50, 90}, cap = {11, 0};
+  kvs_setting st[2]{};
+  st[1].instance = 1;
+  kvs_sizes sa{}, sb{};
+  std::vector<i64> oa(3), ob(3), pa(3);
+  // interleaved: each end is that of its own begin
+  expect("begin", kvs_sizes_begin(x, nullptr, a.data(), 2, cap.data(), 2) == KVS_OK && kvs_sizes_begin(y, nullptr, b.data(), 2, nullptr, 0) == KVS_OK);
+  expect("a second begin is refused", kvs_sizes_begin(x, nullptr, b.data(), 2, nullptr, 0) == KVS_E_STATE && kvs_reader_error(x)[0] != 0);
+  expect("end", kvs_sizes_end(x, st, 2, oa.data(), pa.data(), &sa) == KVS_OK && kvs_sizes_end(y, st, 2, ob.data(), nullptr, &sb) == KVS_OK);
+  expect("sizes of the first", sa.max_jobs == 4 && sa.job_results == 7 && sa.profile_rounds == 11 && oa == a && pa == std::vector<i64>({0, 11, 11}));
+  expect("sizes of the second", sb.max_jobs == 50 && sb.job_results == 90 && sb.profile_rounds == 0 && ob == b);
+  expect("an end without a begin is refused", kvs_sizes_end(x, st, 2, oa.data(), nullptr, &sa) == KVS_E_STATE);
+  // a request that is refused at its end is over
+  st[1].instance = 2;
+  kvs_sizes_begin(x, nullptr, a.data(), 2, nullptr, 0);
+  expect("instance out of range", kvs_sizes_end(x, st, 2, oa.data(), nullptr, &sa) == KVS_E_ARG);
+  kvs_sizes_begin(x, nullptr, a.data(), 2, nullptr, 0);
+  expect("capacities that were not asked for", kvs_sizes_end(x, st, 2, nullptr, pa.data(), &sa) == KVS_E_ARG);
+  expect("the next request", kvs_sizes_begin(x, nullptr, a.data(), 2, nullptr, 0) == KVS_OK && kvs_sizes_end(x, st, 1, oa.data(), nullptr, &sa) == KVS_OK && oa[1] == 3);
+  // requests of growing size under two streams in turn: what one uploads is not overwritten by the next
+  cudaStream_t other = nullptr;
+  cudaStreamCreateWithFlags(&other, 0);
+  std::vector<std::vector<i64>> keep;
+  for (int i = 1; i < 6; ++i) {
+    const size_t P = static_cast<size_t>(200) << (2 * i);
+    keep.emplace_back(P, 3);
+    keep.emplace_back(P + 1, 0);
+    expect("a request", kvs_sizes_begin(x, i % 2 ? other : nullptr, nullptr, 0, keep[keep.size() - 2].data(), static_cast<i64>(P)) == KVS_OK &&
+                            kvs_sizes_end(x, nullptr, static_cast<i64>(P), nullptr, keep.back().data(), &sa) == KVS_OK && sa.profile_rounds == 3 * static_cast<i64>(P));
+  }
+  find_races();
+  kvs_sizes_begin(y, nullptr, b.data(), 2, nullptr, 0);
+  kvs_reader_close(y);
+  kvs_reader_close(x);
+  if (const int n = outstanding(host)) { printf("%d operations in flight\n", n); ++races; }
+}
+
 // A refused call enqueues nothing; a call that fails half-way (every fallible call of the runtime, every launch and every
 // allocation in turn) returns a status and leaves nothing behind that the next call could meet.
 void errors() {
@@ -360,16 +455,20 @@ void errors() {
     if (host_call(c, bad) != KVS_E_ARG || !ops.empty()) { printf("family %d: %zu operations of a refused call\n", family, ops.size()); ++races; }
     next_call("refused", c);
   }
+  enum { HOST, DEVICE, SIZED };
   for (bool memory : {false, true})
-    for (bool device : {false, true}) {
+    for (int kind : {HOST, DEVICE, SIZED}) {
+      const bool device = kind != HOST;
       int rc = KVS_E_CUDA, n = 0;
       for (; rc != KVS_OK && n < 2000; ++n) {
         Caller c(b.I, static_cast<i64>(b.st.size()));
+        kvs_reader* r = nullptr;
+        if (kvs_reader_open(0, &r) != KVS_OK) { printf("kvs_reader_open failed\n"); exit(2); }
         calls = 0;
         news = 0;
         no_memory_at = memory ? n : -1;
         fail_at = memory ? -1 : n;
-        rc = device ? device_call(c, b) : host_call(c, b);
+        rc = kind == SIZED ? sized_call(c, r, b) : (device ? device_call(c, b) : host_call(c, b));
         fail_at = -1;
         no_memory_at = -1;
         if (rc != KVS_OK && rc != (memory ? KVS_E_STATE : KVS_E_CUDA)) { printf("status %d\n", rc); ++races; }
@@ -377,9 +476,15 @@ void errors() {
         if (const int left = outstanding(device ? stream_of(nullptr)->clock : host)) {
           if (races++ < 5) printf("%s call, failure %d: %d operations in flight\n", device ? "device" : "host", n, left);
         }
+        if (kind == SIZED) {
+          // the reader is ready for another request, or is given back with its last one in flight
+          if (n % 2 && sized_call(c, r, b) != KVS_OK) { printf("the reader's next request fails\n"); ++races; }
+          if (n % 3 == 0) kvs_sizes_begin(r, nullptr, b.off.data(), b.I, nullptr, 0);
+        }
+        kvs_reader_close(r);
         next_call("after a failure", c);
       }
-      const int least = memory ? (device ? 1 : 4) : (device ? 10 : 80);
+      const int least = memory ? (device ? 1 : 4) : (kind == SIZED ? 18 : (device ? 10 : 80));
       if (n < least || n == 2000) { printf("%d failures\n", n); ++races; }
     }
 }
@@ -390,6 +495,7 @@ int main(int argc, char** argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "overlaps") overlaps();
   else if (what == "errors") errors();
+  else if (what == "sizes") sizes();
   else { printf("unknown program\n"); return 2; }
   printf("%s: %d faults\n", what.c_str(), races);
   return races ? 1 : 0;

@@ -33,3 +33,9 @@ def test_failures_leave_nothing_in_flight(program):
     """A refused call launches nothing; after one that fails at any point (a runtime call, a launch, host memory), no kernel and no
     copy of it is left for the next call to race with, and no exception leaves the C entry point."""
     _run(program, "errors")
+
+
+def test_requests_for_sizes_belong_to_their_reader(program):
+    """Requests that overlap each get their own sizes; one reader refuses a second request; page-locked memory is neither overwritten nor
+    given back while a copy uses it."""
+    _run(program, "sizes")
