@@ -175,7 +175,8 @@ typedef struct {
  * `capacity` (DEVICE [P]; either may be NULL) to page-locked memory behind what `stream` (a cudaStream_t) holds.  kvs_sizes_end
  * waits for that, fills `out` and uploads, on the same stream, the offsets 0, c_0, c_0 + c_1, .. of the evaluations' job
  * results (`job_out_off`, DEVICE [P + 1]; the jobs of each setting's instance) and profiles (`profile_off`, DEVICE [P + 1]);
- * either may be NULL.  A setting that names no instance of the batch is refused (KVS_E_ARG) before any indexing.
+ * either may be NULL.  A setting that names no instance of the batch is refused (KVS_E_ARG) before any indexing, and so is
+ * a negative capacity; an instance whose offsets decrease, which the call then reports as bad input, has no job results.
  *
  * A request belongs to a reader, which no context shares: page-locked memory of its own for one request at a time.  A request that
  * has been begun is ended, whatever kvs_sizes_end returns, before the next one is begun on the same reader; a begin in between

@@ -854,6 +854,9 @@ static int sizes_end(kvs_reader* r, const kvs_setting* settings, int64_t P, int6
   if (job_out_off)
     for (int64_t e = 0; e < P; ++e)
       if (settings[e].instance < 0 || settings[e].instance + 1 >= r->n_off) return fail(r, KVS_E_ARG, "settings: instance out of range");
+  // a negative count would move the offsets behind it in front of what is reserved for them
+  for (int64_t e = 0; e < r->n_cap; ++e)
+    if (cap[e] < 0) return fail(r, KVS_E_ARG, "sizes: negative capacity");
   if (job_out_off || profile_off) {
     const size_t row = static_cast<size_t>(P) + 1;
     if (r->sending && (ce = cudaEventSynchronize(r->sent)) != cudaSuccess) return fail_cuda(r, ce, "copy of the offsets");
@@ -865,7 +868,7 @@ static int sizes_end(kvs_reader* r, const kvs_setting* settings, int64_t P, int6
       for (int64_t e = 0; e < P; ++e) { at[e] = sum; sum += count(e); }
       return at[P] = sum;
     };
-    if (job_out_off) s.job_results = fill(rows, [&](int64_t e) { return off[settings[e].instance + 1] - off[settings[e].instance]; });
+    if (job_out_off) s.job_results = fill(rows, [&](int64_t e) { return std::max<int64_t>(0, off[settings[e].instance + 1] - off[settings[e].instance]); });
     if (profile_off) s.profile_rounds = fill(rows + row, [&](int64_t e) { return cap[e]; });
     if (job_out_off && profile_off == job_out_off + row) {               // one piece
       ce = cudaMemcpyAsync(job_out_off, rows, 16 * row, cudaMemcpyHostToDevice, r->stream);

@@ -421,6 +421,15 @@ void sizes() {
   kvs_sizes_begin(x, nullptr, a.data(), 2, nullptr, 0);
   expect("capacities that were not asked for", kvs_sizes_end(x, st, 2, nullptr, pa.data(), &sa) == KVS_E_ARG);
   expect("the next request", kvs_sizes_begin(x, nullptr, a.data(), 2, nullptr, 0) == KVS_OK && kvs_sizes_end(x, st, 1, oa.data(), nullptr, &sa) == KVS_OK && oa[1] == 3);
+  // sizes below zero: none of the offsets precedes the one before it
+  const std::vector<i64> negative = {5, -1}, falling = {0, 4, 1, 3};
+  kvs_sizes_begin(x, nullptr, nullptr, 0, negative.data(), 2);
+  expect("a negative capacity is refused", kvs_sizes_end(x, nullptr, 2, nullptr, pa.data(), &sa) == KVS_E_ARG);
+  kvs_setting three[3]{};
+  for (int i = 0; i < 3; ++i) three[i].instance = i;
+  std::vector<i64> of(4);
+  kvs_sizes_begin(x, nullptr, falling.data(), 3, nullptr, 0);
+  expect("falling offsets", kvs_sizes_end(x, three, 3, of.data(), nullptr, &sa) == KVS_OK && of == std::vector<i64>({0, 4, 4, 6}) && sa.max_jobs == 4);
   // requests of growing size under two streams in turn: what one uploads is not overwritten by the next
   cudaStream_t other = nullptr;
   cudaStreamCreateWithFlags(&other, 0);

@@ -495,3 +495,25 @@ def test_sizes_read_by_the_library(par):
     with pytest.raises(binding.KvsError):
         sch.evaluate(inst, st, want_profile=True, profile_capacity=cap[:-1])
     assert torch.equal(sch.evaluate(inst, st).flow, par.scheduler().evaluate(inst, st, want_jobs=False).flow)
+
+
+def test_negative_sizes(par):
+    """A negative capacity is refused before any launch, on both ways that sizes take; an instance whose offsets decrease is bad input with no
+    job results, those behind it are as they are by themselves."""
+    one = workloads.random_small(8400, 3, 50, 30, 60)
+    inst, st = one.to("cuda:0"), binding.settings_grid(range(3), ["GBA", "GSA"], [3_000])
+    for kind in (torch.int64, torch.int32):
+        for at in (0, 5):
+            cap = torch.full((6,), 1 << 12, dtype=kind, device="cuda:0")
+            cap[at] = -1
+            with pytest.raises(binding.KvsError):
+                par.scheduler().evaluate(inst, st, want_profile=True, profile_capacity=cap)
+    off = one.job_off
+    falling = workloads.Instances(torch.stack([off[1], off[0], off[1], off[3]]).to("cuda:0"), inst.s, inst.o)
+    apart = workloads.Instances(torch.stack([off[0], off[1], off[3]]).to("cuda:0"), inst.s, inst.o)
+    want = par.scheduler().evaluate(apart, binding.settings_grid(range(2), ["GBA", "GSA"], [3_000]))
+    for wide in (False, True):
+        got = par.scheduler().evaluate(falling, st, time64=wide)
+        assert got.status.tolist()[:2] == [binding.EVAL_BAD_INPUT] * 2 and got.job_out_off.tolist()[:3] == [0, 0, 0]
+        assert torch.equal(got.job_start, want.job_start.to(got.job_start.dtype)) and torch.equal(got.job_completion, want.job_completion.to(got.job_start.dtype))
+        assert torch.equal(got.flow[2:], want.flow)

@@ -72,6 +72,15 @@ def test_capacities_of_the_wrong_shape_are_refused():
             Scheduler._per_eval(wrong, 3, "capacity")
 
 
+def test_negative_capacities_are_refused():
+    """An offset formed from one would lie in front of what is reserved."""
+    from paper_2601_22996_b200.api import Scheduler
+    assert Scheduler._per_eval(np.zeros(0, np.int64), 0, "capacity").size == 0
+    for wrong in (np.array([-1, 5, 5]), np.array([5, 5, -1])):
+        with pytest.raises(binding.KvsError):
+            Scheduler._per_eval(wrong, 3, "capacity")
+
+
 def test_generators_are_deterministic_and_in_range():
     a, b = workloads.config2(n_inst=3, n=500), workloads.config2(n_inst=3, n=500)
     assert torch.equal(a.s, b.s) and torch.equal(a.o, b.o)
