@@ -335,7 +335,8 @@ __global__ void __launch_bounds__(RT) k_refill(RefillParams p) {
   // the ring goes back to the plan, the rest of which holds the remaining jobs' old ramps only
   const int next = sh_next, filled = sh_filled;
   const bool tail = next < n;
-  const int g_next = tail ? js[perm[next]] : H;
+  const int j_next = tail ? perm[next] : 0;
+  const int g_next = tail && KVS_OK_AT(j_next, n, CHK_RF_JOB) ? js[j_next] : H;
   for (int u = sh_prev + tid; u < min(filled, H); u += RT)
     if (KVS_OK_AT(u, pcap, CHK_RF_PROF_OUT)) prof[u] = ring[u & (RING - 1)];
   for (int u = filled + tid; u < min(g_next, H); u += RT)

@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(ST) k_spec(SpecParams p) {
           const int q = q0 + lane;
           bool keep = false;
           int j = 0;
-          if (q < np) { j = list[q]; keep = cls[j] >= ph; }
+          if (q < np && KVS_OK_AT(q, n, CHK_SP_LIST)) { j = list[q]; keep = KVS_OK_AT(j, n, CHK_SP_JOB) && cls[j] >= ph; }
           const unsigned m = __ballot_sync(0xffffffffu, keep);
           __syncwarp();
           if (keep) { const int d = w + __popc(m & lt_mask); list[d] = j; pos_of[j] = d; }
@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(ST) k_spec(SpecParams p) {
               const int qq = q0 + lane;
               bool live = false;
               int jj = 0, ff = 0;
-              if (qq < top) { jj = stk_job[qq]; ff = stk_fin[qq]; live = sst[jj] == static_cast<int>(static_cast<u32>(ff) - static_cast<u32>(O[jj])); }
+              if (qq < top) { jj = stk_job[qq]; ff = stk_fin[qq]; live = KVS_OK_AT(jj, n, CHK_SP_JOB) && sst[jj] == static_cast<int>(static_cast<u32>(ff) - static_cast<u32>(O[jj])); }
               const unsigned lm = __ballot_sync(0xffffffffu, live);
               __syncwarp();
               if (live) { const int d = w + __popc(lm & lt_mask); stk_job[d] = jj; stk_fin[d] = ff; }
@@ -614,8 +614,11 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
   unsigned start_mask = 0, end_mask = 0, start_masks = 0, end_masks = 0;
   bool all_take_part = true;                            // rank = job index: no list yet
   u32 ahead_start = 0, ahead_end = 0;                   // list entries of ranks rs + lane and re + lane, read ahead
+  // a job number that was read from the list or the stack (checked build: 0 if it is none)
+  auto job_at = [&](u32 j) { return KVS_OK_AT(j, n, CHK_SP_JOB) ? j : 0u; };
+  auto list_at = [&](int r) { return KVS_OK_AT(r, n, CHK_SP_LIST) ? job_at(list[r]) : 0u; };
   // job of rank r < np
-  auto job_of = [&](int r) { return all_take_part ? static_cast<u32>(r) : static_cast<u32>(list[r]); };
+  auto job_of = [&](int r) { return all_take_part ? job_at(static_cast<u32>(r)) : list_at(r); };
   int phase_at = L > 1 && sh.np[1] > 0 ? sh.pbase[1] : NEVER;   // first round of the next phase
   u32 A = 0;                                            // speculative runs hold A + t * cnt tokens in round t (modulo 2^32)
   int cnt = 0, top = 0;                                 // running speculative runs; entries on the stack (some stale)
@@ -703,7 +706,7 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
     for (int c = 0, r0 = rs; r0 < r_hi; ++c, r0 += 32) {
       const int r = r0 + lane;
       const bool on = r < r_hi;
-      const u32 j = !on ? 0u : (all_take_part ? static_cast<u32>(r) : (read && c == 0 ? ahead_start : static_cast<u32>(list[r])));
+      const u32 j = !on ? 0u : (all_take_part ? job_at(static_cast<u32>(r)) : (read && c == 0 ? ahead_start : list_at(r)));
       const u32 so = lengths[j], o = so >> 16, s1 = (so & 0xffffu) + 1u;
       const bool drop = on && is_done(j);
       const int q = ph.start_of(r);
@@ -744,7 +747,7 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
     for (int c = 0, r0 = re; r0 < e_hi; ++c, r0 += 32) {
       const int r = r0 + lane;
       const bool on = r < e_hi;
-      const u32 j = !on ? 0u : (all_take_part ? static_cast<u32>(r) : (read && c == 0 ? ahead_end : static_cast<u32>(list[r])));
+      const u32 j = !on ? 0u : (all_take_part ? job_at(static_cast<u32>(r)) : (read && c == 0 ? ahead_end : list_at(r)));
       const unsigned live = __ballot_sync(0xffffffffu, on && !is_done(j));
       if (live && ne == NEVER) {
         end_mask = live;
@@ -757,8 +760,8 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
     }
     re = e_hi;
     if (!all_take_part) {
-      if (rs + lane < ph.np) ahead_start = list[rs + lane];
-      if (re + lane < ph.np) ahead_end = list[re + lane];
+      if (rs + lane < ph.np) ahead_start = list_at(rs + lane);
+      if (re + lane < ph.np) ahead_end = list_at(re + lane);
     }
     __syncwarp();
   };
@@ -810,7 +813,7 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
 #pragma unroll
       for (int i = 0; i < U; ++i) {
         const int q = q0 + 32 * i + lane;
-        j[i] = q < top ? stk[q] : 0u;
+        j[i] = q < top && KVS_OK_AT(q, m, CHK_SP_STACK) ? job_at(stk[q]) : 0u;
         sm[i] = q < top ? sst[j[i]] : IDLE;
         place[i] = js[j[i]];
       }
@@ -819,8 +822,8 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
       for (int i = 0; i < U; ++i) {
         const bool live = sm[i] != IDLE && place[i] == q0 + 32 * i + lane;
         const unsigned lm = __ballot_sync(0xffffffffu, live);
-        if (live) {
-          const int d = w + __popc(lm & lt_mask);
+        const int d = w + __popc(lm & lt_mask);
+        if (live && KVS_OK_AT(d, m, CHK_SP_STACK)) {
           stk[d] = static_cast<unsigned short>(j[i]);
           js[j[i]] = d;
           atomicMin(&first_fin[d / STK_BLK], static_cast<u32>(t) + (lengths[j[i]] >> 16) - running_for(sm[i]));
@@ -867,7 +870,7 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
           const int b = b0 + __ffs(static_cast<int>(due)) - 1, q = b * STK_BLK + 2 * lane;
           due &= due - 1u;
           const u32 both = q < top ? *reinterpret_cast<const u32*>(stk + q) : 0u;
-          const u32 j0 = both & 0xffffu, j1 = q + 1 < top ? both >> 16 : 0u;
+          const u32 j0 = job_at(both & 0xffffu), j1 = q + 1 < top ? job_at(both >> 16) : 0u;
           const u32 sm0 = q < top ? sst[j0] : IDLE, sm1 = q + 1 < top ? sst[j1] : IDLE, so0 = lengths[j0], so1 = lengths[j1];
           const u32 ran0 = running_for(sm0), ran1 = running_for(sm1), o0 = so0 >> 16, o1 = so1 >> 16;
           const bool fin0 = sm0 != IDLE && ran0 == o0, fin1 = sm1 != IDLE && ran1 == o1;
@@ -949,7 +952,8 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
         const bool keep = q < ph.np && lengths[j] >> 16 > ph.tau;
         const unsigned km = __ballot_sync(0xffffffffu, keep);
         __syncwarp();
-        if (keep) list[kept + __popc(km & lt_mask)] = static_cast<unsigned short>(j);
+        const int d = kept + __popc(km & lt_mask);
+        if (keep && KVS_OK_AT(d, n, CHK_SP_LIST)) list[d] = static_cast<unsigned short>(j);
         kept += __popc(km);
         __syncwarp();
       }
@@ -1095,7 +1099,8 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
     while (cnt > 0 && B + A + tu * static_cast<u32>(cnt) > Mu) {
       u32 j = 0, sm = IDLE;
       while (top > 0 && sm == IDLE) {                   // the live entry nearest to the top: no other of its job is above it
-        j = stk[--top];
+        --top;
+        j = KVS_OK_AT(top, m, CHK_SP_STACK) ? job_at(stk[top]) : 0u;
         sm = sst[j];
       }
       if (sm == IDLE) break;
@@ -1120,8 +1125,8 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
       if (cj == -1) {
         const int f = first_free();
         if (f < 0) { cj = -2; break; }
-        cj = fj = f;
-        cs = prompt(f);
+        cj = fj = static_cast<int>(job_at(static_cast<u32>(f)));
+        cs = prompt(cj);
         if (cs + 1 > room) break;
       }
       const u32 j = (static_cast<u32>(cj) & ~31u) + lane, bits = free_map[j >> 5], so = lengths[j];
@@ -1143,7 +1148,7 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
       const u32 fin = ok ? tu + (so >> 16) : NO_ROUND;
       if (ok) {
         const int d = top + __popc(okm & lt_mask);
-        if (KVS_OK_AT(d, m, CHK_SP_STACK)) {
+        if (KVS_OK_AT(d, m, CHK_SP_STACK) && KVS_OK_AT(j, n, CHK_SP_JOB)) {
           sst[j] = static_cast<unsigned short>(tm);
           stk[d] = static_cast<unsigned short>(j);
           js[j] = d;

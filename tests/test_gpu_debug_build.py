@@ -63,6 +63,14 @@ for i in range(heur.n_instances):
         rows += [dict(instance=i, family=f, M=M, alpha=((2, 1), (3, 2))[i % 2]) for f in ("GBAD", "GSAS")]
 parity.check_batch(heur, binding.make_settings(rows), want_runs=False, label="checked heuristics tiny")
 parity.check_batch(c2, binding.settings_grid(range(3), ["GBAD", "GSAS"], [1 << 17, 1 << 20, 1 << 24]), want_runs=False, label="checked heuristics config 2")
+# speculative runs of five budgets on one instance (lists of several phases, stacks that are purged, a map of more than 4,096 jobs) and of
+# responses beyond the ring of rounds
+c = torch.arange(4_097)
+many = workloads.Instances(torch.tensor([0, 4_097]), workloads.uniform_int(71, c, 0, 20), workloads.pareto_int(72, c, 3.0, 1.1, 1, 60))
+parity.check_batch(many, binding.settings_grid(range(1), ["GSAS"], [1 << 8, 1 << 9, 1 << 11, 1 << 14, 1 << 17]), want_runs=False, label="checked spec maps")
+c = torch.arange(900)
+long = workloads.Instances(torch.tensor([0, 900]), workloads.uniform_int(81, c, 0, 20), workloads.uniform_int(82, c, 2_100, 4_000))
+parity.check_batch(long, binding.settings_grid(range(1), ["GSAS", "GBAD"], [1 << 19]), want_runs=False, label="checked spec long")
 torch.cuda.synchronize()
 word, _ = binding.debug_check_word()
 print("CHECK_WORD", hex(word))
