@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "kvs_internal.cuh"
+#include "kvs_spec_shape.h"
 
 constexpr int KVS_HOST_CHUNKS = 16;   // the host entry point pipelines copies and kernels over at most this many chunks
 constexpr int KVS_CHUNK_EVALS = 512;  // of about this many evaluations
@@ -410,27 +411,33 @@ int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* se
   auto by_budget = [&](int64_t x, int64_t y) { return st_host[x].M < st_host[y].M; };
   std::stable_sort(after, after + n_refill, by_budget);
   std::stable_sort(after + n_refill, after + n_refill + n_spec, by_budget);
-  // The on-chip kernel of the speculative runs takes up to four evaluations of one instance per CTA.
+  // The on-chip kernel of the speculative runs takes a few evaluations of one instance per CTA, smallest budgets first.
   int64_t* const groups = reinterpret_cast<int64_t*>(stg->p + groups_at(P));
-  int64_t n_groups = 0;
-  // An SM holds at least two of its evaluations, or few have to take turns: else the 32 warps per SM of the other kernel make up for
-  // their slower rounds.  Config 2's lengths and budgets, 8,192 evaluations of 500 / 2,000 / 5,000 / 10,000 jobs: 16 / 36 / 100 / 174 ms
-  // on chip, 34 / 96 / 195 / 346 in memory; 16,000 jobs (two per SM), 512 / 4,096 evaluations: 34 / 211 against 189 / 338; 24,000 jobs
-  // (one per SM), 512 / 2,048 / 3,072 / 4,096 evaluations: 79 / 273 / 400 / 532 against 254 / 338 / 457 / 511.
-  int spec_per_cta = n_spec ? kvs_spec_per_cta(max_n) : 0;
-  if (spec_per_cta == 1 && n_spec > 24 * static_cast<int64_t>(ctx->sm_count)) spec_per_cta = 0;
-  if (spec_per_cta > 0) {
+  SpecShape shape;
+  if (n_spec) {
     std::vector<int64_t> by_inst(after + n_refill, after + n_refill + n_spec);
     std::stable_sort(by_inst.begin(), by_inst.end(), [&](int64_t x, int64_t y) { return st_host[x].instance < st_host[y].instance; });
-    std::vector<std::pair<size_t, size_t>> cut;           // [first, last) of by_inst, smallest budget first
-    for (size_t i = 0, j; i < by_inst.size(); i = j) {
-      for (j = i + 1; j < by_inst.size() && j - i < static_cast<size_t>(spec_per_cta) && st_host[by_inst[i]].instance == st_host[by_inst[j]].instance; ++j) {}
-      cut.emplace_back(i, j);
+    std::vector<int64_t> evals_of;
+    for (size_t i = 0; i < by_inst.size(); ++i) {
+      if (i == 0 || st_host[by_inst[i]].instance != st_host[by_inst[i - 1]].instance) evals_of.push_back(0);
+      ++evals_of.back();
     }
-    std::stable_sort(cut.begin(), cut.end(), [&](const auto& x, const auto& y) { return st_host[by_inst[x.first]].M < st_host[by_inst[y.first]].M; });
-    for (const auto& x : cut) {
-      int64_t* const g = groups + KVS_SPEC_GROUP * n_groups++;
-      for (size_t i = 0; i < KVS_SPEC_GROUP; ++i) g[i] = x.first + i < x.second ? by_inst[x.first + i] : -1;
+    shape = kvs_spec_shape(max_n, evals_of, ctx->sm_count);
+    if (shape.warps > 0) {
+      std::vector<std::pair<size_t, size_t>> cut;         // [first, last) of by_inst
+      size_t at = 0;
+      for (int64_t c : evals_of) {
+        const int64_t pieces = spec_groups(c, shape.warps);
+        for (int64_t g = 0; g < pieces; ++g) {
+          const size_t size = static_cast<size_t>(c / pieces + (g < c % pieces ? 1 : 0));
+          cut.emplace_back(at, at + size);
+          at += size;
+        }
+      }
+      std::stable_sort(cut.begin(), cut.end(), [&](const auto& x, const auto& y) { return st_host[by_inst[x.first]].M < st_host[by_inst[y.first]].M; });
+      for (size_t g = 0; g < cut.size(); ++g)
+        for (size_t i = 0; i < KVS_SPEC_GROUP; ++i)
+          groups[KVS_SPEC_GROUP * g + i] = cut[g].first + i < cut[g].second ? by_inst[cut[g].first + i] : -1;
     }
   }
   if (n_refill || n_spec) {
@@ -541,7 +548,7 @@ int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* se
       init[17 + 2 * f] = static_cast<unsigned long long>(full_of[f]);
     }
   }
-  const size_t upload = n_groups ? call_bytes(P) : (parts > 1 ? groups_at(P) : lists_bytes(P));
+  const size_t upload = shape.groups ? call_bytes(P) : (parts > 1 ? groups_at(P) : lists_bytes(P));
   ce = send_stage(stg, counters, upload, rg ? ctx->copy_stream : ctx->stream);
   if (ce != cudaSuccess) return fail_cuda(ctx, ce, "copy of the settings and evaluation lists");
   if (rg && (rc = rg->feed())) return rc;
@@ -695,7 +702,8 @@ int enqueue_fused(kvs_ctx* ctx, const kvs_instances* inst, const kvs_setting* se
     q.n_warps = std::min<i64>(std::min<i64>(room, want), q.n_list);
     q.counter = counters + 24;
     // (its lists of participants take less of the working storage than the CTA scratch of as many evaluations; otherwise the other kernel takes them all)
-    q.groups = reinterpret_cast<const i64*>(call + groups_at(P)); q.n_groups = n_groups * kvs_spec_group_bytes(max_n) <= q.scratch_bytes ? n_groups : 0;
+    q.groups = reinterpret_cast<const i64*>(call + groups_at(P)); q.n_groups = shape.groups * spec_list_bytes(max_n, shape.warps) <= q.scratch_bytes ? shape.groups : 0;
+    q.group_warps = shape.warps; q.ring = shape.ring;
     q.left_list = reinterpret_cast<i64*>(ws + L.slow_list); q.left_count = counters + 26;   // the general kernel has run: its list is free
     ce = kvs_launch_spec(q, ctx->stream);
     if (ce != cudaSuccess) return fail_cuda(ctx, ce, "launch of the speculative runs");

@@ -174,8 +174,10 @@ struct SpecParams {
   i64 max_jobs;
   i64 n_warps;                 // warps launched; each takes evaluations from the list until it is used up
   ull* counter;
-  const i64* groups;           // on-chip kernel: up to KVS_SPEC_GROUP evaluations of one instance per CTA (-1: none)
+  const i64* groups;           // on-chip kernel: KVS_SPEC_GROUP entries per CTA, its evaluations of one instance (-1: none)
   i64 n_groups;
+  int group_warps;             // evaluations that a CTA has room for
+  int ring;                    // rounds of the ring of each
   i64* left_list;              // evaluations that it leaves to the other kernel, and their number
   ull* left_count;
 };
@@ -211,9 +213,6 @@ cudaError_t kvs_launch_generic_tiled(GenericParams p, i64 capacity_total, int sm
 cudaError_t kvs_launch_generic(const GenericParams& p, cudaStream_t stream);
 cudaError_t kvs_launch_refill(const RefillParams& p, cudaStream_t stream);
 i64 kvs_spec_warp_bytes(i64 max_jobs);
-int kvs_spec_per_cta(i64 max_jobs);
-// Bytes of scratch that the on-chip kernel takes for a group: a 16-bit list of participants per evaluation.
-inline i64 kvs_spec_group_bytes(i64 max_jobs) { return 2ll * KVS_SPEC_GROUP * ((max_jobs + 127) & ~127ll); }
 cudaError_t kvs_setup_spec();
 // The caller zeroes the counters.
 cudaError_t kvs_launch_spec(SpecParams p, cudaStream_t stream);

@@ -23,6 +23,7 @@
 // moment; the events that free a job (a slot end, a kill for memory) widen that range, a scan narrows it.
 #include "kvs_check.cuh"
 #include "kvs_ladder.cuh"
+#include "kvs_spec_shape.h"
 
 namespace {
 
@@ -436,7 +437,7 @@ __global__ void __launch_bounds__(ST) k_spec(SpecParams p) {
 // What bounds a simulation is the chain of steps of its one warp, so what counts is the number of rounds at which the warp has to
 // stop, the dependent instructions of each stop, and the evaluations that an SM has in flight.  Instances of at most some 25,000
 // jobs (lengths below 2^16) fit on chip: 4 bytes a job of prompt and response lengths, which the warps of a CTA share (up to four
-// evaluations of one instance), and per evaluation 4 bytes a job - start of the speculative run, stack entry - and two bits.  Besides:
+// evaluations of one instance, see kvs_spec_shape), and per evaluation 4 bytes a job - start of the speculative run, stack entry - and two bits.  Besides:
 //   - a job that is free to start a speculative run has its bit set in a map by job index: the order of the participants is that
 //     of the indices and whoever is no participant any more is done, so the lowest free job is the first bit, found by one
 //     16-byte load a lane over 4,096 jobs; slot ends and kills set a bit and know at once whether it is the lowest;
@@ -450,15 +451,12 @@ __global__ void __launch_bounds__(ST) k_spec(SpecParams p) {
 //   - the stack keeps the earliest completion of every 64 entries, so that a completion looks at few entries;
 //   - sums that nothing in the simulation depends on are kept per lane.
 // Starts are kept modulo 65,535: a speculative run lasts less than that.
-// 512 evaluations (64 instances of 5,000 to 10,000 jobs, eight budgets), four per SM and all in flight: 17.6 ms, the chain of the longest
+// 512 evaluations (64 instances of 5,000 to 10,000 jobs, eight budgets), four per CTA and all in flight: 17.6 ms, the chain of the longest
 // one.  With every run's start and slot end a stop, list scans of 32 positions for the lowest free job and two evaluations per SM: 56.7 ms.
 
-constexpr int SPEC_WARPS = 4;            // evaluations of one CTA
-constexpr int RING_MAX = 1024, RING_MIN = 256;
 constexpr int FAR_SETS = 6;
 constexpr u32 IDLE = 0xffffu;            // sst: not running speculatively
 constexpr u32 MODT = 65535u;
-constexpr int STK_BLK = 64;
 constexpr int LOOK_AHEAD = 1024;         // runs that may start in a window whose runs are looked at together: a mask of 32 per lane
 
 // The phase table of one warp; the powers of the ladder lie where the stack will be.
@@ -469,17 +467,7 @@ struct alignas(16) SpecTable {
   u128 *pw_a, *pw_b;
 };
 
-// Bytes of one warp's state for instances of at most n jobs with a ring of that many rounds, and of the lengths that a CTA's warps share.
-__host__ __device__ inline int smem_jobs(int n) { return (n + 127) & ~127; }
-__host__ __device__ inline int smem_stack_bytes(int m) {
-  const int powers = 2 * (MAXP + 1) * static_cast<int>(sizeof(u128));
-  return 2 * m > powers ? 2 * m : powers;
-}
-__host__ __device__ inline int smem_state_bytes(int n, int ring) {
-  const int m = smem_jobs(n);
-  return static_cast<int>(sizeof(SpecTable)) + ring * 8 + smem_stack_bytes(m) + 2 * m + 2 * (m / 8) + ((m / STK_BLK * 4 + 15) & ~15);
-}
-__host__ __device__ inline int smem_lengths_bytes(int n) { return smem_jobs(n) * 4; }
+static_assert(sizeof(SpecTable) == SPEC_TABLE_BYTES && 2 * (MAXP + 1) * sizeof(u128) == SPEC_POWERS_BYTES, "bytes of a warp's state");
 
 // floor(x / d) by the multiplication with floor(2^64 / d) + 1 where x is below 2^32 (see slot_mul in kvs_fused.cu)
 __device__ __forceinline__ u32 div_by(u64 x, u32 d, u64 dinv) {
@@ -538,8 +526,9 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS) k_spec_smem(SpecParams p, int
     if (lane == 0 && mine >= 0) p.left_list[atomicAdd(p.left_count, 1ull)] = mine;
     return;
   }
-  unsigned short* const list = reinterpret_cast<unsigned short*>(p.scratch) + (SPEC_WARPS * static_cast<i64>(blockIdx.x) + warp) * m;   // kvs_spec_group_bytes a CTA
-  if (!KVS_OK_AT((SPEC_WARPS * static_cast<i64>(blockIdx.x) + warp + 1) * m * 2 - 1, p.scratch_bytes, CHK_SP_SCRATCH)) return;
+  const u32 among_all = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;     // (the stride as a parameter or a variable of its own: 17.74 instead of 17.64 ms)
+  unsigned short* const list = reinterpret_cast<unsigned short*>(p.scratch) + static_cast<i64>(among_all) * m;   // spec_list_bytes a CTA
+  if (!KVS_OK_AT((static_cast<i64>(among_all) + 1) * m * 2 - 1, p.scratch_bytes, CHK_SP_SCRATCH)) return;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     lengths[i] = static_cast<u32>(p.o[lo + i]) << 16 | static_cast<u32>(p.s[lo + i]);
   }
@@ -1209,33 +1198,15 @@ KVS_DEFINE_CHECK_WORD(kvs_spec_check_word)
 
 i64 kvs_spec_warp_bytes(i64 max_jobs) { return spec_stride(max_jobs); }
 
-constexpr int SPEC_SMEM = 227 * 1024;
-
-static int spec_ring(int n, int warps) {
-  for (int r = RING_MAX; r >= RING_MIN; r /= 2)
-    if (smem_lengths_bytes(n) + warps * smem_state_bytes(n, r) <= SPEC_SMEM) return r;
-  return 0;
-}
-
-// Evaluations of one instance that a CTA of the on-chip kernel takes: up to KVS_SPEC_GROUP, 0 where not even one fits.
-int kvs_spec_per_cta(i64 max_jobs) {
-  static_assert(KVS_SPEC_GROUP == SPEC_WARPS, "groups of evaluations");
-  if (max_jobs >= 65535) return 0;                      // 16-bit job numbers, one of them spare
-  for (int w = SPEC_WARPS; w >= 1; --w)
-    if (spec_ring(static_cast<int>(max_jobs), w)) return w;
-  return 0;
-}
-
 // Once per device, before the first launch.
 cudaError_t kvs_setup_spec() { return cudaFuncSetAttribute(k_spec_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, SPEC_SMEM); }
 
 // The on-chip kernel over p.groups, if there are any, and the other one over what it has left (or over the whole list).
 cudaError_t kvs_launch_spec(SpecParams p, cudaStream_t stream) {
   if (p.n_list <= 0 || p.n_warps <= 0) return cudaSuccess;
-  const int per_cta = p.n_groups > 0 ? kvs_spec_per_cta(p.max_jobs) : 0;
-  if (per_cta > 0) {
-    const int n = static_cast<int>(p.max_jobs), ring = spec_ring(n, per_cta);
-    k_spec_smem<<<static_cast<unsigned>(p.n_groups), 32 * per_cta, smem_lengths_bytes(n) + per_cta * smem_state_bytes(n, ring), stream>>>(p, n, ring);
+  if (p.n_groups > 0) {
+    const int n = static_cast<int>(p.max_jobs);
+    k_spec_smem<<<static_cast<unsigned>(p.n_groups), 32 * p.group_warps, spec_cta_bytes(n, p.group_warps, p.ring), stream>>>(p, n, p.ring);
   } else {
     p.left_list = nullptr;
   }

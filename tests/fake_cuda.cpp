@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "kvs_internal.cuh"
+#include "kvs_spec_shape.h"
 
 namespace {
 
@@ -190,7 +191,6 @@ cudaError_t kvs_setup_bounds() { return cudaSuccess; }
 cudaError_t kvs_setup_spec() { return cudaSuccess; }
 int kvs_build_ctas_per_sm() { return 2; }
 int kvs_fused_ctas_per_sm(int light) { return light ? 3 : 2; }
-int kvs_spec_per_cta(i64) { return 0; }
 i64 kvs_spec_warp_bytes(i64 n) { return 64 * (n + 64); }
 i64 kvs_order_chunks(i64 n) { return n / 4096 + 1; }
 i64 kvs_sweep_blocks(i64 n) { return n / 64 + 1; }
@@ -250,7 +250,14 @@ cudaError_t kvs_launch_build(const BuildParams& p, int grid, cudaStream_t s) {
 }
 static cudaError_t unused() { printf("a launch that these tests do not drive\n"); exit(2); }
 cudaError_t kvs_launch_refill(const RefillParams&, cudaStream_t) { return unused(); }
-cudaError_t kvs_launch_spec(SpecParams, cudaStream_t) { return unused(); }
+SpecParams spec_launched;
+std::vector<i64> spec_groups_launched;
+cudaError_t kvs_launch_spec(SpecParams p, cudaStream_t) {
+  Outside outside;
+  spec_launched = p;
+  spec_groups_launched.assign(p.groups, p.groups + KVS_SPEC_GROUP * p.n_groups);
+  return cudaSuccess;
+}
 cudaError_t kvs_launch_generic_tiled(GenericParams, i64, int, cudaStream_t) { return unused(); }
 cudaError_t kvs_launch_bounds(const i64*, const int32_t*, const int32_t*, i64, InstStats*, const kvs_setting*, i64, const i64*, i64, const kvs_bounds_out&, u32*, cudaStream_t) { return unused(); }
 cudaError_t kvs_launch_order_info(const i64*, const int32_t*, const int32_t*, i64, i64, OrderInfo*, int, cudaStream_t) { return unused(); }
@@ -285,12 +292,11 @@ struct Caller {
   kvs_ctx* ctx = nullptr;
   std::vector<unsigned char> memory;
   unsigned char* ws = nullptr;
-  explicit Caller(int I, i64 P) {
+  explicit Caller(int I, i64 P, uint64_t need = 0) {
     ops.clear();
     streams.clear();
     host = Clock{};
-    uint64_t need = 0;
-    kvs_workspace_bytes(static_cast<i64>(I) * JOBS, I, JOBS, P, 0, 1, &need);
+    if (!need) kvs_workspace_bytes(static_cast<i64>(I) * JOBS, I, JOBS, P, 0, 1, &need);
     memory.resize(need + 512);
     ws = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(memory.data()) + 255) & ~static_cast<uintptr_t>(255));
     kvs_init_params prm{};
@@ -448,6 +454,83 @@ void sizes() {
   if (const int n = outstanding(host)) { printf("%d operations in flight\n", n); ++races; }
 }
 
+// How a call's speculative runs are laid out: on which kernel, how many evaluations of an SM are in flight, groups of one instance
+// that hold every evaluation once.  `most`: evaluations of one instance that a CTA takes (0: none, all in memory); `live`: per SM.
+void spec_call(int jobs, const std::vector<int>& evals_of, int most, double live) {
+  const int r0 = races;
+  Batch b(static_cast<int>(evals_of.size()));
+  for (size_t i = 0; i < evals_of.size(); ++i)
+    for (int k = 0; k < evals_of[i]; ++k) { b.add(static_cast<int>(i), KVS_GSAS); b.st.back().M = 1000 + (7 * k + static_cast<int>(i)) % 50; }
+  const i64 P = static_cast<i64>(b.st.size());
+  uint64_t need = 0;
+  kvs_workspace_bytes(static_cast<i64>(b.I) * JOBS, b.I, jobs, P, 0, 1, &need);
+  Caller c(b.I, P, need);
+  kvs_instances in = view(b);
+  in.max_jobs_per_instance = jobs;
+  std::vector<i64> off(static_cast<size_t>(P) + 1, 0), peak(static_cast<size_t>(P)), horizon(peak.size());
+  std::vector<int32_t> out(1), status(peak.size());
+  alignas(16) static int32_t profile[4];
+  kvs_schedule_out so{};
+  so.job_out_off = off.data(); so.job_start = out.data(); so.job_completion = out.data();
+  kvs_eval_out ev{};
+  ev.profile_off = off.data(); ev.profile = profile; ev.peak = peak.data(); ev.horizon = horizon.data(); ev.status = status.data();
+  if (const int rc = kvs_evaluate_built(c.ctx, &in, b.st.data(), P, &so, &ev)) { printf("status %d\n", rc); ++races; return; }
+  const SpecParams& p = spec_launched;
+  std::vector<int> seen(static_cast<size_t>(P), 0);
+  i64 last = 0;
+  for (i64 g = 0; g < p.n_groups; ++g) {
+    const i64* e = spec_groups_launched.data() + KVS_SPEC_GROUP * g;
+    const kvs_setting& first = b.st[static_cast<size_t>(e[0])];
+    const i64 in_all = evals_of[static_cast<size_t>(first.instance)], least = in_all / spec_groups(in_all, p.group_warps);
+    i64 size = 0, budget = 0;
+    for (int i = 0; i < KVS_SPEC_GROUP; ++i) {
+      if (e[i] < 0) continue;
+      const kvs_setting& st = b.st[static_cast<size_t>(e[i])];
+      if (i != size++ || st.instance != first.instance || st.M < budget) { printf("group %ld\n", static_cast<long>(g)); ++races; }
+      budget = st.M;
+      ++seen[static_cast<size_t>(e[i])];
+    }
+    if (size > p.group_warps || size < least || size > least + 1 || first.M < last) { printf("group %ld: %ld evaluations\n", static_cast<long>(g), static_cast<long>(size)); ++races; }
+    last = first.M;
+  }
+  if (p.n_groups && std::count(seen.begin(), seen.end(), 1) != P) { printf("an evaluation is missing\n"); ++races; }
+  const i64 held = p.n_groups ? 148l * spec_resident(jobs, p.group_warps, p.ring) : 0;
+  const double found = p.n_groups ? static_cast<double>(P) / 148 * std::min(1.0, static_cast<double>(held) / static_cast<double>(p.n_groups)) : 0.0;
+  if (p.n_groups && (spec_cta_bytes(jobs, p.group_warps, p.ring) > 227 * 1024 || p.ring & (p.ring - 1) || p.ring < 256)) { printf("CTA\n"); ++races; }
+  if ((p.n_groups ? p.group_warps : 0) != most || found < live - 0.01) { printf("%d per CTA, %.2f per SM\n", p.n_groups ? p.group_warps : 0, found); ++races; }
+  if (races != r0) printf("jobs %d, %ld evaluations\n", jobs, static_cast<long>(P));
+}
+void groups() {
+  auto each = [](int instances, int evals) { return std::vector<int>(static_cast<size_t>(instances), evals); };
+  // one budget per instance: no CTA holds room for more than it has
+  for (int P : {1, 512, 2048, 8192}) {
+    spec_call(500, each(P, 1), 1, std::min(16.0, P / 148.0));
+    spec_call(5000, each(P, 1), 1, std::min(4.0, P / 148.0));
+  }
+  spec_call(10000, each(2048, 1), 1, 2.0);
+  // five: three and two, or none of them waits for a place
+  spec_call(10000, each(410, 5), 3, 2.5);
+  spec_call(5000, each(1639, 5), 2, 5.0);
+  spec_call(500, each(13, 5), 3, 0.43);
+  // eight: as many as an SM holds
+  spec_call(10000, each(64, 8), 4, 3.45);
+  spec_call(10000, each(1024, 8), 4, 4.0);
+  spec_call(5000, each(1024, 8), 2, 6.0);
+  spec_call(16000, each(256, 8), 2, 2.0);
+  // instances with different numbers of them; some with none
+  std::vector<int> mixed;
+  for (int i = 0; i < 300; ++i) mixed.push_back(i % 10);
+  spec_call(3000, mixed, 3, 7.5);
+  // more than can be in flight by far, few of them at a time: the kernel in memory; as many as that one would not win back: on chip
+  spec_call(24000, each(2300, 1), 1, 1.0);
+  spec_call(24000, each(2700, 1), 0, 0.0);
+  spec_call(10000, each(6500, 1), 1, 2.0);
+  spec_call(10000, each(8192, 1), 0, 0.0);
+  // not even one fits, or 16 bits do not number the jobs
+  spec_call(30000, each(10, 2), 0, 0.0);
+  spec_call(65535, each(10, 2), 0, 0.0);
+}
+
 // A refused call enqueues nothing; a call that fails half-way (every fallible call of the runtime, every launch and every
 // allocation in turn) returns a status and leaves nothing behind that the next call could meet.
 void errors() {
@@ -505,6 +588,7 @@ int main(int argc, char** argv) {
   if (what == "overlaps") overlaps();
   else if (what == "errors") errors();
   else if (what == "sizes") sizes();
+  else if (what == "groups") groups();
   else { printf("unknown program\n"); return 2; }
   printf("%s: %d faults\n", what.c_str(), races);
   return races ? 1 : 0;

@@ -97,7 +97,7 @@ def _spec_instance(n, seed, o_max, s_max):
 
 @pytest.mark.parametrize("n", [9_000, 12_000, 20_500])
 def test_evaluations_on_chip_by_size(par, n):
-    """Four evaluations per CTA of the kernel in shared memory, three, one (three budgets leave the fourth warp without one)."""
+    """Three evaluations per CTA of the kernel in shared memory, three with the shortest ring of rounds, one."""
     s, o = _spec_instance(n, 63, 60, 20)
     inst = workloads.Instances(torch.tensor([0, n]), s, o)
     par.check_batch(inst, binding.settings_grid(range(1), ["GSAS"], [1 << 14, 1 << 16, 1 << 18]), want_runs=False, label=f"spec n={n}")
@@ -119,8 +119,8 @@ def test_evaluations_left_by_the_on_chip_kernel(par):
 
 @pytest.mark.parametrize("n", [31, 33, 127, 129, 4_095, 4_097])
 def test_on_chip_maps_and_groups(par, n):
-    """Edges of the words, the 128-job rows and the 4,096-job probes of the map of free jobs; five budgets make a full CTA and a
-    CTA of one.  The small budgets' windows of 32 rounds are looked at as a whole, those of the large ones hold too many starts."""
+    """Edges of the words, the 128-job rows and the 4,096-job probes of the map of free jobs; five budgets make a CTA of
+    three and one of two.  The small budgets' windows of 32 rounds are looked at as a whole, those of the large ones hold too many starts."""
     s, o = _spec_instance(n, 71, 60, 20)
     inst = workloads.Instances(torch.tensor([0, n]), s, o)
     st = binding.settings_grid(range(1), ["GSAS"], [1 << 8, 1 << 9, 1 << 11, 1 << 14, 1 << 17])
@@ -135,3 +135,24 @@ def test_long_runs_leave_the_plan(par, n, lo, hi, M):
     c = torch.arange(n)
     inst = workloads.Instances(torch.tensor([0, n]), workloads.uniform_int(81, c, 0, 20), workloads.uniform_int(82, c, lo, hi))
     par.check_batch(inst, binding.settings_grid(range(1), ["GSAS"], [M]), want_runs=False, label=f"spec long {lo}..{hi} M={M}")
+
+
+@pytest.mark.parametrize("n, instances, budgets", [(500, 2_400, 1), (300, 600, 5), (2_000, 800, 2), (5_000, 640, 1), (9_500, 320, 1)])
+def test_groups_by_the_size_of_the_batch(par, n, instances, budgets):
+    """More evaluations than the GPU holds, with one, two and five budgets per instance, against the same ones a few at a time: rings of other
+    lengths, groups of other sizes.  Two instances against the oracle."""
+    s, o = _spec_instance(n * instances, 91, 60, 20)
+    inst = workloads.Instances(torch.arange(instances + 1) * n, s, o)
+    st = binding.settings_grid(range(instances), ["GSAS"], np.array([[1 << (9 + (i + 2 * b) % 9) for b in range(budgets)] for i in range(instances)]))
+    all_at_once = par.scheduler().evaluate(inst.to("cuda:0"), st, want_profile=True)
+    assert not bool(all_at_once.status.any())
+    step = 64
+    for i in range(0, instances, step):
+        j = min(instances, i + step)
+        some = par.scheduler().evaluate(inst.slice(i, j).to("cuda:0"), binding.settings_grid(range(j - i), ["GSAS"], st["M"].reshape(instances, budgets)[i:j]), want_profile=True)
+        for f in ("flow", "peak", "horizon", "job_steps", "n_runs", "n_unfinished", "feasible"):
+            assert torch.equal(getattr(some, f), getattr(all_at_once, f)[i * budgets:j * budgets]), f
+        for f, off in (("job_start", "job_out_off"), ("job_completion", "job_out_off"), ("profile", "profile_off")):
+            ends = getattr(all_at_once, off)
+            assert torch.equal(getattr(some, f), getattr(all_at_once, f)[int(ends[i * budgets]):int(ends[j * budgets])]), f
+    par.check_batch(inst.slice(0, 2), binding.settings_grid(range(2), ["GSAS"], st["M"].reshape(instances, budgets)[:2]), want_runs=False, label="spec groups")

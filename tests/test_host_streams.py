@@ -39,3 +39,9 @@ def test_requests_for_sizes_belong_to_their_reader(program):
     """Requests that overlap each get their own sizes; one reader refuses a second request; page-locked memory is neither overwritten nor
     given back while a copy uses it."""
     _run(program, "sizes")
+
+
+def test_groups_of_speculative_evaluations(program):
+    """One, two, five and eight budgets per instance, few evaluations and many: a CTA has room for what its group holds, groups are of near-equal
+    size, an SM has as many evaluations in flight as it can hold, and the kernel in memory takes over where it is the faster one."""
+    _run(program, "groups")
