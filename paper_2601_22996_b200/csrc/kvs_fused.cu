@@ -52,8 +52,17 @@ constexpr int RPT = 4;                       // consecutive ranks per thread in 
 constexpr int MAXP = KVS_MAX_PHASES;
 constexpr int RINGW = 2 * TILE + (2 * TILE) / 8;
 constexpr int GCOL = 2049;
-constexpr int PAIR_CYCLES = 60;              // see the use
-constexpr u64 SHARED_PAIRS = 1u << 20;       // more pairs of run ends and runs in a phase are shared between an evaluation's CTAs
+// What a peak without rounds is weighed by (see the uses): cycles that a step of a thread over the pairs of a run end and a run is taken to
+// cost, and the pairs of a phase above which all CTAs of an evaluation look at them.  The step itself - a load, a comparison, two
+// additions - costs less, but at its own cost phases went to the run ends that the bound or the visit settles sooner.  us a call of plain
+// slicing on config 2's lengths, cycles 40 / 60 / 80 / 100 / 150 (2^20 pairs):
+//   sweeps over 64 initial slices: 500 jobs alike, 2,000 (2^20 tokens) 125 / 103 / 101 / 101 / 106, 5,000 183 / 163 / 151 / 147 / 163, 20,000 (2^22) 361 / 337 / 316 / 319 / 319;
+//   2 instances of 100,000 jobs 643 / 643 / 583 / 486 / 486, 1,024 of 20,000 from host memory 3,370 / 3,222 / 3,233 / 3,215 / 3,217.
+// Pairs 2^18 / 2^19 / 2^20 / 2^21 / 2^22 / never (100 cycles):
+//   sweeps: 500 jobs alike, 2,000 (16 values, 2^22) 104 / 99 / 86 / 87 / 87 / 86, 5,000 (64, 2^20) 132 / 133 / 147 / 147 / 149 / 148, (4, 2^22) 93 / 90 / 90 / 112 / 112 / 112,
+//   20,000 (64, 2^18) 223 / 220 / 201 / 202 / 201 / 202, (64, 2^20) 237 / 240 / 237 / 296 / 334 / 331;  2 instances of 100,000 jobs 505 / 506 / 484 / 473 / 474 / 518.
+constexpr int PAIR_CYCLES = 100;
+constexpr u64 SHARED_PAIRS = 1u << 20;
 static_assert((TILE & (TILE - 1)) == 0 && ITEMS % 4 == 0 && ITEMS <= 32 && 32 % ITEMS == 0, "tile layout");
 constexpr u32 TIME_LIMIT = 0x7fffffffu - 4u * TILE;   // phase ends stay below this
 
@@ -1745,7 +1754,7 @@ __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 
           int tile_lo = 0, tile_hi = n_tiles;
           if (SHARED && parts > 1 && peak_only) {
             // The phases are taken in turn, but one of many pairs of run ends and runs is looked at by all CTAs, each of which takes a
-            // share of its run ends: 64 initial slices on 20,000 jobs, whose longest evaluations have few phases, 420 -> 250 us.
+            // share of its run ends: 64 initial slices on 20,000 jobs, whose longest evaluations have few phases, 331 -> 237 us.
             const u64 pairs = static_cast<u64>(N) * min(static_cast<u32>(N), sh.k[ph]), rounds = static_cast<u64>(n_tiles) * 6000;
             if (!batches && !sim && ph >= n_pure && pairs > SHARED_PAIRS && rounds >= static_cast<u64>(N) && pairs / T * PAIR_CYCLES / parts < rounds) { part_of = part; parts_of = parts; }
             else if (turn++ % parts != part) continue;
@@ -1826,9 +1835,7 @@ __global__ void __launch_bounds__(KVS_EVAL_THREADS, LIGHT ? KVS_EVAL_MIN_CTAS + 
               return block_max(W, sh.redA, 0u);
             };
             // Cycles of a CTA, roughly: PAIR_CYCLES per step of a thread over the pairs of a run end and a run that may be active
-            // then, against 6,000 per tile and 8 per run; the bound takes the prefix sums over the ranks.  (A pair costs less by
-            // itself; 40 and 100 instead of 60: 1,024 instances from host memory 3,414 and 3,224 us against 3,235, 128 instances of
-            // 3,000 jobs 472 and 457 against 458, 60 of 10,000 at one budget 177 and 173 against 173.)
+            // then, against 6,000 per tile and 8 per run; the bound takes the prefix sums over the ranks.
             const u64 pairs = static_cast<u64>(N) * kk, by_ends = pairs / T * PAIR_CYCLES / parts_of + 1500, by_rounds = static_cast<u64>(n_tiles) * 6000 + static_cast<u64>(N) * (sliced ? 1 : 8);
             if (pure) {
               // the window of all these phases at their largest parallelism bounds each of them

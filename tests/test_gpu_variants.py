@@ -177,7 +177,7 @@ def test_shared_evaluations_by_kernel(par, kind, want_profile):
     par.check_batch(inst, binding.make_settings(rows), window=window, want_runs=False, want_profile=want_profile, label=f"shared {kind}")
 
 
-@pytest.mark.parametrize("n, alpha", [(6_000, (2, 1)), (2_500, (3, 2)), (513, (2, 1))])
+@pytest.mark.parametrize("n, alpha", [(6_000, (2, 1)), (2_500, (3, 2)), (513, (2, 1)), (30_000, (2, 1))])
 def test_few_long_phases_are_shared_between_ctas(par, n, alpha):
     """Evaluations without a profile whose long slices pair many run ends with many runs: every CTA of an evaluation takes some of the ends."""
     inst = workloads.config2(n_inst=1, n=n)
