@@ -1,6 +1,9 @@
 """Variants inside the geometric classes on the GPU against the oracle: simultaneous batches as the
 subroutine of every phase, the parallelism of a phase sized by the longest prompt among its participants,
 and the sweep over tunable initial slices.  Bit-exact, every output."""
+import os
+import re
+
 import numpy as np
 import pytest
 import torch
@@ -177,10 +180,29 @@ def test_shared_evaluations_by_kernel(par, kind, want_profile):
     par.check_batch(inst, binding.make_settings(rows), window=window, want_runs=False, want_profile=want_profile, label=f"shared {kind}")
 
 
+def _shared_phases(S, n, parts):
+    """Slicing phases of a schedule that all CTAs of its evaluation look at: enough pairs of a run end and a run that may be active then,
+    and cheaper so than round by round (the rule and its constants in kvs_fused.cu; tiles of 4,096 rounds, 512 threads)."""
+    source = open(os.path.join(os.path.dirname(binding.__file__), "csrc", "kvs_fused.cu")).read()
+    cycles = int(re.search(r"constexpr int PAIR_CYCLES = (\d+);", source)[1])
+    least = 1 << int(re.search(r"constexpr u64 SHARED_PAIRS = 1u << (\d+);", source)[1])
+    N, tau, k = (v.astype(np.int64).tolist() for v in (S.n_part, S.tau, S.k))
+    first = next(q for q in range(len(N)) if q + 1 == len(N) or N[q + 1] != n)      # before it no job has left: prefix sums
+    shared = []
+    for q in range(first, len(N)):
+        pairs, rounds = N[q] * min(N[q], k[q]), -(-((N[q] - 1) * tau[q] // k[q] + tau[q]) // 4096) * 6000
+        if N[q] and pairs > least and rounds >= N[q] and pairs // 512 * cycles // parts < rounds:
+            shared.append(q)
+    return shared
+
+
 @pytest.mark.parametrize("n, alpha", [(6_000, (2, 1)), (2_500, (3, 2)), (513, (2, 1)), (30_000, (2, 1))])
 def test_few_long_phases_are_shared_between_ctas(par, n, alpha):
-    """Evaluations without a profile whose long slices pair many run ends with many runs: every CTA of an evaluation takes some of the ends."""
+    """Evaluations without a profile whose long slices pair many run ends with many runs: every CTA of an evaluation takes some of the ends.
+    Of 513 jobs no phase has enough pairs: there the phases are taken in turn.  (The batching rows are evaluated from their classes.)"""
     inst = workloads.config2(n_inst=1, n=n)
     rows = [dict(instance=0, family=fam, M=M, beta0=b, alpha=alpha) for fam in ("GBA", "GSA") for M in (1 << 20, 1 << 22) for b in (0, 40, 700, 3_000)]
+    shared = [bool(_shared_phases(oracle.build_schedule("GSA", inst.s, inst.o, r["M"], alpha=alpha, beta0=r["beta0"]), n, 16)) for r in rows[8:]]
+    assert any(shared) == (n > 513) and (n < 30_000 or shared[0])
     par.check_batch(inst, binding.make_settings(rows), want_runs=False, want_profile=False, label=f"long phases n={n}")
     par.check_batch(inst, binding.make_settings(rows[8:9]), want_runs=False, want_profile=False, label=f"long phases alone n={n}")
