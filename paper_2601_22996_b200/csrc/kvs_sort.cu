@@ -6,7 +6,7 @@
 // (ties keep the original index order) is what makes the order unique, so that the per-job
 // results agree bit for bit with a stable comparison sort.
 //
-// Each pass ranks one tile of KVS_SORT_TILE jobs at a time.  A warp takes 32 * ITEMS consecutive ones, row by row: lanes with equal
+// Each pass ranks one tile of TILE_N jobs at a time.  A warp takes 32 * ITEMS consecutive ones, row by row: lanes with equal
 // digits find each other with a warp match and stand behind what the warp has counted so far of their digit in its row of counters
 // in shared memory; one column scan per tile, eight counters a thread, turns the counters into offsets behind the running
 // bucket position.  Two block barriers per tile.  Only 4 bytes per job move per pass: the index, together with the key in the
