@@ -181,7 +181,8 @@ typedef struct {
  * A request belongs to a reader, which no context shares: page-locked memory of its own for one request at a time.  A request that
  * has been begun is ended, whatever kvs_sizes_end returns, before the next one is begun on the same reader; a begin in between
  * is refused (KVS_E_STATE) and leaves the open request as it is, an end without a begin too.  Threads that read sizes at the same time use a reader each.
- * kvs_reader_close waits for what is in flight, of a request that was never ended too.  kvs_reader_error: as kvs_last_error. */
+ * kvs_reader_close waits for what is in flight, of a request that was never ended too (whose stream may be gone by then).
+ * kvs_reader_error: as kvs_last_error. */
 typedef struct kvs_reader kvs_reader; /* opaque; owned by the library (host object only) */
 int kvs_reader_open(int32_t device, kvs_reader** out);
 int kvs_reader_close(kvs_reader* reader);

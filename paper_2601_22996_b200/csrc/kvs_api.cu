@@ -49,10 +49,11 @@ struct kvs_ctx {
 // thread may use, or replace by a larger one, the context that the call will run on meanwhile.
 struct kvs_reader {
   int device = 0;
-  cudaStream_t stream = nullptr;                           // of the last request
+  cudaStream_t stream = nullptr;                           // of the open request; the caller may destroy it when it never ends that
   struct Pinned { int64_t* p = nullptr; size_t bytes = 0; } in, rows;   // what is read: job offsets, then capacities; what goes up
   int64_t n_off = -1, n_cap = -1;                          // of the open request (-1: not asked for)
   bool open = false;
+  cudaEvent_t arrived = nullptr;                           // the sizes of the open request
   cudaEvent_t sent = nullptr;                              // the rows of the last request have gone up
   bool sending = false;
   std::string err;
@@ -795,8 +796,9 @@ int kvs_reader_open(int32_t device, kvs_reader** out) {
   kvs_reader* r = new (std::nothrow) kvs_reader();
   if (!r) return KVS_E_STATE;
   r->device = device;
-  if (cudaSetDevice(device) != cudaSuccess || cudaEventCreateWithFlags(&r->sent, cudaEventDisableTiming) != cudaSuccess) {
-    delete r;
+  if (cudaSetDevice(device) != cudaSuccess || cudaEventCreateWithFlags(&r->sent, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&r->arrived, cudaEventDisableTiming) != cudaSuccess) {
+    kvs_reader_close(r);
     return KVS_E_CUDA;
   }
   *out = r;
@@ -805,9 +807,9 @@ int kvs_reader_open(int32_t device, kvs_reader** out) {
 
 int kvs_reader_close(kvs_reader* r) {
   if (r) {
-    if (r->open) cudaStreamSynchronize(r->stream);         // begun and never ended
+    if (r->open) cudaEventSynchronize(r->arrived);         // begun and never ended
     if (r->sending) cudaEventSynchronize(r->sent);
-    cudaEventDestroy(r->sent);
+    for (cudaEvent_t e : {r->arrived, r->sent}) if (e) cudaEventDestroy(e);
     for (kvs_reader::Pinned* m : {&r->in, &r->rows}) if (m->p) cudaFreeHost(m->p);
   }
   delete r;
@@ -838,13 +840,14 @@ int kvs_sizes_begin(kvs_reader* r, void* stream, const int64_t* job_off, int64_t
   cudaError_t ce = cudaSetDevice(r->device);
   if (ce == cudaSuccess) ce = make_room(r->in, off_bytes + cap_bytes);
   if (ce == cudaSuccess && off_bytes) ce = cudaMemcpyAsync(r->in.p, job_off, off_bytes, cudaMemcpyDeviceToHost, r->stream);
-  r->open = ce == cudaSuccess;
+  const bool under_way = ce == cudaSuccess;
   if (ce == cudaSuccess && cap_bytes) ce = cudaMemcpyAsync(reinterpret_cast<unsigned char*>(r->in.p) + off_bytes, capacity, cap_bytes, cudaMemcpyDeviceToHost, r->stream);
+  if (ce == cudaSuccess) ce = cudaEventRecord(r->arrived, r->stream);
   if (ce != cudaSuccess) {
-    if (r->open) cudaStreamSynchronize(r->stream);
-    r->open = false;
+    if (under_way) cudaStreamSynchronize(r->stream);
     return fail_cuda(r, ce, "read of the sizes");
   }
+  r->open = true;
   return KVS_OK;
 }
 
@@ -852,7 +855,7 @@ static int sizes_end(kvs_reader* r, const kvs_setting* settings, int64_t P, int6
   if (!r->open) return fail(r, KVS_E_STATE, "sizes: not begun");
   r->open = false;
   cudaError_t ce = cudaSetDevice(r->device);
-  const cudaError_t waited = cudaStreamSynchronize(r->stream);
+  const cudaError_t waited = cudaEventSynchronize(r->arrived);
   if (ce == cudaSuccess) ce = waited;
   if (ce != cudaSuccess) return fail_cuda(r, ce, "read of the sizes");
   if (P < 0 || (job_out_off && (r->n_off < 1 || (P > 0 && !settings))) || (profile_off && r->n_cap != P)) return fail(r, KVS_E_ARG, "sizes: not those that were asked for");

@@ -23,7 +23,7 @@ struct Clock {
   long at[MAX_STREAMS] = {};
   void join(const Clock& c) { for (int i = 0; i < MAX_STREAMS; ++i) at[i] = std::max(at[i], c.at[i]); }
 };
-struct Stream { int id; Clock clock; };
+struct Stream { int id; Clock clock; bool gone = false; };
 struct Event { Clock clock; };
 
 enum Kind { READ, WRITE, ATOMIC };
@@ -40,7 +40,9 @@ bool library = false;
 
 Stream* stream_of(cudaStream_t s) {
   if (streams.empty()) streams.push_back(new Stream{0, {}});       // the default stream
-  return s ? reinterpret_cast<Stream*>(s) : streams[0];
+  Stream* const st = s ? reinterpret_cast<Stream*>(s) : streams[0];
+  if (st->gone && races++ < 5) printf("stream %d is used after it was destroyed\n", st->id);
+  return st;
 }
 bool fails() { return calls++ == fail_at; }
 struct Outside {                       // the fake's own allocations neither count nor fail
@@ -118,7 +120,7 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
   return cudaSuccess;
 }
 cudaError_t cudaStreamCreateWithPriority(cudaStream_t* s, unsigned f, int) { return cudaStreamCreateWithFlags(s, f); }
-cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t s) { stream_of(s)->gone = true; return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) { host.join(stream_of(s)->clock); return fails() ? cudaErrorUnknown : cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { for (Stream* s : streams) host.join(s->clock); return cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
@@ -448,7 +450,9 @@ void sizes() {
                             kvs_sizes_end(x, nullptr, static_cast<i64>(P), nullptr, keep.back().data(), &sa) == KVS_OK && sa.profile_rounds == 3 * static_cast<i64>(P));
   }
   find_races();
-  kvs_sizes_begin(y, nullptr, b.data(), 2, nullptr, 0);
+  // a request that is never ended, on a stream that its caller destroys: the reader waits for the copy, not on the stream
+  kvs_sizes_begin(y, other, b.data(), 2, nullptr, 0);
+  cudaStreamDestroy(other);
   kvs_reader_close(y);
   kvs_reader_close(x);
   if (const int n = outstanding(host)) { printf("%d operations in flight\n", n); ++races; }
